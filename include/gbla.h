@@ -359,15 +359,16 @@ int gbla_bicgstab_solve(int n, const double *A, int lda, const double *b, double
  * the two substitutions of paper section 2 for every system of a batch), in
  * ONE persistent kernel launch: a grid of SMs x ctas_per_sm CTAs pulls system
  * indices from a counter (in d_order, or index order if d_order is NULL); one
- * CTA factors and solves one whole system, in shared memory when it fits, in
- * place in global memory otherwise. No host synchronisation and no
- * allocation: the call can be captured in a CUDA graph.
+ * CTA factors and solves one whole system, in panels staged in shared memory
+ * up to n = 512, column by column in global memory above. No host
+ * synchronisation and no allocation: the call can be captured in a CUDA graph.
  * Device arrays of length batch: d_n (orders), d_A (column-major matrices,
  * overwritten by their L\U), d_lda, d_ipiv (n_i ints each, 1-based),
  * d_nrhs (0..4 right-hand sides each; NULL = factor only), d_B (n_i x nrhs_i,
  * overwritten by X), d_ldb, d_info (first zero pivot per system or 0; may be
  * NULL). max_n: an upper bound on the orders (sizes shared memory).
- * threads (multiple of 32, 0 = 256) and ctas_per_sm (0 = 1) are tuning knobs.
+ * ctas_per_sm (0 = as many as fit) is a tuning knob; threads (a multiple of 32,
+ * or 0) is checked and otherwise ignored: every CTA has 256.
  * ------------------------------------------------------------------------ */
 size_t gbla_lu_batched_workspace(int batch);
 int gbla_lu_solve_batched(int batch, const int *d_n, double *const *d_A, const int *d_lda,
@@ -414,7 +415,7 @@ int gbla_lu_solve_factored_batched_f32(int batch, const int *d_n, float *const *
  * Batched Cholesky + solve (step a9 for symmetric positive definite systems:
  * A = L L^t and the two substitutions of paper section 2, for every system of
  * a batch) in ONE persistent kernel launch, with the launch structure of
- * gbla_lu_solve_batched (same counter-driven grid, same shared-memory /
+ * gbla_lu_solve_batched (same counter-driven grid, same panel /
  * in-place split, no host synchronisation, no allocation, graph-capturable).
  * Only the lower triangle of each A is read and overwritten by L; the strict
  * upper triangle is untouched. d_info[i] = j + 1 when the j-th leading minor

@@ -18,7 +18,7 @@ import torch
 from . import _lib
 from .api import _check, _stream, _ws
 
-CANDIDATES = [(t, c) for t in (128, 256, 512) for c in (1, 2, 4)]
+CANDIDATES = [(256, c) for c in (0, 1, 2)]  # CTAs per SM; 0: as many as fit
 
 
 def _cache_path():
@@ -97,7 +97,7 @@ class BatchedLU:
         L = _lib.load()
         wsf = L.gbla_lu_batched_workspace if method == "lu" else L.gbla_chol_batched_workspace
         self.ws = _ws(wsf(self.batch), dev)
-        self.threads, self.ctas_per_sm = 256, 1
+        self.threads, self.ctas_per_sm = 256, 0
         self.graph = None
 
     # -- execution ---------------------------------------------------------------

@@ -82,6 +82,38 @@ GBLA_DEVINL void warp_argmax(double& bv, int& bi) {
   }
 }
 
+// *l = sqrt(d), *rl = 1 / sqrt(d) for d > 0.
+GBLA_DEVINL void sqrt_rcp(float d, float* l, float* rl) {
+  *l = sqrtf(d);
+  *rl = 1.0f / *l;
+}
+// FP64: sqrt followed by a division is a chain of some twenty dependent FP64
+// operations per column, at the latency this GPU's FP64 pipe has. Instead, d is
+// scaled by a power of four to x in [1/2, 2), 1 / sqrt(x) comes from the FP32
+// approximation y and one third-order step of the series
+//   x^-1/2 = y (1 - e)^-1/2 = y (1 + e/2 + 3/8 e^2 + O(e^3)),  e = 1 - x y^2,
+// |e| < 2^-20, so the neglected term is below 2^-61; four dependent FP64
+// operations, and the result is within one rounding of 1 / sqrt(d). The root is
+// x times it, corrected once by its own residual (off the chain).
+GBLA_DEVINL void sqrt_rcp(double d, double* l, double* rl) {
+  const int hi = __double2hiint(d);
+  const int ex = hi >> 20;  // d > 0: no sign
+  if (ex == 0 || ex >= 0x7ff) {  // subnormal or infinite
+    *l = sqrt(d);
+    *rl = 1.0 / *l;
+    return;
+  }
+  const int q = (ex - 1022) >> 1;  // d = x 4^q, exponent of x: 1022 or 1023
+  const double x = __hiloint2double(hi - (q << 21), __double2loint(d));
+  const double y = (double)rsqrtf((float)x);
+  const double e = fma(-(x * y), y, 1.0);
+  const double r = fma(y * e, fma(0.375, e, 0.5), y);
+  const double h = x * r;
+  const double s = fma(fma(-h, h, x), 0.5 * r, h);
+  *rl = __hiloint2double(__double2hiint(r) - (q << 20), __double2loint(r));
+  *l = __hiloint2double(__double2hiint(s) + (q << 20), __double2loint(s));
+}
+
 // Final sources of the rows touched by kb <= 256 sequential interchanges
 // (row t <-> row p_t for t = 0 .. kb - 1 in order, p_t >= t, rows relative to
 // the block's first row), worked out by the threads t < kb in parallel. With
