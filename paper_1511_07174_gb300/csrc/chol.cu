@@ -3,7 +3,7 @@
 // autotunable), each processed in 64-column steps:
 //   potf2   -- the 64 x 64 diagonal block factored by one CTA in shared memory
 //              (column by column: d = a_jj, stop with info = j + 1 if d <= 0,
-//              l_jj = sqrt(d), l_ij = a_ij / l_jj, a_ik -= l_ij l_kj);
+//              l_jj = sqrt(d), l_ij = a_ij * (1 / l_jj), a_ik -= l_ij l_kj);
 //   trsm    -- the rows below it: L21 = A21 L11^{-t} in two 32-column halves
 //              (one thread per row, its 32 values in registers, the triangle
 //              in shared memory; the second half first receives the update
@@ -20,40 +20,65 @@ namespace gbla {
 
 constexpr int kCholNb = 64;
 
+// The kb x kb diagonal block (kb <= 64) in shared memory. A GPU-wide FP64 rate of
+// 2 multiply-adds per clock and SM is half a lane per clock for each of its
+// four schedulers: one FP64 instruction of one warp takes 64 clocks however few
+// of its lanes are active. So per column the reciprocal root is formed by one
+// warp only, which first updates the next diagonal element and then works on
+// it while the other seven update the rest of the triangle, each warp with 32
+// live elements of it (columns c and m - 1 - c of the triangle are m + 1
+// elements together).
+// d <= 0 (or NaN) stops; the columns to the right have received the updates of
+// the finished ones. An earlier block that failed leaves the rest of the
+// factor undefined; the first failure stays in info.
 template <typename T>
 __global__ void __launch_bounds__(256)
     potf2_kernel(int kb, T* __restrict__ A, int lda, int row0, int* __restrict__ info) {
   __shared__ T D[kCholNb][kCholNb + 1];
+  __shared__ T s_rl;
   __shared__ int s_bad;
   const int tid = threadIdx.x;
   for (int idx = tid; idx < kCholNb * kCholNb; idx += blockDim.x) {
     const int r = idx & 63, c = idx >> 6;
     D[r][c] = (r < kb && c < kb && r >= c) ? A[r + (size_t)c * lda] : (T)0;
   }
-  if (tid == 0) s_bad = 0;
+  if (tid == 0) s_bad = kCholNb;
   __syncthreads();
-  // an earlier block that failed leaves the rest of the factor undefined; the
-  // first failure stays in info
-  for (int j = 0; j < kb; ++j) {
-    if (tid == 0) {
-      const T d = D[j][j];
-      if (!(d > (T)0)) {
-        s_bad = 1;
+  // d = the finished diagonal element of column j (one warp)
+  auto root = [&](int j, T d) {
+    if (!(d > (T)0)) {
+      if (tid == 0) {
+        s_bad = j;
+        D[j][j] = d;
         atomicCAS(info, 0, row0 + j + 1);
-      } else {
-        D[j][j] = sqrt(d);
+      }
+    } else {
+      T l, rl;
+      sqrt_rcp(d, &l, &rl);
+      if (tid == 0) {
+        D[j][j] = l;
+        s_rl = rl;
       }
     }
+  };
+  if (tid < 32) root(0, D[0][0]);
+  __syncthreads();
+  for (int j = 0; j < kb && s_bad > j; ++j) {
+    const T rl = s_rl;
+    if (tid > j && tid < kb) D[tid][j] *= rl;
     __syncthreads();
-    if (s_bad) break;
-    const T rl = (T)1 / D[j][j];
-    for (int i = j + 1 + tid; i < kb; i += blockDim.x) D[i][j] *= rl;
-    __syncthreads();
-    // trailing part of the block: a_ik -= l_ij l_kj for i >= k > j
     const int m = kb - j - 1;
-    for (int idx = tid; idx < m * m; idx += blockDim.x) {
-      const int i = j + 1 + idx % m, k = j + 1 + idx / m;
-      if (i >= k) D[i][k] = fma(-D[i][j], D[k][j], D[i][k]);
+    if (tid < 32) {
+      if (m > 0) root(j + 1, fma(-D[j + 1][j], D[j + 1][j], D[j + 1][j + 1]));
+    } else {
+      const int half = (m + 1) >> 1;
+      for (int e = tid - 32; e < half * (m + 1); e += 224) {
+        const int c = e / (m + 1), r = e - c * (m + 1);
+        const bool first = r < m - c;
+        const int k = first ? c : m - 1 - c, i = first ? c + r : k + r - (m - c);
+        if (i + k > 0 && (first || 2 * c != m - 1))  // (0, 0) belongs to the first warp
+          D[j + 1 + i][j + 1 + k] = fma(-D[j + 1 + i][j], D[j + 1 + k][j], D[j + 1 + i][j + 1 + k]);
+      }
     }
     __syncthreads();
   }
