@@ -160,6 +160,15 @@ int gbla_fma_peak(int precision, int iters, double *tflops, gbla_stream_t stream
  *   nb     block size in [32, 256], multiple of 32; 0 = default (256)
  * ------------------------------------------------------------------------ */
 size_t gbla_lu_factor_workspace(int n, int nb);
+/* The scratch with which gbla_lu_factor does its trailing updates on the
+ * tensor cores: gbla_lu_factor_workspace(n, nb) plus, when nb is a multiple of
+ * 128, 8 bytes per element of two n x nb operands in 8-bit digits and their
+ * scales. The operands are split exactly to 2^-55 of a row's largest magnitude
+ * and multiplied exactly, and tiles for which that would be less accurate than
+ * FP64 multiply-adds are done by those. Any work_bytes from
+ * gbla_lu_factor_workspace up is accepted; below this size every update runs
+ * on the FP64 pipe. */
+size_t gbla_lu_factor_workspace_tensor(int n, int nb);
 int gbla_lu_factor(int n, double *A, int lda, int *ipiv, int *d_info, int nb,
                    void *d_work, size_t work_bytes, gbla_stream_t stream);
 
@@ -212,6 +221,15 @@ int gbla_lu_solve(int trans, int n, int nrhs, const double *LU, int lda, const i
  * positive definite (the rest of the factor is then undefined).
  * ------------------------------------------------------------------------ */
 int gbla_chol_factor(int n, double *A, int lda, int *d_info, int nb, gbla_stream_t stream);
+
+/* The same factorisation with scratch: the trailing updates run on the tensor
+ * cores, as in gbla_lu_factor with gbla_lu_factor_workspace_tensor bytes.
+ * nb = 0: 128. Workspace: gbla_chol_factor_workspace(n, nb) bytes, 256-byte
+ * aligned. Returns -i for an invalid i-th argument, GBLA_ERR_WORKSPACE,
+ * GBLA_ERR_CUDA; d_info may also receive GBLA_INFO_TIMEOUT. */
+size_t gbla_chol_factor_workspace(int n, int nb);
+int gbla_chol_factor_ws(int n, double *A, int lda, int *d_info, int nb, void *d_work,
+                        size_t work_bytes, gbla_stream_t stream);
 
 /* Solve A X = B from gbla_chol_factor: L y = b (forward), L^t x = y (back).
  * B (n x nrhs, ldb) is overwritten by X. */

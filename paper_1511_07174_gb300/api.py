@@ -82,7 +82,7 @@ def lu_factor(A, nb=0):
     LU = colmajor(A, torch.float64, copy=True)
     ipiv = torch.empty(max(n, 1), dtype=torch.int32, device=A.device)
     info = torch.zeros(1, dtype=torch.int32, device=A.device)
-    ws = _ws(L.gbla_lu_factor_workspace(n, nb), A.device)
+    ws = _ws(L.gbla_lu_factor_workspace_tensor(n, nb), A.device)
     _check("gbla_lu_factor", L.gbla_lu_factor(n, _p(LU), _ld(LU), _p(ipiv), _p(info), nb, _p(ws),
                                               ws.numel(), _stream()))
     return LU, ipiv[:n], info
@@ -108,13 +108,15 @@ def lu_solve(LU, ipiv, B, trans=False, info=None):
 def chol_factor(A, nb=0):
     """A = L L^t (FP64, lower). Returns (matrix with L in its lower triangle, info device int32[1]).
     The strict upper triangle is copied from A and left untouched. nb: outer block width
-    (64, 128, 192 or 256; 0 = 64; see tune_chol_nb)."""
+    (64, 128, 192 or 256; 0: the library's choice; see tune_chol_nb)."""
     _require_cuda(A)
     L = _lib.load()
     n = A.shape[0]
     F = colmajor(A, torch.float64, copy=True)
     info = torch.zeros(1, dtype=torch.int32, device=A.device)
-    _check("gbla_chol_factor", L.gbla_chol_factor(n, _p(F), _ld(F), _p(info), int(nb), _stream()))
+    ws = _ws(L.gbla_chol_factor_workspace(n, int(nb)), A.device)
+    _check("gbla_chol_factor_ws", L.gbla_chol_factor_ws(n, _p(F), _ld(F), _p(info), int(nb), _p(ws), ws.numel(),
+                                                        _stream()))
     return F, info
 
 

@@ -21,6 +21,7 @@ static std::atomic<int> g_subst_ctas{0};
 int substitution_ctas() { return g_subst_ctas.load(std::memory_order_relaxed); }
 static std::atomic<int> g_lookahead{0};
 bool lookahead_enabled() { return g_lookahead.load(std::memory_order_relaxed) != 0; }
+constexpr int kCholWsNb = 128;    // default outer block of the FP64 Cholesky with scratch
 constexpr int kClusterSms = 16;  // SMs of the panel's thread-block cluster
 
 const DeviceProps& device_props() {
@@ -214,6 +215,24 @@ static void lookahead_release(const LookAhead& r) {
 // update runs on the caller's stream on all SMs but 16 (the panel's cluster);
 // the caller's stream then waits for the panels. Every element receives the
 // same operations in the same order as without look-ahead.
+// Scratch of the FP64 trailing update on the tensor cores (both operands when
+// `cols`, else the rows of A only).
+static void digits_layout(Carver& c, int n, int nb, bool cols, F64Digits* d) {
+  const size_t rows = (size_t)std::max(n, 1);
+  F64Digits t;
+  t.a = c.take<char>(rows * f64tc_ld(nb) * 2);
+  if (cols) t.b = c.take<char>(rows * f64tc_ld(nb) * 2);
+  t.ea = c.take<int>(rows);
+  if (cols) t.eb = c.take<int>(rows);
+  t.list = c.take<int>(f64tc_list_ints(n, n));
+  if (d && c.ok) *d = t;
+}
+
+// The digits of L21 and U12 in 128 x 128 tiles: with nb a multiple of 128 the
+// look-ahead's split of an update falls on a tile boundary, so the same tiles
+// go to the FP64 pipe with and without it.
+static bool lu_uses_digits(int nb) { return nb % 128 == 0; }
+
 static size_t lu_work_layout(Carver& c, int n, int nb, int prec, LuWork* w) {
   double* slots = c.take<double>(panel_slots_doubles());
   const size_t li = left_perm_ints(n, nb);
@@ -251,6 +270,7 @@ cudaError_t blocked_lu(int n, Ts* A, int lda, int* ipiv, int* info, int nb, int 
   // the columns left of each block get its interchanges at the end when possible
   const bool defer_left = w.left != nullptr && left_deferred_fits<Ts>(n, nb);
   const bool tensor = prec_is_tensor(prec);
+  const bool digits = sizeof(Ts) == 8 && w.dig.a != nullptr && lu_uses_digits(nb);
   cudaError_t e;
   // the panels of outer block [k0, k0 + kb) and the inner updates, on stream st
   auto panels = [&](int k0, int kb, cudaStream_t st) -> cudaError_t {
@@ -299,6 +319,19 @@ cudaError_t blocked_lu(int n, Ts* A, int lda, int* ipiv, int* info, int nb, int 
         return cudaErrorInvalidValue;
       }
     }
+    if constexpr (sizeof(Ts) == 8) {
+      if (digits) {
+        const char* Bd = static_cast<const char*>(w.dig.b) + (size_t)c0 * f64tc_ld(kb) * 2;
+        double* C = A + (k0 + kb) + (size_t)(k0 + kb + c0) * lda;
+        PROF(KK_GEMM_TC, st, launch_gemm_f64tc(nt, nc, kb, w.dig.a, Bd, w.dig.ea, w.dig.eb + c0, C, lda, w.dig.list,
+                                               info, false, st, grid_cap));
+        if (e != cudaSuccess) return e;
+        PROF(KK_GEMM_SIMT, st, launch_gemm_f64_list(nt, nc, kb, A + (k0 + kb) + (size_t)k0 * lda, lda,
+                                                    A + k0 + (size_t)(k0 + kb + c0) * lda, lda, false, C, lda, false,
+                                                    w.dig.list, st));
+        return e;
+      }
+    }
     PROF(KK_GEMM_SIMT, st, launch_gemm_simt<Ts>(nt, nc, kb, (Ts)-1, A + (k0 + kb) + (size_t)k0 * lda, lda,
                                                 A + k0 + (size_t)(k0 + kb + c0) * lda, lda, false, (Ts)1,
                                                 A + (k0 + kb) + (size_t)(k0 + kb + c0) * lda, lda, false, st));
@@ -335,6 +368,14 @@ cudaError_t blocked_lu(int n, Ts* A, int lda, int* ipiv, int* info, int nb, int 
       if constexpr (sizeof(Ts) == 4) {
         PROF(KK_CONVERT, s, launch_convert_rows(reinterpret_cast<const float*>(A + (k0 + kb) + (size_t)k0 * lda), lda,
                                 nt, kb, prec, w.Ak, w.ldk, w.eA, false, s));
+        if (e != cudaSuccess) { record_error(e, "blocked_lu step", __LINE__); status = e; break; }
+      }
+    }
+    if constexpr (sizeof(Ts) == 8) {
+      if (digits) {
+        PROF(KK_CONVERT, s, launch_f64_digits_rows(A + (k0 + kb) + (size_t)k0 * lda, lda, nt, kb, w.dig.a, w.dig.ea, s));
+        if (e == cudaSuccess)
+          PROF(KK_CONVERT, s, launch_f64_digits_cols(A + k0 + (size_t)(k0 + kb) * lda, lda, nt, kb, w.dig.b, w.dig.eb, s));
         if (e != cudaSuccess) { record_error(e, "blocked_lu step", __LINE__); status = e; break; }
       }
     }
@@ -481,6 +522,15 @@ size_t gbla_lu_factor_workspace(int n, int nb) {
   return lu_work_layout(c, n, nb, 0, nullptr);
 }
 
+size_t gbla_lu_factor_workspace_tensor(int n, int nb) {
+  nb = check_nb(nb);
+  if (n < 0 || nb < 0) return 0;
+  Carver c(nullptr, 0);
+  lu_work_layout(c, n, nb, 0, nullptr);
+  if (lu_uses_digits(nb) && n > nb) digits_layout(c, n, nb, true, nullptr);
+  return c.off;
+}
+
 int gbla_lu_factor(int n, double* A, int lda, int* ipiv, int* d_info, int nb, void* d_work,
                    size_t work_bytes, gbla_stream_t stream) {
   clear_error();
@@ -497,6 +547,8 @@ int gbla_lu_factor(int n, double* A, int lda, int* ipiv, int* d_info, int nb, vo
   LuWork w;
   lu_work_layout(c, n, nb, 0, &w);
   if (!c.ok) return GBLA_ERR_WORKSPACE;
+  // room for the digits: the trailing update runs on the tensor cores
+  if (lu_uses_digits(nb) && n > nb) digits_layout(c, n, nb, true, &w.dig);
   const DeviceProps& dp = device_props();
   if (dp.device < 0) return GBLA_ERR_CUDA;
   if (!dp.coop) return GBLA_ERR_DEVICE;
@@ -603,7 +655,37 @@ int gbla_chol_factor(int n, double* A, int lda, int* d_info, int nb, gbla_stream
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   GBLA_TRY(cudaMemsetAsync(d_info, 0, sizeof(int), s));
   if (n == 0) return GBLA_OK;
-  return cuda_status(launch_chol(n, A, lda, nb, d_info, s));
+  return cuda_status(launch_chol(n, A, lda, nb, d_info, F64Digits{}, s));
+}
+
+static int chol_ws_nb(int nb) { return nb == 0 ? kCholWsNb : ((nb % 64 == 0 && nb >= 64 && nb <= 256) ? nb : -1); }
+
+size_t gbla_chol_factor_workspace(int n, int nb) {
+  nb = chol_ws_nb(nb);
+  if (n < 0 || nb < 0) return 0;
+  Carver c(nullptr, 0);
+  digits_layout(c, n, nb, false, nullptr);
+  return c.off;
+}
+
+int gbla_chol_factor_ws(int n, double* A, int lda, int* d_info, int nb, void* d_work, size_t work_bytes,
+                        gbla_stream_t stream) {
+  clear_error();
+  if (n < 0) return -1;
+  if (n > 0 && !A) return -2;
+  if (lda < std::max(1, n)) return -3;
+  if (!d_info) return -4;
+  nb = chol_ws_nb(nb);
+  if (nb < 0) return -5;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (!d_work || !aligned256(d_work)) return GBLA_ERR_WORKSPACE;
+  Carver c(d_work, work_bytes);
+  F64Digits dig;
+  digits_layout(c, n, nb, false, &dig);
+  if (!c.ok) return GBLA_ERR_WORKSPACE;
+  GBLA_TRY(cudaMemsetAsync(d_info, 0, sizeof(int), s));
+  if (n == 0) return GBLA_OK;
+  return cuda_status(launch_chol(n, A, lda, nb, d_info, dig, s));
 }
 
 size_t gbla_chol_solve_workspace(int n, int nrhs) {

@@ -323,14 +323,13 @@ template cudaError_t launch_inner_update<float>(int, int, float*, int, unsigned*
 // tx + i*(BM/TM) and columns ty + j*(BN/TN) of the tile, so that the lanes of
 // a warp touch consecutive rows of column-major C.
 template <typename T, int BM, int BN, int BK, int TM, int TN, bool TRANSB, bool LOWER>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-    gemm_simt_kernel(int M, int N, int K, T alpha, const T* __restrict__ A, int lda,
-                     const T* __restrict__ B, int ldb, T beta, T* __restrict__ C, int ldc) {
+GBLA_DEVINL void gemm_simt_tile(int m0, int n0, int M, int N, int K, T alpha, const T* __restrict__ A,
+                                int lda, const T* __restrict__ B, int ldb, T beta,
+                                T* __restrict__ C, int ldc) {
   constexpr int NT = (BM / TM) * (BN / TN);
   constexpr int RX = BM / TM, RY = BN / TN;
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
-  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
   if (LOWER && m0 + BM - 1 < n0) return;  // tile strictly above the diagonal
   const int tid = threadIdx.x;
   const int tx = tid % RX, ty = tid / RX;
@@ -407,6 +406,48 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
       }
     }
   }
+}
+
+template <typename T, int BM, int BN, int BK, int TM, int TN, bool TRANSB, bool LOWER>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+    gemm_simt_kernel(int M, int N, int K, T alpha, const T* __restrict__ A, int lda,
+                     const T* __restrict__ B, int ldb, T beta, T* __restrict__ C, int ldc) {
+  gemm_simt_tile<T, BM, BN, BK, TM, TN, TRANSB, LOWER>(blockIdx.x * BM, blockIdx.y * BN, M, N, K, alpha, A,
+                                                       lda, B, ldb, beta, C, ldc);
+}
+
+// C -= A op(B) on the 128 x 128 tiles named by list[1 .. list[0]] (numbered as
+// the tensor-core update numbers them), four 64 x 64 tiles each.
+template <bool TRANSB, bool LOWER>
+__global__ void __launch_bounds__(256)
+    gemm_f64_list_kernel(int M, int N, int K, const double* __restrict__ A, int lda,
+                         const double* __restrict__ B, int ldb, double* __restrict__ C, int ldc,
+                         int tilesM, const int* __restrict__ list) {
+  const int count = 4 * list[0];
+  for (int i = blockIdx.x; i < count; i += gridDim.x) {
+    int ti, tj;
+    tile_coords(list[1 + (i >> 2)], tilesM, LOWER ? 1 : 0, ti, tj);
+    const int m0 = ti * 128 + (i & 1) * 64, n0 = tj * 128 + ((i >> 1) & 1) * 64;
+    if (m0 < M && n0 < N)
+      gemm_simt_tile<double, 64, 64, 16, 4, 4, TRANSB, LOWER>(m0, n0, M, N, K, -1.0, A, lda, B, ldb, 1.0, C,
+                                                              ldc);
+  }
+}
+
+cudaError_t launch_gemm_f64_list(int M, int N, int K, const double* A, int lda, const double* B, int ldb,
+                                 bool transB, double* C, int ldc, bool lower, const int* list,
+                                 cudaStream_t s) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  if (lower != transB) return cudaErrorInvalidValue;  // the two forms the factorisations use
+  const DeviceProps& dp = device_props();
+  const int tilesM = (M + 127) / 128;
+  const int grid = 4 * (dp.num_sms > 0 ? dp.num_sms : 1);
+  if (lower)
+    gemm_f64_list_kernel<true, true><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, tilesM, list);
+  else
+    gemm_f64_list_kernel<false, false><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, tilesM, list);
+  count_launch();
+  return cudaGetLastError();
 }
 
 template <typename T>

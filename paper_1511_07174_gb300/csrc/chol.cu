@@ -173,8 +173,10 @@ static cudaError_t chol_outer_block(int n, T* A, int lda, int o0, int ob, int* i
 
 // Two-level blocking: outer blocks of nb columns (a multiple of 64, up to
 // 256); inside one, 64-column steps; after the outer block, one rank-nb
-// update of the trailing lower triangle.
-cudaError_t launch_chol(int n, double* A, int lda, int nb, int* info, cudaStream_t s) {
+// update of the trailing lower triangle, on the tensor cores when the caller
+// gave scratch for the digits (gemm_f64.cu), by FP64 multiply-adds otherwise.
+cudaError_t launch_chol(int n, double* A, int lda, int nb, int* info, const F64Digits& dig,
+                        cudaStream_t s) {
   if (nb <= 0) nb = kCholNb;
   if (nb % kCholNb != 0 || nb > 256) return cudaErrorInvalidValue;
   for (int o0 = 0; o0 < n; o0 += nb) {
@@ -185,6 +187,23 @@ cudaError_t launch_chol(int n, double* A, int lda, int nb, int* info, cudaStream
     const int mt = n - o0 - ob;
     if (mt > 0) {
       double* L21 = A + (o0 + ob) + (size_t)o0 * lda;
+      if (dig.a) {
+        prof_begin(KK_CONVERT, s);
+        e = launch_f64_digits_rows(L21, lda, mt, ob, dig.a, dig.ea, s);
+        prof_end(KK_CONVERT, s);
+        if (e != cudaSuccess) return e;
+        prof_begin(KK_GEMM_TC, s);
+        e = launch_gemm_f64tc(mt, mt, ob, dig.a, dig.a, dig.ea, dig.ea, L21 + (size_t)ob * lda, lda, dig.list,
+                              info, true, s);
+        prof_end(KK_GEMM_TC, s);
+        if (e != cudaSuccess) return e;
+        prof_begin(KK_GEMM_SIMT, s);
+        e = launch_gemm_f64_list(mt, mt, ob, L21, lda, L21, lda, true, L21 + (size_t)ob * lda, lda, true,
+                                 dig.list, s);
+        prof_end(KK_GEMM_SIMT, s);
+        if (e != cudaSuccess) return e;
+        continue;
+      }
       prof_begin(KK_GEMM_SIMT, s);
       e = launch_gemm_simt<double>(mt, mt, ob, -1.0, L21, lda, L21, lda, true, 1.0,
                                    L21 + (size_t)ob * lda, lda, true, s);

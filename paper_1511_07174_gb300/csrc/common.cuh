@@ -82,6 +82,21 @@ GBLA_DEVINL void warp_argmax(double& bv, int& bi) {
   }
 }
 
+// Output tile t -> (row tile, column tile): column-major over the tile grid,
+// or, for the lower triangle of tiles, row by row over (i, j), j <= i.
+GBLA_DEVINL void tile_coords(int t, int tilesM, int lower, int& ti, int& tj) {
+  if (!lower) {
+    ti = t % tilesM;
+    tj = t / tilesM;
+    return;
+  }
+  int i = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while ((long long)(i + 1) * (i + 2) / 2 <= t) ++i;
+  while ((long long)i * (i + 1) / 2 > t) --i;
+  ti = i;
+  tj = t - i * (i + 1) / 2;
+}
+
 // *l = sqrt(d), *rl = 1 / sqrt(d) for d > 0.
 GBLA_DEVINL void sqrt_rcp(float d, float* l, float* rl) {
   *l = sqrtf(d);

@@ -92,6 +92,8 @@ inline int prec_mma_kind(int p) {
 // K-major copies hold kmult * K elements per row ([hi|hi|lo] for L21, [hi|lo|hi] for U12)
 inline int prec_kmult(int p) { return prec_is_split(p) ? 3 : 1; }
 
+struct F64Digits;
+
 // ---- kernel launchers (all stream-ordered; return cudaError_t) -------------
 constexpr int kPanelWidth = 32;  // inner panel width handled by the panel kernels
 constexpr int kPanelSlotW = 72;  // doubles per published candidate slot
@@ -269,13 +271,41 @@ cudaError_t launch_chol_batched(int batch, const int* n, T* const* A, const int*
 
 // ---- Cholesky (chol.cu) ------------------------------------------------------
 // nb: outer block width, a multiple of 64 up to 256 (0: 64)
-cudaError_t launch_chol(int n, double* A, int lda, int nb, int* info, cudaStream_t s);
+cudaError_t launch_chol(int n, double* A, int lda, int nb, int* info, const F64Digits& dig,
+                        cudaStream_t s);
 // Mixed-precision Cholesky of the FP32 lower triangle of F (see chol.cu); the
 // strict upper triangle receives L^t. Ak, Bk: K-major copies (n x ldk of the
 // precision's element), eA: n ints.
 cudaError_t launch_chol_mixed(int n, float* F, int ldf, int nb, int prec, void* Ak, void* Bk, int ldk,
                               int* eA, int* info, cudaStream_t s);
 cudaError_t launch_mirror_lower(int n, float* F, int ldf, cudaStream_t s);
+
+// ---- FP64 trailing update as exact digit products on the tensor cores -----------
+// Scratch of one update C -= A B (M x N x K, K <= 256): the digits of A's rows
+// and B's columns (f64tc_ld(K) 16-bit words per row), one scale word per row
+// and column, and the list of tiles that the digits cannot represent well
+// enough (f64tc_list_ints), which launch_gemm_f64_list then updates in FP64.
+struct F64Digits {
+  void* a = nullptr;
+  void* b = nullptr;  // nullptr: B = A^t (Cholesky), one set of digits
+  int* ea = nullptr;
+  int* eb = nullptr;
+  int* list = nullptr;
+};
+size_t f64tc_ld(int K);
+size_t f64tc_list_ints(int M, int N);
+cudaError_t launch_f64_digits_rows(const double* F, int ldf, int M, int K, void* out, int* scale,
+                                   cudaStream_t s);
+cudaError_t launch_f64_digits_cols(const double* B, int ldb, int N, int K, void* out, int* scale,
+                                   cudaStream_t s);
+cudaError_t launch_gemm_f64tc(int M, int N, int K, const void* Ad, const void* Bd, const int* eA,
+                              const int* eB, double* C, int ldc, int* list, int* info, bool lower,
+                              cudaStream_t s, int grid_cap = 0);
+// C -= A op(B) in FP64 multiply-adds on the listed 128 x 128 tiles (transB and
+// lower together: Cholesky; neither: LU)
+cudaError_t launch_gemm_f64_list(int M, int N, int K, const double* A, int lda, const double* B, int ldb,
+                                 bool transB, double* C, int ldc, bool lower, const int* list,
+                                 cudaStream_t s);
 
 // ---- blocked LU driver (api.cu) ---------------------------------------------
 struct LuWork {
@@ -289,6 +319,7 @@ struct LuWork {
   int* eA;
   int* eB;
   int ldk;
+  F64Digits dig;  // FP64: scratch of the tensor-core update (dig.a == nullptr: FP64 multiply-adds)
 };
 template <typename Ts>
 cudaError_t blocked_lu(int n, Ts* A, int lda, int* ipiv, int* info, int nb, int prec,
