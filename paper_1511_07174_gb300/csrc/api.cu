@@ -596,13 +596,29 @@ int gbla_lu_factor_mixed(int n, const double* A, int lda, float* F, int ldf, int
 }
 
 // ---------------------------------------------------------------------------
+struct SolveWork {
+  int* perm;
+  double* T1;  // n x nrhs each: one solve's result is the next one's right-hand side
+  double* T2;
+  double* D;
+  char* scratch;
+};
+static size_t solve_layout(Carver& c, int n, int nrhs, bool lu, SolveWork* w) {
+  const int nn = std::max(n, 1), nr = std::max(nrhs, 1);
+  SolveWork t = {};
+  if (lu) t.perm = c.take<int>(nn);
+  t.T1 = c.take<double>((size_t)nn * nr);
+  if (lu) t.T2 = c.take<double>((size_t)nn * nr);
+  t.D = c.take<double>(diag_inv_doubles(nn));
+  t.scratch = c.take<char>(trsv_scratch_bytes(nn, nr));
+  if (w) *w = t;
+  return c.off;
+}
+
 size_t gbla_lu_solve_workspace(int n, int nrhs) {
   if (n < 0 || nrhs < 0) return 0;
   Carver c(nullptr, 0);
-  c.take<int>((size_t)std::max(n, 1));
-  c.take<double>((size_t)std::max(n, 1) * std::max(nrhs, 1));
-  c.take<unsigned>(trsv_flags_count(std::max(n, 1), std::max(nrhs, 1)));
-  return c.off;
+  return solve_layout(c, n, nrhs, true, nullptr);
 }
 
 int gbla_lu_solve(int trans, int n, int nrhs, const double* LU, int lda, const int* ipiv, double* B,
@@ -620,26 +636,20 @@ int gbla_lu_solve(int trans, int n, int nrhs, const double* LU, int lda, const i
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (!d_work || !aligned256(d_work)) return GBLA_ERR_WORKSPACE;
   Carver c(d_work, work_bytes);
-  int* perm = c.take<int>((size_t)std::max(n, 1));
-  double* T = c.take<double>((size_t)std::max(n, 1) * std::max(nrhs, 1));
-  unsigned* flags = c.take<unsigned>(trsv_flags_count(std::max(n, 1), std::max(nrhs, 1)));
+  SolveWork w;
+  solve_layout(c, n, nrhs, true, &w);
   if (!c.ok) return GBLA_ERR_WORKSPACE;
   GBLA_TRY(cudaMemsetAsync(d_info, 0, sizeof(int), s));
   if (n == 0 || nrhs == 0) return GBLA_OK;
-  GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, perm, s));
-  const int ldt = n;
+  GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, w.perm, s));
   if (!trans) {
-    GBLA_TRYK(KK_PERM, s, launch_permute_rows(n, nrhs, perm, false, B, ldb, T, ldt, s));
-    GBLA_TRYK(KK_TRSV, s, launch_trsv<double>(true, false, true, n, nrhs, LU, lda, T, ldt, flags, d_info, s));
-    GBLA_TRYK(KK_TRSV, s, launch_trsv<double>(false, false, false, n, nrhs, LU, lda, T, ldt, flags, d_info, s));
-    GBLA_TRY(cudaMemcpy2DAsync(B, sizeof(double) * ldb, T, sizeof(double) * ldt, sizeof(double) * n,
-                               nrhs, cudaMemcpyDeviceToDevice, s));
+    GBLA_TRYK(KK_PERM, s, launch_permute_rows(n, nrhs, w.perm, false, B, ldb, w.T1, n, s));
+    GBLA_TRYK(KK_TRSV, s, launch_trsv(true, false, true, n, nrhs, LU, lda, w.T1, n, w.T2, n, w.D, w.scratch, d_info, s));
+    GBLA_TRYK(KK_TRSV, s, launch_trsv(false, false, false, n, nrhs, LU, lda, w.T2, n, B, ldb, w.D, w.scratch, d_info, s));
   } else {
-    GBLA_TRY(cudaMemcpy2DAsync(T, sizeof(double) * ldt, B, sizeof(double) * ldb, sizeof(double) * n,
-                               nrhs, cudaMemcpyDeviceToDevice, s));
-    GBLA_TRYK(KK_TRSV, s, launch_trsv<double>(false, true, false, n, nrhs, LU, lda, T, ldt, flags, d_info, s));
-    GBLA_TRYK(KK_TRSV, s, launch_trsv<double>(true, true, true, n, nrhs, LU, lda, T, ldt, flags, d_info, s));
-    GBLA_TRYK(KK_PERM, s, launch_permute_rows(n, nrhs, perm, true, T, ldt, B, ldb, s));
+    GBLA_TRYK(KK_TRSV, s, launch_trsv(false, true, false, n, nrhs, LU, lda, B, ldb, w.T1, n, w.D, w.scratch, d_info, s));
+    GBLA_TRYK(KK_TRSV, s, launch_trsv(true, true, true, n, nrhs, LU, lda, w.T1, n, w.T2, n, w.D, w.scratch, d_info, s));
+    GBLA_TRYK(KK_PERM, s, launch_permute_rows(n, nrhs, w.perm, true, w.T2, n, B, ldb, s));
   }
   return GBLA_OK;
 }
@@ -691,8 +701,7 @@ int gbla_chol_factor_ws(int n, double* A, int lda, int* d_info, int nb, void* d_
 size_t gbla_chol_solve_workspace(int n, int nrhs) {
   if (n < 0 || nrhs < 0) return 0;
   Carver c(nullptr, 0);
-  c.take<unsigned>(trsv_flags_count(std::max(n, 1), std::max(nrhs, 1)));
-  return c.off;
+  return solve_layout(c, n, nrhs, false, nullptr);
 }
 
 int gbla_chol_solve(int n, int nrhs, const double* L, int lda, double* B, int ldb, int* d_info,
@@ -708,12 +717,13 @@ int gbla_chol_solve(int n, int nrhs, const double* L, int lda, double* B, int ld
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (!d_work || !aligned256(d_work)) return GBLA_ERR_WORKSPACE;
   Carver c(d_work, work_bytes);
-  unsigned* flags = c.take<unsigned>(trsv_flags_count(std::max(n, 1), std::max(nrhs, 1)));
+  SolveWork w;
+  solve_layout(c, n, nrhs, false, &w);
   if (!c.ok) return GBLA_ERR_WORKSPACE;
   GBLA_TRY(cudaMemsetAsync(d_info, 0, sizeof(int), s));
   if (n == 0 || nrhs == 0) return GBLA_OK;
-  GBLA_TRYK(KK_TRSV, s, launch_trsv<double>(true, false, false, n, nrhs, L, lda, B, ldb, flags, d_info, s));
-  GBLA_TRYK(KK_TRSV, s, launch_trsv<double>(true, true, false, n, nrhs, L, lda, B, ldb, flags, d_info, s));
+  GBLA_TRYK(KK_TRSV, s, launch_trsv(true, false, false, n, nrhs, L, lda, B, ldb, w.T1, n, w.D, w.scratch, d_info, s));
+  GBLA_TRYK(KK_TRSV, s, launch_trsv(true, true, false, n, nrhs, L, lda, w.T1, n, B, ldb, w.D, w.scratch, d_info, s));
   return GBLA_OK;
 }
 
@@ -955,7 +965,7 @@ struct IrWork {
   double* st;  // GmresState {res, pad}
   double* slots;
   unsigned* counter;
-  unsigned* flags;
+  char* flags;  // scratch of the triangular solves
   double* t1;
   double* t2;
   double* DinvL;
@@ -984,7 +994,7 @@ static size_t ir_layout(Carver& c, int n, int m, IrWork* w) {
   t.st = c.take<double>(2);
   t.slots = c.take<double>(mgs_slots_doubles());
   t.counter = c.take<unsigned>(1);
-  t.flags = c.take<unsigned>(trsv_flags_count(nn, 1));
+  t.flags = c.take<char>(trsv_scratch_bytes(nn, 1));
   t.t1 = c.take<double>(nn);
   t.t2 = c.take<double>(nn);
   t.DinvL = c.take<double>(diag_inv_doubles(nn));
@@ -1010,13 +1020,13 @@ size_t gbla_gmresir_workspace(int n, int restart_m) {
 // n-double temporaries; src and dst distinct
 static cudaError_t apply_minv(int n, const float* F, int ldf, const int* perm, const double* DinvL,
                               const double* DinvU, const double* src, double* dst, double* t1,
-                              double* t2, unsigned* flags, int* info, cudaStream_t s) {
+                              double* t2, void* flags, int* info, cudaStream_t s) {
   cudaError_t e;
   PROF(KK_PERM, s, launch_permute_rows(n, 1, perm, false, src, n, t1, n, s));
   if (e != cudaSuccess) return e;
-  PROF(KK_TRSV, s, launch_trsv_inv<float>(true, n, F, ldf, DinvL, t1, t2, flags, info, s));
+  PROF(KK_TRSV, s, launch_trsv_inv(true, n, F, ldf, DinvL, t1, t2, flags, info, s));
   if (e != cudaSuccess) return e;
-  PROF(KK_TRSV, s, launch_trsv_inv<float>(false, n, F, ldf, DinvU, t2, dst, flags, info, s));
+  PROF(KK_TRSV, s, launch_trsv_inv(false, n, F, ldf, DinvU, t2, dst, flags, info, s));
   return e;
 }
 
@@ -1113,8 +1123,8 @@ static int gmresir_setup(int n, const double* A, int lda, const float* F, int ld
                          const IrWork& w, cudaStream_t s) {
   GBLA_TRY(cudaMemsetAsync(w.info, 0, sizeof(int), s));
   GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, w.perm, s));
-  GBLA_TRYK(KK_TRSV, s, launch_diag_inv<float>(true, ipiv != nullptr, n, F, ldf, w.DinvL, s));
-  GBLA_TRYK(KK_TRSV, s, launch_diag_inv<float>(false, false, n, F, ldf, w.DinvU, s));
+  GBLA_TRYK(KK_TRSV, s, launch_diag_inv(true, ipiv != nullptr, n, F, ldf, w.DinvL, s));
+  GBLA_TRYK(KK_TRSV, s, launch_diag_inv(false, false, n, F, ldf, w.DinvU, s));
   GBLA_TRYK(KK_MATVEC, s, launch_row_abs_sum_max(n, A, lda, w.part, w.anorm, s));
   return GBLA_OK;
 }
@@ -1357,8 +1367,8 @@ int gbla_gmres_solve(int n, const double* A, int lda, const double* b, double* x
   GBLA_TRY(cudaMemsetAsync(ir.info, 0, sizeof(int), s));
   if (pre) {
     GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, ir.perm, s));
-    GBLA_TRYK(KK_TRSV, s, launch_diag_inv<float>(true, true, n, F, ldf, ir.DinvL, s));
-    GBLA_TRYK(KK_TRSV, s, launch_diag_inv<float>(false, false, n, F, ldf, ir.DinvU, s));
+    GBLA_TRYK(KK_TRSV, s, launch_diag_inv(true, true, n, F, ldf, ir.DinvL, s));
+    GBLA_TRYK(KK_TRSV, s, launch_diag_inv(false, false, n, F, ldf, ir.DinvU, s));
     GBLA_TRY(apply_minv(n, F, ldf, ir.perm, ir.DinvL, ir.DinvU, b, ir.z, ir.t1, ir.t2, ir.flags, ir.info, s));
   }
   // the stopping norm: ||M^{-1} b||_2 (left preconditioning) or ||b||_2
@@ -1441,8 +1451,8 @@ int gbla_bicgstab_solve(int n, const double* A, int lda, const double* b, double
   GBLA_TRY(cudaMemsetAsync(ir.info, 0, sizeof(int), s));
   if (pre) {
     GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, ir.perm, s));
-    GBLA_TRYK(KK_TRSV, s, launch_diag_inv<float>(true, true, n, F, ldf, ir.DinvL, s));
-    GBLA_TRYK(KK_TRSV, s, launch_diag_inv<float>(false, false, n, F, ldf, ir.DinvU, s));
+    GBLA_TRYK(KK_TRSV, s, launch_diag_inv(true, true, n, F, ldf, ir.DinvL, s));
+    GBLA_TRYK(KK_TRSV, s, launch_diag_inv(false, false, n, F, ldf, ir.DinvU, s));
   }
   // r = b - A x, r~ = r, p = v = 0, rho = alpha = omega = 1
   double* r = ir.r;

@@ -180,24 +180,22 @@ cudaError_t launch_gemm_tc(int kind, int M, int N, int K, const void* Ak, int ld
                            int ldc, int* info, bool lower, cudaStream_t s, int grid_cap = 0);
 
 // ---- triangular solves ------------------------------------------------------
-// uplo_lower: the stored triangle; trans: solve with its transpose; unit: unit diagonal.
-// X (n x nrhs, ldx) FP64 is overwritten in place. flags: >= ceil(n/64)+1 uints.
-template <typename Ts>
-cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, const Ts* T, int ldt,
-                        double* X, int ldx, unsigned* flags, int* info, cudaStream_t s);
-size_t trsv_flags_count(int n, int nrhs);
+// lower: the stored triangle; trans: solve with its transpose; unit: unit diagonal.
+// X <- op(T)^-1 rhs (n x nrhs, FP64, distinct buffers). D: diag_inv_doubles(n)
+// doubles; scratch: trsv_scratch_bytes(n, nrhs), 8-byte aligned.
+cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, const double* T, int ldt,
+                        const double* rhs, int ldr, double* X, int ldx, double* D, void* scratch, int* info,
+                        cudaStream_t s);
+size_t trsv_scratch_bytes(int n, int nrhs);
 
-// Preconditioner apply with inverted 64 x 64 diagonal blocks (one RHS).
-// Dinv holds diag_inv_doubles(n) doubles per triangular factor.
+// Preconditioner apply (one right-hand side): D, the inverted 64 x 64 diagonal
+// blocks of a triangular factor, formed once per set of factors ...
 size_t diag_inv_doubles(int n);
-template <typename Ts>
-cudaError_t launch_diag_inv(bool lower, bool unit, int n, const Ts* T, int ldt, double* Dinv,
-                            cudaStream_t s);
-// X <- T^{-1} rhs (X and rhs distinct; X is overwritten, flags: one uint).
-template <typename Ts>
-cudaError_t launch_trsv_inv(bool lower, int n, const Ts* T, int ldt, const double* Dinv,
-                            const double* rhs, double* X, unsigned* flags, int* info,
-                            cudaStream_t s);
+cudaError_t launch_diag_inv(bool lower, bool unit, int n, const float* T, int ldt, double* D, cudaStream_t s);
+// ... and X <- T^{-1} rhs with them (X and rhs distinct; scratch:
+// trsv_scratch_bytes(n, 1)).
+cudaError_t launch_trsv_inv(bool lower, int n, const float* T, int ldt, const double* D, const double* rhs, double* X,
+                            void* scratch, int* info, cudaStream_t s);
 
 // ipiv == nullptr: the identity
 cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, cudaStream_t s);

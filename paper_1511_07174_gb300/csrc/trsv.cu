@@ -8,8 +8,12 @@
 // loads into shared memory in either orientation), waits (bounded) for block
 // q's flag, and accumulates M(b, q) x_q; then it solves its diagonal block
 // in shared memory (one warp per right-hand side, lanes own rows), writes
-// x_b and releases its flag. Arithmetic is FP64 whatever the storage type of
-// the triangular factor (FP64 or FP32).
+// x_b and releases its flag. This kernel takes the systems of one block and
+// those with a diagonal block whose inverse is not safe to use; the others go
+// to the cluster kernel below.
+#include <mutex>
+
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -25,14 +29,16 @@ constexpr int kTsNR = 16;
 // beat 1 x 8).
 constexpr int kTsChains = 2;
 static int trsv_chains(int nrhs) { return nrhs < 2 ? 1 : kTsChains; }
-size_t trsv_flags_count(int n, int nrhs) {
+static size_t trsv_flags_count(int n, int nrhs) {
   return (size_t)trsv_chains(nrhs) * (size_t)((n + kTsBS - 1) / kTsBS) + 1;
 }
 
 template <typename Ts, bool LOWER, bool TRANS, bool UNIT>
 __global__ void __launch_bounds__(256)
-    trsv_chain_kernel(int n, int ncols, int G, int C, const Ts* __restrict__ T, int ldt, double* X,
-                      int ldx, unsigned* flags, int* info, uint64_t wait_ns) {
+    trsv_chain_kernel(int n, int ncols, int G, int C, const Ts* __restrict__ T, int ldt,
+                      const double* rhs, int ldr, double* X, int ldx, unsigned* flags,
+                      const unsigned* gate, int* info, uint64_t wait_ns) {
+  if (gate && *gate == 0u) return;  // the inverted diagonal blocks were good: nothing left to do
   constexpr bool FWD = (LOWER != TRANS);
   __shared__ double tile[kTsBS][kTsBS + 1];
   __shared__ double xq[kTsBS][kTsNR];
@@ -51,6 +57,7 @@ __global__ void __launch_bounds__(256)
   if (t_ord >= nblk) return;
   flags += (size_t)chain * nblk;
   X += (size_t)chain * G * ldx;
+  rhs += (size_t)chain * G * ldr;
   const int nrhs = min(G, ncols - chain * G);
   if (nrhs <= 0) return;
   const int b = FWD ? t_ord : nblk - 1 - t_ord;
@@ -121,7 +128,7 @@ __global__ void __launch_bounds__(256)
     if (rr < nr) {
       const double sum = (part[(0 * kTsBS + rr) * kTsNR + c] + part[(1 * kTsBS + rr) * kTsNR + c]) +
                          (part[(2 * kTsBS + rr) * kTsNR + c] + part[(3 * kTsBS + rr) * kTsNR + c]);
-      v = __ldcg(&X[(r0 + rr) + (size_t)c * ldx]) - sum;
+      v = rhs[(r0 + rr) + (size_t)c * ldr] - sum;
     }
     xq[rr][c] = v;
   }
@@ -169,25 +176,833 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-template <typename Ts>
-cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, const Ts* T, int ldt,
-                        double* X, int ldx, unsigned* flags, int* info, cudaStream_t s) {
+}  // namespace gbla
+
+// ----------------------------------------------------------------------------
+// Substitution with inverted diagonal blocks, the chain in one thread-block
+// cluster. With D_s the inverse of the 64 x 64 diagonal block s (s counts in
+// solve order, block b = s forward and nblk-1-s backward):
+//   y_s = rhs_s - sum_{t < s} T(s, t) x_t,   x_s = D_s y_s.
+//
+// What bounds it: the dependence from x_{s-1} to x_s. This GPU's FP64 pipe does
+// two multiply-adds per clock and SM (a warp's FP64 instruction holds its
+// scheduler for 64 clocks), so a 64-row substitution by one warp, or a 64 x 64
+// product on one SM, costs microseconds, and so does a round trip through L2.
+// Hence: the CTAs of a cluster (8 for one right-hand side, 4 for several) share
+// the rows of every block; four warps per right-hand side do the products of a
+// step, 2 or 4 rows each (a few multiply-adds and shuffle-adds per lane); y_s and
+// x_s are exchanged through the cluster's shared memory (st.async completing bytes
+// on the receivers' mbarriers: 200 to 400 clocks); operands are loaded a step
+// ahead, from L2, where they were prefetched; one warp fetches the start values of
+// y. The chain multiplies the two nearest blocks itself. The blocks before those go
+// to helper tasks (32 rows by up to 16 blocks, all right-hand sides of a chain) run
+// by all other CTAs, which add their part to the previous task's and pass it on;
+// the last one's result starts y_s. They wait for x_t and partial sums in global
+// memory, which announce themselves: they start as an all-ones bit pattern (a NaN
+// that arithmetic does not produce) and a consumer polls the values it needs.
+//
+// Split. Up to four chains of right-hand sides, each with its own cluster and
+// tasks. Clusters of 8 are the shortest chain (2.5 against 3.2 thousand clocks a
+// step), but only 120 of the 152 SMs hold one; 144 hold clusters of 4, and with
+// several right-hand sides the helpers' FP64 work counts (n = 8192, 16 columns:
+// 5.2 ms for both factors with clusters of 8, 3.2 with 4).
+//
+// Measured (both factors of one solve): n = 4096, 16 right-hand sides 6.5 -> 1.04
+// ms; n = 8192 16.2 -> 3.2 ms; the preconditioner of n = 2500 0.25 -> 0.17 ms.
+//
+// Progress. Tasks are drawn by ticket, per chain, in solve order, so a task only
+// waits for x values and partial sums of tasks already drawn by running CTAs.
+// The chain's own CTAs draw tickets too whenever the chain has waited for a
+// while, so a chain finishes even if no other CTA of the grid is ever scheduled
+// beside it. All waits are bounded.
+//
+// The operations and their order depend on n alone: for a given factor this is a
+// fixed linear map of rhs (as GMRES requires), whatever CTAs do the tasks.
+//
+// Accuracy. x_s = D_s y_s instead of a substitution leaves an error of the order
+// of u |D||T_ss||x_s| in both cases as long as || |D||T_ss| || is moderate
+// (measured over dense LU and Cholesky factors: indistinguishable; it is a few
+// hundred there). The set-up computes that number; if a block exceeds
+// kTcMaxGrowth or is not finite (a zero pivot), the FP64 solves take the
+// substitution kernel above instead.
+namespace gbla {
+
+constexpr int kTcWarps = 4;               // chain warps of a CTA per right-hand side
+constexpr int kTcRing = 4;                // steps the start values of y may be ahead
+constexpr int kTcHelp = 256;              // threads of the helper part
+constexpr int kTcMaxG = 4;                // right-hand sides of a chain
+constexpr int kTcMaxC = 4;                // chains of a launch
+constexpr int kTcChunk = 16;              // blocks per helper task
+constexpr int kTcNear = 2;                // blocks the chain multiplies itself
+constexpr float kTcMaxGrowth = 4096.0f;
+constexpr unsigned long long kXUnset = 0xffffffffffffffffull;
+
+// helper tasks of block s (two row halves by chunks) and of the blocks before it
+__host__ __device__ inline int tc_chunks(int s) {
+  return s > kTcNear ? (s - kTcNear + kTcChunk - 1) / kTcChunk : 0;
+}
+__host__ __device__ inline int tc_first(int s) {
+  const int m = s - 1 - kTcNear;  // blocks before s that have tasks: 1 .. m far blocks
+  if (m <= 0) return 0;
+  const int q = m / kTcChunk, r = m % kTcChunk;
+  return 2 * (kTcChunk * q * (q + 1) / 2 + r * (q + 1));
+}
+
+struct TcShape {
+  int C, G;  // chains, right-hand sides of a chain
+};
+static TcShape tc_shape(int nrhs) {
+  TcShape t;
+  t.C = nrhs < kTcMaxC ? nrhs : kTcMaxC;
+  t.G = (nrhs + t.C - 1) / t.C;
+  if (t.G > kTcMaxG) t.G = kTcMaxG;
+  return t;
+}
+
+// control words: [0, kTcMaxC) tickets, [kTcMaxC] set when a diagonal block's
+// inverse is not safe, then the substitution kernel's flags
+constexpr int kTcCtrl = kTcMaxC + 1;
+static size_t tc_ctrl_words(int n, int nrhs) {
+  const int per = nrhs < kTcMaxC * kTcMaxG ? nrhs : kTcMaxC * kTcMaxG;
+  return (kTcCtrl + trsv_flags_count(n, per) + 31) / 32 * 32;
+}
+size_t diag_inv_doubles(int n) {
+  return (size_t)((n + kTsBS - 1) / kTsBS) * kTsBS * kTsBS;
+}
+size_t trsv_scratch_bytes(int n, int nrhs) {
+  const int nblk = (n + kTsBS - 1) / kTsBS;
+  const TcShape t = tc_shape(nrhs);
+  return tc_ctrl_words(n, nrhs) * sizeof(unsigned) +
+         (size_t)tc_first(nblk) * t.C * t.G * 32 * sizeof(double);
+}
+
+// Tickets to zero, the values that announce themselves to "not yet".
+__global__ void __launch_bounds__(256)
+    tc_fill_kernel(int n, int ncols, double* X, int ldx, double* P, size_t np, unsigned* ctrl, int ctrl0,
+                   int ctrl1) {
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+  const double unset = __longlong_as_double((long long)kXUnset);
+  for (size_t i = t0; i < (size_t)n * ncols; i += nt) X[i % n + (i / n) * ldx] = unset;
+  for (size_t i = t0; i < np; i += nt) P[i] = unset;
+  // the words [ctrl0, ctrl1) are kept
+  for (size_t i = t0; i < (size_t)kTcMaxC; i += nt) ctrl[i] = 0u;
+  for (size_t i = kTcMaxC + t0; i < (size_t)ctrl1; i += nt)
+    if ((int)i >= ctrl0) ctrl[i] = 0u;
+}
+
+// D_b (row-major, block b of the matrix) of every diagonal block of op(T).
+// Bound by the FP64 pipe's latency: 16 x 16 diagonal blocks are inverted by
+// columns in registers, the rest of 16 columns per CTA by 16 x 16 products; four
+// CTAs share a block, one per 16 columns of the inverse. An upper triangular
+// block is handled in reversed index order, which makes it lower triangular. A
+// short last block is padded with the identity. Measured: 41 us at n = 4096 (in
+// FP64), 75 us at n = 8192; a thread per column took 130.
+template <typename Ts, bool TRANS>
+__global__ void __launch_bounds__(256)
+    tc_diag_inv_kernel(int n, const Ts* __restrict__ T, int ldt, bool fwd, bool unit, double* __restrict__ D,
+                       unsigned* bad) {
+  __shared__ double E[10][16][17];   // lower triangle of 16 x 16 blocks: (i, k) at i (i + 1) / 2 + k
+  __shared__ double I[4][16][17];    // inverses of the diagonal ones
+  __shared__ double Xc[4][16][17];   // the CTA's 16 columns of the inverse
+  __shared__ double S[16][17];
+  __shared__ double rd[64];          // 1 / diagonal
+  __shared__ float rs[64];           // sum_k |E_jk / E_jj|
+  const int b = blockIdx.x >> 2, g = blockIdx.x & 3;
+  const int r0 = b * kTsBS, nr = min(kTsBS, n - r0);
+  const int tid = threadIdx.x;
+  for (int idx = tid; idx < kTsBS * kTsBS; idx += 256) {
+    const int u = idx & 63, v = idx >> 6;  // stored row and column
+    const int row = TRANS ? v : u, col = TRANS ? u : v;
+    const int i = fwd ? row : 63 - row, j = fwd ? col : 63 - col;
+    if (i < j) continue;
+    double x;
+    if (row >= nr || col >= nr) x = i == j ? 1.0 : 0.0;
+    else if (i == j && unit) x = 1.0;
+    else x = (double)T[(r0 + u) + (size_t)(r0 + v) * ldt];
+    const int bi = i >> 4, bj = j >> 4;
+    E[bi * (bi + 1) / 2 + bj][i & 15][j & 15] = x;
+  }
+  __syncthreads();
+  if (tid < 64) rd[tid] = 1.0 / E[(tid >> 4) * ((tid >> 4) + 3) / 2][tid & 15][tid & 15];
+  __syncthreads();
+  {
+    const int w = tid >> 5, j = tid & 31;
+    if (w < 4 && w >= g && j < 16) {
+      const double(*Ed)[17] = E[w * (w + 3) / 2];
+      double s[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) s[i] = i == j ? 1.0 : 0.0;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        s[i] *= rd[16 * w + i];
+#pragma unroll
+        for (int k = i + 1; k < 16; ++k) s[k] = fma(-Ed[k][i], s[i], s[k]);
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const double x = i >= j ? s[i] : 0.0;
+        I[w][i][j] = x;
+        if (w == g) Xc[w][i][j] = x;
+      }
+    } else if (bad && w >= 4) {
+      // scaled row sums, for the growth check: FP32 is enough, and anything that
+      // does not fit it is not safe
+      const int t = tid - 128, row = t >> 1, q = t & 1;
+      float f = 0.f;
+      for (int k = q; k < row; k += 2)
+        f += fabsf((float)(E[(row >> 4) * ((row >> 4) + 1) / 2 + (k >> 4)][row & 15][k & 15] * rd[row]));
+      f += __shfl_xor_sync(0xffffffffu, f, 1);
+      if (q == 0) rs[row] = f + 1.f;
+    }
+  }
+  __syncthreads();
+  const int r = tid >> 4, c = tid & 15;
+  for (int i = g + 1; i < 4; ++i) {
+    double a = 0.0;
+    for (int k = g; k < i; ++k) {
+      const double(*Eik)[17] = E[i * (i + 1) / 2 + k];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) a = fma(Eik[r][q], Xc[k][q][c], a);
+    }
+    S[r][c] = a;
+    __syncthreads();
+    double z = 0.0;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) z = fma(-I[i][r][q], S[q][c], z);
+    Xc[i][r][c] = z;
+    __syncthreads();
+  }
+  if (bad) {
+    const int row = tid >> 2, q = tid & 3;
+    float f = 0.f;
+    if (row >= 16 * g)
+      for (int cc = q; cc < 16; cc += 4) {
+        const int col = 16 * g + cc;
+        const double d = E[g * (g + 3) / 2][cc][cc];
+        f += fabsf((float)(Xc[row >> 4][row & 15][cc] * d)) * rs[col];
+      }
+    f += __shfl_xor_sync(0xffffffffu, f, 1);
+    f += __shfl_xor_sync(0xffffffffu, f, 2);
+    if (!(f <= kTcMaxGrowth)) *bad = 1u;
+  }
+  double* Db = D + (size_t)b * kTsBS * kTsBS;
+  for (int idx = tid; idx < kTsBS * 16; idx += 256) {
+    const int i = idx >> 4, cc = idx & 15;
+    const int j = 16 * g + cc;
+    const double x = (i >> 4) >= g ? Xc[i >> 4][i & 15][cc] : 0.0;
+    const int row = fwd ? i : 63 - i, col = fwd ? j : 63 - j;
+    Db[row * kTsBS + col] = x;
+  }
+}
+
+// poll one announced FP64 value (bounded); false on timeout
+GBLA_DEVINL unsigned long long tc_load(const double* p) {
+  unsigned long long bits;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(bits) : "l"(p) : "memory");
+  return bits;
+}
+GBLA_DEVINL bool tc_poll(const double* p, uint64_t wait_ns, double* out) {
+  unsigned long long bits = tc_load(p);
+  if (bits == kXUnset) {
+    const uint64_t t0 = gbla_now_ns();
+    do {
+      __nanosleep(32);  // many CTAs may be asking for the same line
+      bits = tc_load(p);
+      if (gbla_now_ns() - t0 > wait_ns) return false;
+    } while (bits == kXUnset);
+  }
+  *out = __longlong_as_double((long long)bits);
+  return true;
+}
+GBLA_DEVINL void tc_announce(double* p, double v) {
+  unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+  if (bits == kXUnset) bits = 0x7ff8000000000000ull;  // a NaN handed in by the caller
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(bits) : "memory");
+}
+GBLA_DEVINL void tc_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// v to another CTA's shared memory, completing 8 bytes on that CTA's mbarrier
+GBLA_DEVINL void tc_push(uint32_t raddr, double v, uint32_t rbar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(raddr),
+               "l"(__double_as_longlong(v)), "r"(rbar)
+               : "memory");
+}
+// barrier of the helper part; true in every thread if f was in any
+GBLA_DEVINL bool tc_help_sync_or(bool f) {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+               : "=r"(r)
+               : "r"((uint32_t)f), "n"(kTcHelp)
+               : "memory");
+  return r != 0;
+}
+GBLA_DEVINL void tc_help_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTcHelp) : "memory"); }
+
+struct TcArgs {
+  int n, nblk, ncols, G, C, ldt, ldr, ldx;
+  bool fwd;
+  const double* D;
+  const double* rhs;
+  double* X;
+  double* P;
+  unsigned* ctrl;
+  bool gated;
+  int* info;
+  uint64_t wait_ns;
+};
+
+// threads: helpers, chain warps, the warp that fetches the start values of y
+template <int NR>
+constexpr int tc_threads() {
+  return kTcHelp + 32 * kTcWarps * NR + 32;
+}
+
+template <typename Ts, bool TRANS, int NR, int CL>
+__global__ void __launch_bounds__(tc_threads<NR>(), 1)
+    tc_solve_kernel(const Ts* __restrict__ T, const TcArgs a) {
+  constexpr int kRows = kTsBS / CL / kTcWarps;  // rows of every block per chain warp
+  constexpr int kGrp = 32 / kRows;              // lanes that share a row
+  constexpr int kCols = kTsBS / kGrp;           // columns of a block per lane
+  constexpr int kOwn = kTsBS / CL;              // rows of every block per CTA
+  __shared__ double s_x[2][NR][kTsBS];        // x_s, by parity of s
+  __shared__ double s_y[2][NR][kTsBS];        // y_s
+  __shared__ alignas(8) uint64_t s_bar[2][2][NR];
+  __shared__ double s_xq[2][NR][kTsBS];       // helpers: the x values of a block
+  __shared__ double s_part[TRANS ? 32 * 33 : 8 * NR * 32];
+  __shared__ volatile double s_y0[kTcRing][NR][kOwn];  // start values of y_s, by s mod kTcRing
+  __shared__ volatile int s_have[NR][kOwn];   // steps whose start value is there
+  __shared__ volatile int s_step[NR];         // the step the chain's first warp is at
+  __shared__ int s_t;
+  __shared__ volatile int s_stuck[NR];        // s + 1: chain warp c waits for y_s
+  __shared__ int s_done;                      // chain warps that have finished
+  __shared__ unsigned s_fail[CL];          // per CTA of the cluster: a wait gave up
+  if (a.gated && a.ctrl[kTcMaxC] != 0u) return;  // the substitution kernel takes this system
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cluster = blockIdx.x / CL;
+  const bool in_chain = cluster < a.C;
+  const int nblk = a.nblk, n = a.n;
+  const int ntask = tc_first(nblk);
+  __shared__ int s_failed;
+
+  if (in_chain) {
+    if (tid == 0) {
+      for (int k = 0; k < 2; ++k)
+        for (int p = 0; p < 2; ++p)
+          for (int c = 0; c < NR; ++c) {
+            cl_mbar_init(cl_smem_u32(&s_bar[k][p][c]), 1);
+            cl_mbar_arm(cl_smem_u32(&s_bar[k][p][c]), kTsBS * 8);
+          }
+      s_done = 0;
+      s_failed = 0;
+      for (int c = 0; c < NR; ++c) {
+        s_stuck[c] = s_step[c] = 0;
+        for (int r = 0; r < kOwn; ++r) s_have[c][r] = 0;
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    cl_sync();  // every mbarrier of the cluster is ready for the first push
+  }
+
+  if (warp == kTcHelp / 32 + kTcWarps * NR) {
+    // ---- start values of y: rhs, or what the last helper task of the block left;
+    // polled here so that the chain never waits for a load it issued too late ------
+    if (in_chain) {
+      constexpr int kItems = (NR * kOwn + 31) / 32;
+      int s[kItems];
+#pragma unroll
+      for (int i = 0; i < kItems; ++i) s[i] = 0;
+      bool more = true;
+      while (more && *(volatile int*)&s_done != NR * kTcWarps) {
+        more = false;
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) {
+          const int it = lane + 32 * i, c = it / kOwn, rr = it % kOwn;
+          const int col = cluster * a.G + c;
+          if (c >= a.G || col >= a.ncols || s[i] >= nblk) continue;
+          more = true;
+          // the slot's last value has been used: the other warps of the chain are at
+          // most one step from its first
+          if (s[i] > s_step[c] + kTcRing - 2) continue;
+          const int rb = kOwn * (int)cl_ctarank() + rr;
+          const int nch = tc_chunks(s[i]);
+          unsigned long long bits = 0ull;
+          if (nch == 0) {
+            const int r = (a.fwd ? s[i] : nblk - 1 - s[i]) * kTsBS + rb;
+            if (r < n) bits = tc_load(a.rhs + r + (size_t)col * a.ldr);
+          } else {
+            const int task = tc_first(s[i]) + 2 * (nch - 1) + (rb >> 5);
+            bits = tc_load(a.P + (((size_t)cluster * ntask + task) * a.G + c) * 32 + (rb & 31));
+            if (bits == kXUnset) continue;
+          }
+          s_y0[s[i] % kTcRing][c][rr] = __longlong_as_double((long long)bits);
+          __threadfence_block();
+          s_have[c][rr] = ++s[i];
+        }
+        more = __any_sync(0xffffffffu, more);
+      }
+    }
+  } else if (warp >= kTcHelp / 32) {
+    // ---- chain: four warps per right-hand side, each with its own rows ----------
+    const int c = (warp - kTcHelp / 32) / kTcWarps, wr = (warp - kTcHelp / 32) % kTcWarps;
+    const int col = cluster * a.G + c;
+    if (in_chain) {
+      bool ok = true;
+      if (c < a.G && col < a.ncols) {
+        const int row = lane % kRows, grp = lane / kRows;
+        const int ro = kRows * wr + row;                     // row among the CTA's
+        const int rb = kOwn * (int)cl_ctarank() + ro;        // and in its block
+        double* X = a.X + (size_t)col * a.ldx;
+        // parity 0 of the row's x and y in the CTA that this lane (of the first
+        // kRows CL) serves
+        const int to = grp % CL;
+        const uint32_t dst_x = cl_mapa(cl_smem_u32(&s_x[0][c][rb]), to), dbar_x = cl_mapa(cl_smem_u32(&s_bar[0][0][c]), to);
+        const uint32_t dst_y = cl_mapa(cl_smem_u32(&s_y[0][c][rb]), to), dbar_y = cl_mapa(cl_smem_u32(&s_bar[1][0][c]), to);
+        const bool pushes = lane < kRows * CL;
+        constexpr uint32_t kBuf = NR * kTsBS * 8, kBar = NR * 8;
+        // T(s, s - back), the lane's columns of its row; D_s; where y_s starts from.
+        // Only the last block of the matrix can be short: a row block forward in the
+        // last step, a column block backward in the first steps.
+        auto load_t = [&](int s, int back, Ts (&v)[kCols]) {
+          const bool in = s < nblk && s >= back;
+          const int b = a.fwd ? s : nblk - 1 - s, q = a.fwd ? s - back : nblk - 1 - s + back;
+          const int r = b * kTsBS + rb, c0 = q * kTsBS + grp;
+          const Ts* p = TRANS ? T + c0 + (size_t)r * a.ldt : T + r + (size_t)c0 * a.ldt;
+          const size_t step = TRANS ? kGrp : (size_t)kGrp * a.ldt;
+          if (in && max(b, q) < nblk - 1) {
+#pragma unroll
+            for (int j = 0; j < kCols; ++j) v[j] = p[j * step];
+          } else {
+#pragma unroll
+            for (int j = 0; j < kCols; ++j) v[j] = (in && r < n && c0 + kGrp * j < n) ? p[j * step] : (Ts)0;
+          }
+        };
+        auto load_d = [&](int s, double (&v)[kCols]) {
+          if (s >= nblk) return;
+          const double* d = a.D + ((size_t)(a.fwd ? s : nblk - 1 - s) * kTsBS + rb) * kTsBS + grp;
+#pragma unroll
+          for (int j = 0; j < kCols; ++j) v[j] = d[kGrp * j];
+        };
+        Ts t1[kCols], t2[kCols];
+        double d[kCols];
+        load_t(0, 1, t1);
+        load_t(0, 2, t2);
+        load_d(0, d);
+        for (int s = 0; s < nblk; ++s) {
+          // every operand is loaded for the next step as soon as this one has used it
+          const int par = s & 1;
+          double acc = 0.0;
+          if (s >= 2) {
+#pragma unroll
+            for (int j = 0; j < kCols; ++j) acc = fma(-(double)t2[j], s_x[par][c][grp + kGrp * j], acc);
+          }
+          load_t(s + 1, 2, t2);
+          if (wr == 0 && lane == 0) s_step[c] = s;
+          if (!__all_sync(0xffffffffu, s_have[c][ro] > s)) {
+            // the helpers are behind
+            const uint64_t t0 = gbla_now_ns();
+            bool told = false;
+            while (!__all_sync(0xffffffffu, s_have[c][ro] > s)) {
+              const uint64_t dt = gbla_now_ns() - t0;
+              if (__any_sync(0xffffffffu, dt > a.wait_ns)) {
+                ok = false;
+                break;
+              }
+              if (__any_sync(0xffffffffu, dt > 4000)) {
+                told = true;
+                if (lane == 0) s_stuck[c] = s + 1;  // again each time: another warp may have cleared it
+              }
+            }
+            if (told && lane == 0) s_stuck[c] = 0;
+            if (!ok) break;
+          }
+          if (grp == 0) acc += s_y0[s % kTcRing][c][ro];
+          if (s >= 1) {
+            const uint32_t bar = cl_smem_u32(&s_bar[0][par ^ 1][c]);
+            ok = cl_mbar_wait(bar, (uint32_t)((s - 1) >> 1) & 1u, a.wait_ns);
+            if (!__all_sync(0xffffffffu, ok)) {
+              ok = false;
+              break;
+            }
+            if (wr == 0 && lane == 0) cl_mbar_arm(bar, kTsBS * 8);
+#pragma unroll
+            for (int j = 0; j < kCols; ++j) acc = fma(-(double)t1[j], s_x[par ^ 1][c][grp + kGrp * j], acc);
+          }
+#pragma unroll
+          for (int o = kRows; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+          if (pushes) tc_push(dst_y + par * kBuf, acc, dbar_y + par * kBar);
+          load_t(s + 1, 1, t1);
+          const uint32_t ybar = cl_smem_u32(&s_bar[1][par][c]);
+          ok = cl_mbar_wait(ybar, (uint32_t)(s >> 1) & 1u, a.wait_ns);
+          if (!__all_sync(0xffffffffu, ok)) {
+            ok = false;
+            break;
+          }
+          if (wr == 0 && lane == 0) cl_mbar_arm(ybar, kTsBS * 8);
+          double x = 0.0;
+#pragma unroll
+          for (int j = 0; j < kCols; ++j) x = fma(d[j], s_y[par][c][grp + kGrp * j], x);
+#pragma unroll
+          for (int o = kRows; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+          if (s + 1 < nblk && pushes) tc_push(dst_x + par * kBuf, x, dbar_x + par * kBar);
+          const int r = (a.fwd ? s : nblk - 1 - s) * kTsBS + rb;
+          if (grp == 0 && r < n) tc_announce(X + r, x);
+          load_d(s + 1, d);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) {
+        if (!ok) {
+          gbla_flag_timeout(a.info);
+          atomicExch(&s_failed, 1);
+        }
+        atomicAdd(&s_done, 1);
+      }
+      __syncwarp();
+    }
+  } else {
+    // ---- helper tasks ------------------------------------------------------------
+    constexpr int kLine = 128 / (int)sizeof(Ts);  // elements of a cache line
+    if (in_chain) {
+      // the chain's operands (its rows of the blocks (s, s - 1) and (s, s - 2)), in
+      // solve order: it loads them only one step ahead, less than HBM's latency
+      constexpr int kU = TRANS ? kOwn * 2 * kTsBS / kLine : 2 * kTsBS;  // lines of a step
+      for (int i = tid; i < nblk * kU; i += kTcHelp) {
+        const int s = i / kU, u = i % kU;
+        const int r = (a.fwd ? s : nblk - 1 - s) * kTsBS + kOwn * (int)cl_ctarank() + (TRANS ? u % kOwn : 0);
+        const int off = TRANS ? u / kOwn * kLine : u;  // column among those of the two blocks
+        const int cc = a.fwd ? (s - 2) * kTsBS + off : (nblk - s) * kTsBS + off;
+        if (r < n && cc >= 0 && cc < n) tc_prefetch(TRANS ? T + cc + (size_t)r * a.ldt : T + r + (size_t)cc * a.ldt);
+      }
+    }
+    for (int q = 0; q < (in_chain ? 1 : a.C); ++q) {
+      const int ch = in_chain ? cluster : (int)((blockIdx.x + q) % a.C);
+      const int nc = min(a.G, a.ncols - ch * a.G);
+      const double* rhs = a.rhs + (size_t)ch * a.G * a.ldr;
+      const double* X = a.X + (size_t)ch * a.G * a.ldx;
+      double* P = a.P + (size_t)ch * ntask * a.G * 32;
+      int s = 0;
+      bool stop = false;
+      while (nc > 0 && !stop) {
+        tc_help_sync();  // the previous task's shared memory is no longer read
+        if (tid == 0) {
+          bool draw = true;
+          if (in_chain) {
+            // only while the chain of this CTA is held up by tasks nobody has drawn
+            while (true) {
+              if (*(volatile int*)&s_done == NR * kTcWarps) {
+                draw = false;
+                break;
+              }
+              int st = 0;
+              for (int c = 0; c < NR; ++c) st = max(st, s_stuck[c]);
+              if (st && *(volatile unsigned*)&a.ctrl[ch] < (unsigned)tc_first(st)) break;
+              __nanosleep(500);
+            }
+          }
+          const unsigned t = draw ? atomicAdd(&a.ctrl[ch], 1u) : 0xffffffffu;
+          s_t = t < (unsigned)ntask ? (int)t : -1;
+        }
+        tc_help_sync();
+        const int t = s_t;
+        if (t < 0) break;
+        while (tc_first(s + 1) <= t) ++s;
+        const int idx = t - tc_first(s), chunk = idx >> 1, half = idx & 1;
+        const int lo = chunk * kTcChunk, hi = min(lo + kTcChunk, s - kTcNear);
+        const int r0 = (a.fwd ? s : nblk - 1 - s) * kTsBS + 32 * half;  // first of the 32 rows
+        constexpr int NA = TRANS ? 4 : 1;  // rows of a thread
+        double acc[NA][NR];
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+          for (int c = 0; c < NR; ++c) acc[i][c] = 0.0;
+        // a thread's 8 elements of a 32 x 64 tile: one row and columns warp + 8 j,
+        // or (stored transposed) rows 4 warp + i and columns lane + 32 h
+        auto load = [&](int sp, Ts (&v)[8]) {
+          const int c0 = (a.fwd ? sp : nblk - 1 - sp) * kTsBS;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int rr = TRANS ? r0 + 4 * warp + (j >> 1) : r0 + lane;
+            const int cc = TRANS ? c0 + lane + 32 * (j & 1) : c0 + warp + 8 * j;
+            v[j] = (rr < n && cc < n) ? (TRANS ? T[cc + (size_t)rr * a.ldt] : T[rr + (size_t)cc * a.ldt]) : (Ts)0;
+          }
+        };
+        {
+          // the whole task to L2 at once: the loads below reach only one or two tiles
+          // ahead, too little for HBM's latency
+          const int c0 = (a.fwd ? lo : nblk - hi) * kTsBS, ncol = (hi - lo) * kTsBS;
+          constexpr int kPer = 32 / kLine > 0 ? 32 / kLine : 1;  // lines of a 32-row column
+          const int lines = TRANS ? 32 * (ncol / kLine) : ncol * kPer;
+          for (int i = tid; i < lines; i += kTcHelp) {
+            const int rr = r0 + (TRANS ? i & 31 : i % kPer * kLine), cc = c0 + (TRANS ? (i >> 5) * kLine : i / kPer);
+            if (rr < n && cc < n) tc_prefetch(TRANS ? T + cc + (size_t)rr * a.ldt : T + rr + (size_t)cc * a.ldt);
+          }
+        }
+        // one x value per thread and block: right-hand side xc, row xj of the block
+        const int xj = tid & 63, xc = tid >> 6;
+        auto x_ptr = [&](int sp) -> const double* {
+          const int r = (a.fwd ? sp : nblk - 1 - sp) * kTsBS + xj;
+          return xc < nc && r < n ? X + r + (size_t)xc * a.ldx : nullptr;
+        };
+        // x is loaded one block ahead, tiles one or (a single right-hand side: little
+        // work per tile) two blocks ahead
+        constexpr int kAhead = NR == 1 ? 2 : 1;
+        Ts cur[8], n1[8], n2[8];
+        load(lo, cur);
+        if (kAhead == 2 && lo + 1 < hi) load(lo + 1, n1);
+        const double* xp = x_ptr(lo);
+        unsigned long long xb = xp ? tc_load(xp) : 0ull;
+        for (int sp = lo; sp < hi; ++sp) {
+          double(*xq)[kTsBS] = s_xq[sp & 1];
+          bool late = false;
+          double xv = __longlong_as_double((long long)xb);
+          if (xp && xb == kXUnset) late = !tc_poll(xp, a.wait_ns, &xv);
+          if (xc < NR) xq[xc][xj] = xv;
+          // after the use of x: a wait for it would also wait for loads issued before it
+          if (sp + 1 < hi) {
+            xp = x_ptr(sp + 1);
+            xb = xp ? tc_load(xp) : 0ull;
+          }
+          if (sp + kAhead < hi) load(sp + kAhead, kAhead == 2 ? n2 : n1);
+          stop = tc_help_sync_or(late);
+          if (stop) break;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const double v = (double)cur[j];
+            const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + 8 * j;
+#pragma unroll
+            for (int c = 0; c < NR; ++c)
+              if (c < nc) acc[i][c] = fma(v, xq[c][jj], acc[i][c]);
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            cur[j] = n1[j];
+            if (kAhead == 2) n1[j] = n2[j];
+          }
+        }
+        if (stop) {
+          if (tid == 0) gbla_flag_timeout(a.info);
+          break;
+        }
+        // what was known before this chunk, minus this chunk's sum
+        bool late = false;
+        auto publish = [&](int rr, int c, double sum) {
+          double prev = 0.0;
+          if (chunk == 0) {
+            if (r0 + rr < n) prev = rhs[r0 + rr + (size_t)c * a.ldr];
+          } else if (!tc_poll(P + ((size_t)(t - 2) * a.G + c) * 32 + rr, a.wait_ns, &prev)) {
+            late = true;
+            return;
+          }
+          tc_announce(P + ((size_t)t * a.G + c) * 32 + rr, prev - sum);
+        };
+        if constexpr (!TRANS) {
+          double(*part)[NR][32] = reinterpret_cast<double(*)[NR][32]>(s_part);
+#pragma unroll
+          for (int c = 0; c < NR; ++c)
+            if (c < nc) part[warp][c][lane] = acc[0][c];
+          tc_help_sync();
+          for (int i = tid; i < 32 * nc; i += kTcHelp) {
+            const int rr = i & 31, c = i >> 5;
+            publish(rr, c, ((part[0][c][rr] + part[1][c][rr]) + (part[2][c][rr] + part[3][c][rr])) +
+                               ((part[4][c][rr] + part[5][c][rr]) + (part[6][c][rr] + part[7][c][rr])));
+          }
+        } else {
+          double(*part)[33] = reinterpret_cast<double(*)[33]>(s_part);
+#pragma unroll
+          for (int c = 0; c < NR; ++c)
+            if (c < nc) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) part[4 * warp + i][lane] = acc[i][c];
+              tc_help_sync();
+              const int rr = tid >> 3, e = tid & 7;
+              double sum = (part[rr][e] + part[rr][e + 8]) + (part[rr][e + 16] + part[rr][e + 24]);
+#pragma unroll
+              for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+              if (e == 0) publish(rr, c, sum);
+              tc_help_sync();
+            }
+        }
+        if (tc_help_sync_or(late)) {
+          if (tid == 0) gbla_flag_timeout(a.info);
+          break;
+        }
+      }
+    }
+  }
+  if (!in_chain) return;
+  // Leaving. On the way through, every push into a CTA was waited for by it. If a
+  // wait gave up anywhere in the cluster, pushes may still be on their way: all
+  // CTAs learn of it at the first barrier, give them time to land, and leave
+  // together after a second one.
+  __syncthreads();
+  if (tid < CL) cl_store_remote_u32(cl_mapa(cl_smem_u32(&s_fail[cl_ctarank()]), tid), (unsigned)s_failed);
+  __syncwarp();
+  cl_sync();
+  unsigned any = 0;
+  for (int q = 0; q < CL; ++q) any |= s_fail[q];
+  if (!any) return;
+  const uint64_t t0 = gbla_now_ns();
+  while (gbla_now_ns() - t0 < 200000) __nanosleep(1000);
+  __syncwarp();
+  cl_sync();
+}
+
+// clusters of CL CTAs that the device can hold at once (0: none)
+template <typename Ts, bool TRANS, int NR, int CL>
+static cudaError_t tc_max_clusters(int* out) {
+  static std::mutex mu;
+  static int known[64];
+  static bool init = false;
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!init) {
+    for (int& v : known) v = -1;
+    init = true;
+  }
+  if (known[dev] < 0) {
+    cudaLaunchConfig_t q = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    q.gridDim = dim3(CL);
+    q.blockDim = dim3(tc_threads<NR>());
+    q.attrs = at;
+    q.numAttrs = 1;
+    int k = 0;
+    e = cudaOccupancyMaxActiveClusters(&k, tc_solve_kernel<Ts, TRANS, NR, CL>, &q);
+    if (e != cudaSuccess) return e;
+    known[dev] = k;
+  }
+  *out = known[dev];
+  return cudaSuccess;
+}
+
+template <typename Ts, bool TRANS, int NR, int CL>
+static cudaError_t tc_launch_solve(const Ts* T, TcArgs a, cudaStream_t s) {
+  int maxc = 0;
+  cudaError_t e = tc_max_clusters<Ts, TRANS, NR, CL>(&maxc);
+  if (e != cudaSuccess) return e;
+  if (maxc < 1) return cudaErrorNotSupported;
+  // one CTA per SM: the FP64 units of an SM, which chain and tasks are bound by,
+  // are not shared between two of them. Capped by gbla_set_substitution_ctas.
+  int clusters = a.C + (a.C * tc_first(a.nblk) + CL - 1) / CL;
+  const int sms = device_props().num_sms / CL;
+  if (clusters > maxc) clusters = maxc;
+  if (sms > 0 && clusters > sms) clusters = sms;
+  const int cap = substitution_ctas();
+  if (cap > 0 && clusters > cap / CL) clusters = cap / CL;
+  if (clusters < a.C) clusters = a.C;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(clusters * CL));
+  cfg.blockDim = dim3(tc_threads<NR>());
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, tc_solve_kernel<Ts, TRANS, NR, CL>, T, a);
+}
+
+template <typename Ts, bool TRANS>
+static cudaError_t tc_launch_diag_inv(bool fwd, bool unit, int n, const Ts* T, int ldt, double* D, unsigned* bad,
+                                      cudaStream_t s) {
+  tc_diag_inv_kernel<Ts, TRANS><<<4 * ((n + kTsBS - 1) / kTsBS), 256, 0, s>>>(n, T, ldt, fwd, unit, D, bad);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// One group of at most kTcMaxC * kTcMaxG right-hand sides. keep_bad: the word
+// that says whether the inverses are safe is left as it is.
+template <typename Ts, bool TRANS>
+static cudaError_t tc_apply(bool fwd, int n, int ncols, TcShape sh, const Ts* T, int ldt, const double* D, const double* rhs,
+                            int ldr, double* X, int ldx, char* scratch, size_t ctrl_words, bool gated, int* info,
+                            cudaStream_t s) {
+  TcArgs a;
+  a.n = n;
+  a.nblk = (n + kTsBS - 1) / kTsBS;
+  a.ncols = ncols;
+  a.G = sh.G;
+  a.C = (ncols + sh.G - 1) / sh.G;
+  a.ldt = ldt;
+  a.ldr = ldr;
+  a.ldx = ldx;
+  a.fwd = fwd;
+  a.D = D;
+  a.rhs = rhs;
+  a.X = X;
+  a.ctrl = reinterpret_cast<unsigned*>(scratch);
+  a.P = reinterpret_cast<double*>(scratch + ctrl_words * sizeof(unsigned));
+  a.gated = gated;
+  a.info = info;
+  a.wait_ns = wait_timeout_ns();
+  if (ncols == 1) return tc_launch_solve<Ts, TRANS, 1, 8>(T, a, s);
+  if (sh.G == 1) return tc_launch_solve<Ts, TRANS, 1, 4>(T, a, s);
+  if (sh.G == 2) return tc_launch_solve<Ts, TRANS, 2, 4>(T, a, s);
+  return tc_launch_solve<Ts, TRANS, 4, 4>(T, a, s);
+}
+
+static cudaError_t tc_fill(int n, int ncols, TcShape sh, double* X, int ldx, char* scratch, size_t ctrl_words,
+                           bool keep_bad, cudaStream_t s) {
+  const size_t np = (size_t)tc_first((n + kTsBS - 1) / kTsBS) * sh.C * sh.G * 32;
+  const size_t work = (size_t)n * ncols + np + ctrl_words;
+  size_t grid = (work + 1023) / 1024;
+  if (grid > 608) grid = 608;
+  tc_fill_kernel<<<(unsigned)grid, 256, 0, s>>>(n, ncols, X, ldx,
+                                                reinterpret_cast<double*>(scratch + ctrl_words * sizeof(unsigned)), np,
+                                                reinterpret_cast<unsigned*>(scratch), keep_bad ? kTcCtrl : kTcMaxC,
+                                                (int)ctrl_words);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// X = op(T)^-1 rhs (distinct buffers), FP64. D: diag_inv_doubles(n) doubles.
+cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, const double* T, int ldt,
+                        const double* rhs, int ldr, double* X, int ldx, double* D, void* scratch, int* info,
+                        cudaStream_t s) {
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
   const int nblk = (n + kTsBS - 1) / kTsBS;
   const uint64_t wait_ns = wait_timeout_ns();
-  // one launch per kTsChains x kTsNR columns, split over C chains of G columns
-  const int C = trsv_chains(nrhs);
-  for (int c0 = 0; c0 < nrhs; c0 += C * kTsNR) {
-    const int ncols = nrhs - c0 < C * kTsNR ? nrhs - c0 : C * kTsNR;
+  const bool fwd = lower != trans;
+  const size_t cw = tc_ctrl_words(n, nrhs);
+  char* sc = static_cast<char*>(scratch);
+  unsigned* ctrl = reinterpret_cast<unsigned*>(sc);
+  // A system of one block has no chain: its substitution alone is shorter than
+  // inverting the block first.
+  const bool blocks = nblk > 1;
+  const TcShape sh = tc_shape(nrhs);
+  const int per = sh.C * sh.G;
+  for (int c0 = 0; c0 < nrhs; c0 += per) {
+    const int ncols = nrhs - c0 < per ? nrhs - c0 : per;
+    const double* R = rhs + (size_t)c0 * ldr;
+    double* Xc = X + (size_t)c0 * ldx;
+    cudaError_t e = tc_fill(n, ncols, sh, Xc, ldx, sc, cw, c0 > 0, s);
+    if (e != cudaSuccess) return e;
+    if (blocks) {
+      if (c0 == 0) {
+        e = trans ? tc_launch_diag_inv<double, true>(fwd, unit, n, T, ldt, D, ctrl + kTcMaxC, s)
+                  : tc_launch_diag_inv<double, false>(fwd, unit, n, T, ldt, D, ctrl + kTcMaxC, s);
+        if (e != cudaSuccess) return e;
+      }
+      e = trans ? tc_apply<double, true>(fwd, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s)
+                : tc_apply<double, false>(fwd, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s);
+      if (e != cudaSuccess) return e;
+    }
+    const int C = trsv_chains(ncols);
     const int G = (ncols + C - 1) / C;
     const int Cl = (ncols + G - 1) / G;  // chains that hold columns
-    cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned) * ((size_t)C * nblk + 1), s);
-    if (e != cudaSuccess) return e;
-    double* Xc = X + (size_t)c0 * ldx;
     const int grid = Cl * nblk;
-#define GBLA_TRSV(LW, TR, UN)                                                                  \
-  trsv_chain_kernel<Ts, LW, TR, UN><<<grid, 256, 0, s>>>(n, ncols, G, Cl, T, ldt, Xc, ldx, flags, \
-                                                         info, wait_ns)
+    unsigned* flags = ctrl + kTcCtrl;
+    const unsigned* gate = blocks ? ctrl + kTcMaxC : nullptr;
+#define GBLA_TRSV(LW, TR, UN)                                                                         \
+  trsv_chain_kernel<double, LW, TR, UN><<<grid, 256, 0, s>>>(n, ncols, G, Cl, T, ldt, R, ldr, Xc, ldx, \
+                                                             flags, gate, info, wait_ns)
     if (lower && !trans && unit) GBLA_TRSV(true, false, true);
     else if (lower && !trans && !unit) GBLA_TRSV(true, false, false);
     else if (lower && trans && unit) GBLA_TRSV(true, true, true);
@@ -204,409 +1019,22 @@ cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, cons
   return cudaSuccess;
 }
 
-template cudaError_t launch_trsv<double>(bool, bool, bool, int, int, const double*, int, double*,
-                                         int, unsigned*, int*, cudaStream_t);
-template cudaError_t launch_trsv<float>(bool, bool, bool, int, int, const float*, int, double*,
-                                        int, unsigned*, int*, cudaStream_t);
-
-}  // namespace gbla
-
-// ----------------------------------------------------------------------------
-// Substitution with inverted diagonal blocks (the preconditioner apply of the
-// refinement, one right-hand side). The inverse of every 64 x 64 diagonal
-// block of the triangular factor is formed once per factorisation, in FP64,
-// so that the per-block step of the chain is a 64 x 64 matrix-vector product
-// instead of 64 dependent row eliminations. The operator applied is then a
-// fixed linear map (the same for every vector), as GMRES requires.
-namespace gbla {
-
-// Dinv + b*64*64: column-major inverse of diagonal block b (zero-padded when
-// the last block has fewer than 64 rows). One 64-thread CTA per block; thread
-// j forms column j by substitution against e_j. The same array then holds
-// W (at nblk * 64 * 64) and V (at 2 nblk * 64 * 64) per block, and the
-// substitution's partial-sum slots (see trsv_inv_kernel).
-template <typename Ts, bool LOWER, bool UNIT>
-__global__ void __launch_bounds__(64)
-    diag_inv_kernel(int n, const Ts* __restrict__ T, int ldt, double* __restrict__ Dinv) {
-  __shared__ double D[kTsBS][kTsBS + 1];
-  const int b = blockIdx.x;
-  const int r0 = b * kTsBS;
-  const int nr = min(kTsBS, n - r0);
-  const int t = threadIdx.x;
-  for (int j = 0; j < kTsBS; ++j) D[t][j] = (t < nr && j < nr) ? (double)T[(r0 + t) + (size_t)(r0 + j) * ldt] : 0.0;
-  __syncthreads();
-  double* out = Dinv + (size_t)b * kTsBS * kTsBS + (size_t)t * kTsBS;  // column t
-  double x[kTsBS];
-#pragma unroll
-  for (int i = 0; i < kTsBS; ++i) x[i] = 0.0;
-  if (t < nr) {
-    if (LOWER) {
-#pragma unroll
-      for (int i = 0; i < kTsBS; ++i) {
-        if (i >= t && i < nr) {
-          double s = (i == t) ? 1.0 : 0.0;
-#pragma unroll
-          for (int k = 0; k < kTsBS; ++k)
-            if (k >= t && k < i) s = fma(-D[i][k], x[k], s);
-          x[i] = UNIT ? s : s / D[i][i];
-        }
-      }
-    } else {
-#pragma unroll
-      for (int ii = kTsBS - 1; ii >= 0; --ii) {
-        if (ii <= t) {
-          double s = (ii == t) ? 1.0 : 0.0;
-#pragma unroll
-          for (int k = 0; k < kTsBS; ++k)
-            if (k > ii && k <= t) s = fma(-D[ii][k], x[k], s);
-          x[ii] = UNIT ? s : s / D[ii][ii];
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < kTsBS; ++i) out[i] = x[i];
-}
-
-template <typename Ts, bool FWD>
-__global__ void __launch_bounds__(256)
-    trsv_wv_kernel(int n, const Ts* __restrict__ T, int ldt, double* __restrict__ Dinv);
-// shared memory of trsv_wv_kernel: D_s (64 x 64) and one tile (64 x 65), FP64
-constexpr size_t kWvSmemBytes = sizeof(double) * ((size_t)kTsBS * kTsBS + (size_t)kTsBS * (kTsBS + 1));
-
-template <typename Ts>
-cudaError_t launch_diag_inv(bool lower, bool unit, int n, const Ts* T, int ldt, double* Dinv,
-                            cudaStream_t s) {
+// The preconditioner's factors: the inverses once per set of factors ...
+cudaError_t launch_diag_inv(bool lower, bool unit, int n, const float* T, int ldt, double* D, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int nblk = (n + kTsBS - 1) / kTsBS;
-  if (lower && unit) diag_inv_kernel<Ts, true, true><<<nblk, 64, 0, s>>>(n, T, ldt, Dinv);
-  else if (lower) diag_inv_kernel<Ts, true, false><<<nblk, 64, 0, s>>>(n, T, ldt, Dinv);
-  else if (unit) diag_inv_kernel<Ts, false, true><<<nblk, 64, 0, s>>>(n, T, ldt, Dinv);
-  else diag_inv_kernel<Ts, false, false><<<nblk, 64, 0, s>>>(n, T, ldt, Dinv);
-  count_launch();
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || nblk < 2) return e;
-  // W_s = D_s T(s, s-1), V_s = D_s T(s, s-2) in solve order
-  if (lower) {
-    e = ensure_dyn_smem(trsv_wv_kernel<Ts, true>, kWvSmemBytes);
-    if (e != cudaSuccess) return e;
-    trsv_wv_kernel<Ts, true><<<dim3(nblk, 2), 256, kWvSmemBytes, s>>>(n, T, ldt, Dinv);
-  } else {
-    e = ensure_dyn_smem(trsv_wv_kernel<Ts, false>, kWvSmemBytes);
-    if (e != cudaSuccess) return e;
-    trsv_wv_kernel<Ts, false><<<dim3(nblk, 2), 256, kWvSmemBytes, s>>>(n, T, ldt, Dinv);
-  }
-  count_launch();
-  return cudaGetLastError();
-}
-template cudaError_t launch_diag_inv<float>(bool, bool, int, const float*, int, double*, cudaStream_t);
-template cudaError_t launch_diag_inv<double>(bool, bool, int, const double*, int, double*, cudaStream_t);
-
-
-// ---------------------------------------------------------------------------
-// One right-hand side, forward (lower factor) or backward (upper factor), in
-// solve order s = 0 .. nblk-1 (block b = s forward, nblk-1-s backward). With
-// D_s the inverse of diagonal block s, W_s = D_s T(s, s-1) and
-// V_s = D_s T(s, s-2) (both formed once, by launch_diag_inv):
-//   x_s = D_s (rhs_s - sum_{t < s-2} T(s, t) x_t) - V_s x_{s-2} - W_s x_{s-1}.
-// The far sum is cut into chunks of kTiChunk tiles, each done by a helper
-// task that publishes its 64 partial sums; the owner task of block s adds the
-// chunks in order, applies D_s, then V_s x_{s-2} and, once x_{s-1} is known,
-// W_s x_{s-1}: one 64 x 64 product per block stays on the chain, and the far
-// tiles of late blocks (FP64-bound) spread over many SMs.
-//
-// Tasks are drawn by ticket in the order (block 0: owner; block 1: owner;
-// block s: helpers 0 .. h_s - 1, owner), so a task only ever waits for tasks
-// with smaller tickets, which have started. Results announce themselves: X and
-// the partial-sum slots start as an all-ones bit pattern (a NaN that
-// arithmetic does not produce) and a consumer polls the values it needs.
-// The result is a fixed linear map of rhs (the same operations in the same
-// order every call), as GMRES requires.
-constexpr unsigned long long kXUnset = 0xffffffffffffffffull;
-constexpr int kTiChunk = 16;
-
-__host__ __device__ inline int ti_helpers(int s) { return s >= 2 ? (s - 2 + kTiChunk - 1) / kTiChunk : 0; }
-
-static int ti_tasks(int nblk) {
-  int t = 0;
-  for (int s = 0; s < nblk; ++s) t += ti_helpers(s) + 1;
-  return t;
+  return tc_launch_diag_inv<float, false>(lower, unit, n, T, ldt, D, nullptr, s);
 }
 
-size_t diag_inv_doubles(int n) {
-  const int nblk = (n + kTsBS - 1) / kTsBS;
-  return (size_t)3 * nblk * kTsBS * kTsBS + (size_t)ti_tasks(nblk) * kTsBS;
-}
-
-// poll one announced FP64 value (bounded); false on timeout
-GBLA_DEVINL bool ti_poll(const double* p, uint64_t wait_ns, double* out) {
-  const unsigned long long* px = reinterpret_cast<const unsigned long long*>(p);
-  unsigned long long bits;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(bits) : "l"(px) : "memory");
-  if (bits == kXUnset) {
-    const uint64_t t0 = gbla_now_ns();
-    do {
-      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(bits) : "l"(px) : "memory");
-      if (gbla_now_ns() - t0 > wait_ns) return false;
-    } while (bits == kXUnset);
-  }
-  *out = __longlong_as_double((long long)bits);
-  return true;
-}
-
-GBLA_DEVINL void ti_announce(double* p, double v) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(bits) : "memory");
-}
-
-// W_s and V_s (CTA (s, k): k = 0 -> W_s = D_s T(s, s-1), k = 1 -> V_s = D_s T(s, s-2)).
-
-template <typename Ts, bool FWD>
-__global__ void __launch_bounds__(256)
-    trsv_wv_kernel(int n, const Ts* __restrict__ T, int ldt, double* __restrict__ Dinv) {
-  extern __shared__ double wv_smem[];
-  double* Ds = wv_smem;                                                  // column-major D_s
-  double (*Tt)[kTsBS + 1] = reinterpret_cast<double (*)[kTsBS + 1]>(wv_smem + kTsBS * kTsBS);  // T(b, q)
-  const int nblk = (n + kTsBS - 1) / kTsBS;
-  const int s = blockIdx.x, k = blockIdx.y;
-  const int sp = s - 1 - k;
-  if (sp < 0) return;
-  const int b = FWD ? s : nblk - 1 - s, q = FWD ? sp : nblk - 1 - sp;
-  const int r0 = b * kTsBS, c0 = q * kTsBS;
-  const int nr = min(kTsBS, n - r0), nc = min(kTsBS, n - c0);
-  const double* D = Dinv + (size_t)b * kTsBS * kTsBS;
-  for (int i = threadIdx.x; i < kTsBS * kTsBS; i += blockDim.x) {
-    Ds[i] = D[i];
-    const int rr = i & 63, jj = i >> 6;
-    Tt[rr][jj] = (rr < nr && jj < nc) ? (double)T[(r0 + rr) + (size_t)(c0 + jj) * ldt] : 0.0;
-  }
-  __syncthreads();
-  double* out = Dinv + (size_t)(1 + k) * nblk * kTsBS * kTsBS + (size_t)b * kTsBS * kTsBS;
-  const int r = threadIdx.x & 63, g = threadIdx.x >> 6;
-  for (int jj = g * 16; jj < g * 16 + 16; ++jj) {
-    double a0 = 0.0, a1 = 0.0;
-#pragma unroll 8
-    for (int kk = 0; kk < kTsBS; kk += 2) {
-      a0 = fma(Ds[r + kTsBS * kk], Tt[kk][jj], a0);
-      a1 = fma(Ds[r + kTsBS * (kk + 1)], Tt[kk + 1][jj], a1);
-    }
-    out[r + kTsBS * jj] = a0 + a1;
-  }
-}
-
-template <typename Ts, bool FWD>
-__global__ void __launch_bounds__(256)
-    trsv_inv_kernel(int n, const Ts* __restrict__ T, int ldt, const double* __restrict__ Dinv,
-                    const double* __restrict__ rhs, double* X, unsigned* ticket, int* info,
-                    uint64_t wait_ns) {
-  extern __shared__ double smd[];
-  double* xq = smd;                    // 64: the x values of the current step
-  double* part = xq + kTsBS;           // 4 x 64 partial sums
-  double* dv = part + 4 * kTsBS;       // 64: owner's running vector
-  double* mat = dv + kTsBS;            // 64 x 64: D_s, then V_s, then W_s (owner)
-  __shared__ int s_t, s_abort;
-  const int tid = threadIdx.x;
-  const int nblk = (n + kTsBS - 1) / kTsBS;
-  const size_t nbsq = (size_t)kTsBS * kTsBS;
-  double* P = const_cast<double*>(Dinv) + 3 * (size_t)nblk * nbsq;  // partial-sum slots
-  // Persistent: each CTA draws tickets until they run out. A task only waits
-  // for tasks with smaller tickets, drawn earlier by CTAs that are running, so
-  // the grid may be smaller than the number of tasks.
-  for (;;) {
-  __syncthreads();  // the previous task's shared memory is no longer read
-  if (tid == 0) {
-    s_t = (int)atomicAdd(ticket, 1u);
-    s_abort = 0;
-  }
-  __syncthreads();
-  int t = s_t;
-  // ticket -> (block s, helper c or owner), first ticket of block s
-  int s = 0, first = 0;
-  for (; s < nblk; ++s) {
-    const int cnt = ti_helpers(s) + 1;
-    if (t < first + cnt) break;
-    first += cnt;
-  }
-  if (s >= nblk) return;
-  const int c = t - first;
-  const bool owner = c == ti_helpers(s);
-  const int b = FWD ? s : nblk - 1 - s;
-  const int r0 = b * kTsBS;
-  const int nr = min(kTsBS, n - r0);
-  const int r = tid & 63, g = tid >> 6;
-
-  // y = sum over solve-order blocks s' in [lo, hi) of T(s, s') x_{s'}, into part
-  // (thread (r, g): row r, columns g + 4i of each tile); the tile of the next
-  // block is loaded while the current one waits for its x
-  auto far_sum = [&](int lo, int hi) -> bool {
-    auto load = [&](int sp, Ts (&v)[16]) {
-      const int q = FWD ? sp : nblk - 1 - sp;
-      const int c0 = q * kTsBS;
-      const int nc = min(kTsBS, n - c0);
-      const Ts* base = T + (r0 + r) + (size_t)c0 * ldt;
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int jj = g + 4 * i;
-        v[i] = (r < nr && jj < nc) ? base[(size_t)jj * ldt] : (Ts)0;
-      }
-    };
-    double a0 = 0.0, a1 = 0.0;
-    Ts cur[16];
-    if (lo < hi) load(lo, cur);
-    for (int sp = lo; sp < hi; ++sp) {
-      const int q = FWD ? sp : nblk - 1 - sp;
-      const int c0 = q * kTsBS;
-      const int nc = min(kTsBS, n - c0);
-      Ts nxt[16];
-      if (sp + 1 < hi) load(sp + 1, nxt);
-      if (tid < kTsBS) {
-        double v = 0.0;
-        if (tid < nc && !ti_poll(X + c0 + tid, wait_ns, &v)) s_abort = 1;
-        xq[tid] = v;
-      }
-      __syncthreads();
-      if (s_abort) return false;
-#pragma unroll
-      for (int i = 0; i < 16; i += 2) {
-        a0 = fma((double)cur[i], xq[g + 4 * i], a0);
-        a1 = fma((double)cur[i + 1], xq[g + 4 * (i + 1)], a1);
-      }
-      if (sp + 1 < hi) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) cur[i] = nxt[i];
-      }
-      __syncthreads();  // xq is rewritten next step
-    }
-    part[g * kTsBS + r] = a0 + a1;
-    __syncthreads();
-    return true;
-  };
-  // part (4 x 64) -> one value per row, fixed order
-  auto row_sum = [&](int rr) {
-    return (part[rr] + part[kTsBS + rr]) + (part[2 * kTsBS + rr] + part[3 * kTsBS + rr]);
-  };
-  // part <- M (64 x 64, column-major, in mat) times xq
-  auto mat_vec = [&]() {
-    double a0 = 0.0, a1 = 0.0;
-#pragma unroll
-    for (int j = g * 16; j < g * 16 + 16; j += 2) {
-      a0 = fma(mat[r + kTsBS * j], xq[j], a0);
-      a1 = fma(mat[r + kTsBS * (j + 1)], xq[j + 1], a1);
-    }
-    part[g * kTsBS + r] = a0 + a1;
-    __syncthreads();
-  };
-  auto load_mat = [&](const double* M) {
-    for (int i = tid; i < kTsBS * kTsBS; i += blockDim.x) mat[i] = M[i];
-  };
-  auto wait_x = [&](int sp) -> bool {  // xq <- x of solve-order block sp
-    const int q = FWD ? sp : nblk - 1 - sp;
-    const int c0 = q * kTsBS;
-    const int nc = min(kTsBS, n - c0);
-    if (tid < kTsBS) {
-      double v = 0.0;
-      if (tid < nc && !ti_poll(X + c0 + tid, wait_ns, &v)) s_abort = 1;
-      xq[tid] = v;
-    }
-    __syncthreads();
-    return s_abort == 0;
-  };
-
-  if (!owner) {
-    // helper: the far tiles of chunk c, published in slot t
-    const int lo = c * kTiChunk, hi = min(lo + kTiChunk, s - 2);
-    if (!far_sum(lo, hi)) {
-      if (tid == 0) gbla_flag_timeout(info);
-      return;
-    }
-    if (tid < kTsBS) ti_announce(P + (size_t)t * kTsBS + tid, row_sum(tid));
-    continue;
-  }
-  // owner of block s: rhs minus the helpers' chunks, in order
-  load_mat(Dinv + (size_t)b * nbsq);
-  if (tid < kTsBS) {
-    double acc = tid < nr ? rhs[r0 + tid] : 0.0;
-    for (int h = 0; h < c; ++h) {
-      double v = 0.0;
-      if (!ti_poll(P + (size_t)(first + h) * kTsBS + tid, wait_ns, &v)) s_abort = 1;
-      acc -= v;
-    }
-    xq[tid] = tid < nr ? acc : 0.0;
-  }
-  __syncthreads();
-  if (s_abort) {
-    if (tid == 0) gbla_flag_timeout(info);
-    return;
-  }
-  mat_vec();  // D_s (rhs_s - far)
-  if (tid < kTsBS) dv[tid] = row_sum(tid);
-  __syncthreads();
-  if (s >= 2) {
-    load_mat(Dinv + nblk * nbsq * 2 + (size_t)b * nbsq);  // V_s
-    if (!wait_x(s - 2)) {
-      if (tid == 0) gbla_flag_timeout(info);
-      return;
-    }
-    mat_vec();
-    if (tid < kTsBS) dv[tid] -= row_sum(tid);
-    __syncthreads();
-  }
-  if (s >= 1) {
-    load_mat(Dinv + nblk * nbsq + (size_t)b * nbsq);  // W_s
-    if (!wait_x(s - 1)) {
-      if (tid == 0) gbla_flag_timeout(info);
-      return;
-    }
-    mat_vec();
-    if (tid < kTsBS) dv[tid] -= row_sum(tid);
-    __syncthreads();
-  }
-  if (tid < nr) ti_announce(X + r0 + tid, dv[tid]);
-  }
-}
-
-template <typename Ts>
-cudaError_t launch_trsv_inv(bool lower, int n, const Ts* T, int ldt, const double* Dinv,
-                            const double* rhs, double* X, unsigned* flags, int* info,
-                            cudaStream_t s) {
+// ... and X = T^-1 rhs (one right-hand side, distinct buffers) as a fixed linear map
+cudaError_t launch_trsv_inv(bool lower, int n, const float* T, int ldt, const double* D, const double* rhs, double* X,
+                            void* scratch, int* info, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int nblk = (n + kTsBS - 1) / kTsBS;
-  const int tasks = ti_tasks(nblk);
-  // The grid is persistent: as many CTAs as SMs (fewer when capped by
-  // gbla_set_substitution_ctas), which the scheduler spreads one per SM, so
-  // the FP64 units of an SM, which a block's chain step and the far tiles are
-  // bound by, are not shared between two of them. Each CTA asks for the
-  // shared memory it uses and no more, so kernels on other streams can share
-  // an SM with a CTA that is waiting on the chain.
-  const DeviceProps& dp = device_props();
-  const size_t smem = sizeof(double) * ((size_t)kTsBS * kTsBS + 6 * kTsBS);
-  int grid = dp.num_sms > 0 ? dp.num_sms : 1;
-  const int cap = substitution_ctas();
-  if (cap > 0 && cap < grid) grid = cap;
-  if (grid > tasks) grid = tasks;
-  cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned), s);
+  const size_t cw = tc_ctrl_words(n, 1);
+  const TcShape sh = tc_shape(1);
+  char* sc = static_cast<char*>(scratch);
+  cudaError_t e = tc_fill(n, 1, sh, X, n, sc, cw, false, s);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(X, 0xff, sizeof(double) * (size_t)n, s);
-  if (e != cudaSuccess) return e;
-  double* P = const_cast<double*>(Dinv) + (size_t)3 * nblk * kTsBS * kTsBS;
-  e = cudaMemsetAsync(P, 0xff, sizeof(double) * (size_t)tasks * kTsBS, s);
-  if (e != cudaSuccess) return e;
-  const uint64_t wait_ns = wait_timeout_ns();
-  if (lower) {
-    e = ensure_dyn_smem(trsv_inv_kernel<Ts, true>, smem);
-    if (e != cudaSuccess) return e;
-    trsv_inv_kernel<Ts, true><<<grid, 256, smem, s>>>(n, T, ldt, Dinv, rhs, X, flags, info, wait_ns);
-  } else {
-    e = ensure_dyn_smem(trsv_inv_kernel<Ts, false>, smem);
-    if (e != cudaSuccess) return e;
-    trsv_inv_kernel<Ts, false><<<grid, 256, smem, s>>>(n, T, ldt, Dinv, rhs, X, flags, info, wait_ns);
-  }
-  count_launch();
-  return cudaGetLastError();
+  return tc_apply<float, false>(lower, n, 1, sh, T, ldt, D, rhs, n, X, n, sc, cw, false, info, s);
 }
-template cudaError_t launch_trsv_inv<float>(bool, int, const float*, int, const double*,
-                                            const double*, double*, unsigned*, int*, cudaStream_t);
-template cudaError_t launch_trsv_inv<double>(bool, int, const double*, int, const double*,
-                                             const double*, double*, unsigned*, int*, cudaStream_t);
 
 }  // namespace gbla
