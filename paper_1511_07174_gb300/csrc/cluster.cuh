@@ -13,20 +13,15 @@ GBLA_DEVINL uint32_t cl_mapa(uint32_t a, int rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
   return r;
 }
-// Bulk copy of `bytes` (a multiple of 16) from this CTA's shared memory to
-// another CTA's, completing the bytes on that CTA's mbarrier.
-GBLA_DEVINL void cl_bulk_push(uint32_t rdst, uint32_t src, uint32_t bytes, uint32_t rbar) {
+// 16 bytes to another CTA's shared memory, completing them on that CTA's mbarrier.
+GBLA_DEVINL void cl_push16(uint32_t rdst, ulonglong2 v, uint32_t rbar) {
   asm volatile(
-      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          rdst),
-      "r"(src), "r"(bytes), "r"(rbar)
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(rdst),
+      "l"(v.x), "l"(v.y), "r"(rbar)
       : "memory");
 }
 GBLA_DEVINL void cl_store_remote_u32(uint32_t raddr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(raddr), "r"(v) : "memory");
-}
-GBLA_DEVINL void cl_fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 GBLA_DEVINL void cl_mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
