@@ -4,10 +4,8 @@
 //   potf2   -- the 64 x 64 diagonal block factored by one CTA in shared memory
 //              (column by column: d = a_jj, stop with info = j + 1 if d <= 0,
 //              l_jj = sqrt(d), l_ij = a_ij * (1 / l_jj), a_ik -= l_ij l_kj);
-//   trsm    -- the rows below it: L21 = A21 L11^{-t} in two 32-column halves
-//              (one thread per row, its 32 values in registers, the triangle
-//              in shared memory; the second half first receives the update
-//              from the first);
+//   trsm    -- the rows below it: L21 = A21 L11^{-t} (four lanes per row, its
+//              values in registers, the triangle in shared memory);
 //   update  -- A22 -= L21 L21^t on the lower triangle (the SIMT GEMM with its
 //              lower-triangle mask; tiles above the diagonal are skipped):
 //              inside the outer block for its remaining columns, then once
@@ -88,37 +86,46 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// X L11^t = B for the M rows of B (M x kb, ldb); L11 kb x kb lower (kb <= 32),
-// one thread per row with its values in registers.
-constexpr int kCholTrsmW = 32;
+// X L11^t = B for the M rows of B (M x kb, ldb); L11 kb x kb lower (kb <= 64).
+// Four lanes share a row, each with the columns g + 4 t of it in registers; per
+// column one broadcast and the update of the columns to its right. Bound by the
+// FP64 pipe (a warp's instruction takes 64 clocks) and, with few rows, by the
+// chain over the columns; one thread per row would leave two thirds of the
+// schedulers idle at m = 6000 and take four times as long per row.
+constexpr int kCholRows = 32;  // rows per CTA of 128 threads
 
 template <typename T>
 __global__ void __launch_bounds__(128)
     chol_trsm_kernel(int M, int kb, const T* __restrict__ L, int lda, T* __restrict__ B, int ldb) {
-  __shared__ T Ls[kCholTrsmW][kCholTrsmW + 1];
-  __shared__ T rdiag[kCholTrsmW];
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < kCholTrsmW * kCholTrsmW; idx += blockDim.x) {
-    const int r = idx % kCholTrsmW, c = idx / kCholTrsmW;
+  __shared__ T Ls[kCholNb][kCholNb + 1];
+  __shared__ T rdiag[kCholNb];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int row0 = blockIdx.x * kCholRows;
+  for (int idx = tid; idx < kCholNb * kCholNb; idx += 128) {
+    const int r = idx & 63, c = idx >> 6;
     Ls[r][c] = (r < kb && c < kb && r >= c) ? L[r + (size_t)c * lda] : (r == c ? (T)1 : (T)0);
   }
+  const int r = row0 + 8 * (tid >> 5) + (lane & 7), g = lane >> 3;
+  T x[kCholNb / 4];
+#pragma unroll
+  for (int t = 0; t < kCholNb / 4; ++t) x[t] = (r < M && g + 4 * t < kb) ? B[r + (size_t)(g + 4 * t) * ldb] : (T)0;
   __syncthreads();
-  if (tid < kCholTrsmW) rdiag[tid] = (T)1 / Ls[tid][tid];
+  if (tid < kCholNb) rdiag[tid] = (T)1 / Ls[tid][tid];
   __syncthreads();
-  const int row = blockIdx.x * blockDim.x + tid;
-  if (row >= M) return;
-  T x[kCholTrsmW];
 #pragma unroll
-  for (int k = 0; k < kCholTrsmW; ++k) x[k] = k < kb ? B[row + (size_t)k * ldb] : (T)0;
+  for (int j = 0; j < kCholNb; ++j) {
+    const T xj = __shfl_sync(0xffffffffu, x[j / 4], (lane & 7) + 8 * (j & 3)) * rdiag[j];
+    if (g == (j & 3)) x[j / 4] = xj;
 #pragma unroll
-  for (int j = 0; j < kCholTrsmW; ++j) {
-    x[j] *= rdiag[j];
-#pragma unroll
-    for (int k = j + 1; k < kCholTrsmW; ++k) x[k] = fma(-x[j], Ls[k][j], x[k]);
+    for (int t = j / 4; t < kCholNb / 4; ++t) {
+      const int k = g + 4 * t;
+      if (t > j / 4) x[t] = fma(-xj, Ls[k][j], x[t]);
+      else if (k > j) x[t] = fma(-xj, Ls[k][j], x[t]);
+    }
   }
 #pragma unroll
-  for (int k = 0; k < kCholTrsmW; ++k)
-    if (k < kb) B[row + (size_t)k * ldb] = x[k];
+  for (int t = 0; t < kCholNb / 4; ++t)
+    if (r < M && g + 4 * t < kb) B[r + (size_t)(g + 4 * t) * ldb] = x[t];
 }
 
 // One outer block [o0, o0 + ob) in 64-column steps: diagonal block, the
@@ -138,25 +145,12 @@ static cudaError_t chol_outer_block(int n, T* A, int lda, int o0, int ob, int* i
     const int m = n - k0 - kb;
     if (m <= 0) break;
     T* A21 = A11 + kb;
-    // L21 = A21 L11^{-t} in 32-column halves: solve the first half, update the
-    // second with it, solve the second half
-    for (int h0 = 0; h0 < kb; h0 += kCholTrsmW) {
-      const int hb = kb - h0 < kCholTrsmW ? kb - h0 : kCholTrsmW;
-      if (h0 > 0) {
-        prof_begin(KK_GEMM_SIMT, s);
-        e = launch_gemm_simt<T>(m, hb, h0, (T)-1, A21, lda, A11 + h0, lda, true, (T)1,
-                                A21 + (size_t)h0 * lda, lda, false, s);
-        prof_end(KK_GEMM_SIMT, s);
-        if (e != cudaSuccess) return e;
-      }
-      prof_begin(KK_TRSM, s);
-      chol_trsm_kernel<T><<<(m + 127) / 128, 128, 0, s>>>(m, hb, A11 + h0 + (size_t)h0 * lda, lda,
-                                                          A21 + (size_t)h0 * lda, lda);
-      count_launch();
-      prof_end(KK_TRSM, s);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
+    prof_begin(KK_TRSM, s);
+    chol_trsm_kernel<T><<<(m + kCholRows - 1) / kCholRows, 128, 0, s>>>(m, kb, A11, lda, A21, lda);
+    count_launch();
+    prof_end(KK_TRSM, s);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     // the rest of the outer block's columns (lower part): rows k0 + kb .. n,
     // columns k0 + kb .. o0 + ob
     const int nrest = o0 + ob - k0 - kb;
