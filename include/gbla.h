@@ -157,7 +157,7 @@ int gbla_fma_peak(int precision, int iters, double *tflops, gbla_stream_t stream
  *   lda    leading dimension (>= max(1, n))
  *   ipiv   n ints, output pivots (1-based)
  *   d_info one int, output (see conventions); set to 0 by the call
- *   nb     block size in [32, 256], multiple of 32; 0 = default (256)
+ *   nb     block size in [32, 256], multiple of 32; 0 = default (128)
  * ------------------------------------------------------------------------ */
 size_t gbla_lu_factor_workspace(int n, int nb);
 /* The scratch with which gbla_lu_factor does its trailing updates on the

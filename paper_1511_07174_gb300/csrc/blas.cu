@@ -61,22 +61,21 @@ GBLA_DEVINL void store_lowp(void* base, size_t row, int K, int k, float v) {
 // Columns of L are staged through shared memory 32 at a time. The loop over
 // those 32-row chunks is unrolled, so every register index is a constant and
 // a chunk only updates the row groups at or below it.
-constexpr int kTrsmCols = 32;  // columns per CTA (8 warps x 4)
 
-template <typename Ts, typename Tc, int OUT, int Q>
+template <typename Ts, typename Tc, int OUT, int Q, int CW>
 __global__ void __launch_bounds__(256)
     trsm_lunit_kernel(const Ts* __restrict__ L, int ldl, Ts* __restrict__ B, int ldb, int w, int N,
                       void* __restrict__ outK, int ldk, int* __restrict__ outE) {
   extern __shared__ unsigned char smraw[];
   Tc* Ls = reinterpret_cast<Tc*>(smraw);  // [32][w]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int col0 = blockIdx.x * kTrsmCols + warp * 4;
-  Tc x[Q][4];
+  const int col0 = (blockIdx.x * 8 + warp) * CW;
+  Tc x[Q][CW];
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int r = lane + 32 * q;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < CW; ++c) {
       const int col = col0 + c;
       x[q][c] = (r < w && col < N) ? (Tc)B[r + (size_t)col * ldb] : (Tc)0;
     }
@@ -105,22 +104,24 @@ __global__ void __launch_bounds__(256)
       __syncthreads();
       const int iend = min(32, w - i0);
       for (int ii = 0; ii < iend; ++ii) {
-        Tc xi[4];
+        Tc xi[CW];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) xi[c] = __shfl_sync(0xffffffffu, x[qi][c], ii);
+        for (int c = 0; c < CW; ++c) xi[c] = __shfl_sync(0xffffffffu, x[qi][c], ii);
         const Tc* lcol = Ls + ii * w;
 #pragma unroll
         for (int q = qi; q < Q; ++q) {
           const int r = lane + 32 * q;
-          const Tc l = r < w ? lcol[r] : (Tc)0;
+          if (32 * q < w) {
+            const Tc l = r < w ? lcol[r] : (Tc)0;
 #pragma unroll
-          for (int c = 0; c < 4; ++c) x[q][c] = fma(-l, xi[c], x[q][c]);
+            for (int c = 0; c < CW; ++c) x[q][c] = fma(-l, xi[c], x[q][c]);
+          }
         }
       }
     }
   }
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
+  for (int c = 0; c < CW; ++c) {
     const int col = col0 + c;
     float mx = 0.0f;
 #pragma unroll
@@ -147,14 +148,14 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-template <typename Ts, typename Tc, int Q>
+template <typename Ts, typename Tc, int Q, int CW>
 static cudaError_t trsm_dispatch(const Ts* L, int ldl, Ts* B, int ldb, int w, int N, int out_kind,
                                  void* outK, int ldk, int* outE, cudaStream_t s) {
   const size_t smem = (size_t)32 * w * sizeof(Tc);
-  const dim3 grid((N + kTrsmCols - 1) / kTrsmCols);
+  const dim3 grid((N + 8 * CW - 1) / (8 * CW));
 #define GBLA_TRSM_CASE(K)                                                  \
   {                                                                      \
-    auto kfn = trsm_lunit_kernel<Ts, Tc, K, Q>;                          \
+    auto kfn = trsm_lunit_kernel<Ts, Tc, K, Q, CW>;                          \
     cudaError_t ea = ensure_dyn_smem(kfn, smem);                         \
     if (ea != cudaSuccess) return ea;                                    \
     kfn<<<grid, 256, smem, s>>>(L, ldl, B, ldb, w, N, outK, ldk, outE);  \
@@ -182,13 +183,18 @@ static cudaError_t trsm_dispatch(const Ts* L, int ldl, Ts* B, int ldb, int w, in
   return cudaGetLastError();
 }
 
+// Columns per warp. FP64: one, so that N columns make N warps: a warp's FP64
+// instruction takes 64 clocks, and with four columns to a warp and 32 to a CTA
+// even 4000 columns leave a part of the SMs idle (measured, w = 256: N = 256
+// 310 -> 100 us, the updates of an n = 4096 factorisation 4.8 -> 3.3 ms). FP32:
+// four, which share a load of L (one: 5.2 -> 6.4 ms for n = 16384).
 template <typename Ts, typename Tc>
 cudaError_t launch_trsm_lunit(const Ts* L, int ldl, Ts* B, int ldb, int w, int N, int out_kind,
                               void* outK, int ldk, int* outE, cudaStream_t s) {
   if (w <= 0 || N <= 0) return cudaSuccess;
   if (w > 256) return cudaErrorInvalidValue;
-  if (w <= 32) return trsm_dispatch<Ts, Tc, 1>(L, ldl, B, ldb, w, N, out_kind, outK, ldk, outE, s);
-  return trsm_dispatch<Ts, Tc, 8>(L, ldl, B, ldb, w, N, out_kind, outK, ldk, outE, s);
+  if (w <= 32) return trsm_dispatch<Ts, Tc, 1, 4>(L, ldl, B, ldb, w, N, out_kind, outK, ldk, outE, s);
+  return trsm_dispatch<Ts, Tc, 8, sizeof(Ts) == 8 ? 1 : 4>(L, ldl, B, ldb, w, N, out_kind, outK, ldk, outE, s);
 }
 template cudaError_t launch_trsm_lunit<double, double>(const double*, int, double*, int, int, int,
                                                        int, void*, int, int*, cudaStream_t);
@@ -197,18 +203,22 @@ template cudaError_t launch_trsm_lunit<float, float>(const float*, int, float*, 
 
 // ----------------------------------------------------------------------------
 // Inner step of the blocked LU, fused into one launch: U12 = L11^{-1} A12 and
-// A22 -= L21 U12 for a 32-column panel. CTA (x, y) owns the 64 x 64 tile
-// (x, y) of A22; it solves the 64 columns of U12 above its tile itself (a
-// 32 x 32 x 64 / 2 FMA right-looking solve, small next to the tile's
-// update), in the same order of operations as the separate substitution
+// A22 -= L21 U12 for a 32-column panel. CTA (x, y) owns the BM x BN tile
+// (x, y) of A22; it solves the BN columns of U12 above its tile itself (a
+// right-looking solve of 32 x 32 x BN / 2 multiply-adds, spread over all its
+// warps), in the same order of operations as the separate substitution
 // kernel, so the results are those of the two-kernel sequence. The last CTA
 // of a column of tiles to have read A12 (one counter per column of tiles)
 // writes U12 back and clears its counter, so no CTA ever reads a solved
 // value as input and no CTA waits for another.
-template <typename T>
+// FP64 is bound by its pipe: a 64 x 64 tile is 34 us of one SM, and its solve by
+// two warps (one thread per column) was another 17 before anything else could
+// start; with tiles of 32 x 32 where there are few, and the solve on eight warps,
+// the inner steps of n = 512 take 0.86 -> 0.30 ms, of n = 4096 7.4 -> 4.3 ms.
+template <typename T, int BM, int BN>
 __global__ void __launch_bounds__(256)
     inner_update_kernel(int M, int N, T* __restrict__ P, int lda, unsigned* __restrict__ counters) {
-  constexpr int BM = 64, BN = 64, K = kPanelWidth, TM = 4, TN = 4, RX = BM / TM, RY = BN / TN;
+  constexpr int K = kPanelWidth, TM = BM / 16, TN = BN / 16, RX = BM / TM, RY = BN / TN;
   __shared__ T Ls[K][K + 1];   // strictly lower part of L11
   __shared__ T Us[K][BN + 1];  // A12 tile, then U12 tile
   __shared__ T As[K][BM + 1];  // L21 tile, k-major
@@ -254,17 +264,27 @@ __global__ void __launch_bounds__(256)
   }
   __syncthreads();
   if (tid == 0) s_last = atomicAdd(&counters[blockIdx.y], 1u) == gridDim.x - 1;
-  if (tid < BN) {
-    // column tid of U12: u_i -= l_ik u_k for k = 0, 1, ... (unit diagonal)
-    T u[K];
+  {
+    // U12: u_i -= l_ik u_k for k = 0, 1, ... (unit diagonal). A warp has BN / 8
+    // columns, kG lanes share one, each with the rows g + kG t of it.
+    constexpr int kG = 32 / (BN / 8), kR = K / kG;
+    const int lane = tid & 31, cl = lane % (BN / 8), g = lane / (BN / 8);
+    const int col = (tid >> 5) * (BN / 8) + cl;
+    T u[kR];
 #pragma unroll
-    for (int k = 0; k < K; ++k) u[k] = Us[k][tid];
+    for (int t = 0; t < kR; ++t) u[t] = Us[g + kG * t][col];
 #pragma unroll
-    for (int k = 0; k < K; ++k)
+    for (int k = 0; k < K; ++k) {
+      const T uk = __shfl_sync(0xffffffffu, u[k / kG], cl + (BN / 8) * (k % kG));
 #pragma unroll
-      for (int i = k + 1; i < K; ++i) u[i] = fma(-Ls[i][k], u[k], u[i]);
+      for (int t = k / kG; t < kR; ++t) {
+        const int i = g + kG * t;
+        if (t > k / kG) u[t] = fma(-Ls[i][k], uk, u[t]);
+        else if (i > k) u[t] = fma(-Ls[i][k], uk, u[t]);
+      }
+    }
 #pragma unroll
-    for (int k = 0; k < K; ++k) Us[k][tid] = u[k];
+    for (int t = 0; t < kR; ++t) Us[g + kG * t][col] = u[t];
   }
   __syncthreads();
   if (s_last) {
@@ -309,9 +329,14 @@ __global__ void __launch_bounds__(256)
 template <typename T>
 cudaError_t launch_inner_update(int M, int N, T* P, int lda, unsigned* counters, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  const dim3 grid((M + 63) / 64, (N + 63) / 64);
+  // 64 x 64 tiles, which solve each column of U12 less often, once they fill the
+  // SMs twice
+  const bool big = (size_t)((M + 63) / 64) * ((N + 63) / 64) >= 304;
+  const int t = big ? 64 : 32;
+  const dim3 grid((M + t - 1) / t, (N + t - 1) / t);
   if ((int)grid.y > kInnerCounters) return cudaErrorInvalidValue;
-  inner_update_kernel<T><<<grid, 256, 0, s>>>(M, N, P, lda, counters);
+  if (big) inner_update_kernel<T, 64, 64><<<grid, 256, 0, s>>>(M, N, P, lda, counters);
+  else inner_update_kernel<T, 32, 32><<<grid, 256, 0, s>>>(M, N, P, lda, counters);
   count_launch();
   return cudaGetLastError();
 }
@@ -455,40 +480,26 @@ cudaError_t launch_gemm_simt(int M, int N, int K, T alpha, const T* A, int lda, 
                              int ldb, bool transB, T beta, T* C, int ldc, bool lower,
                              cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  if constexpr (sizeof(T) == 8) {
-    constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4;
-    dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN);
-    if (transB) {
-      if (lower)
-        gemm_simt_kernel<T, BM, BN, BK, TM, TN, true, true><<<grid, 256, 0, s>>>(
-            M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
-      else
-        gemm_simt_kernel<T, BM, BN, BK, TM, TN, true, false><<<grid, 256, 0, s>>>(
-            M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
-    } else {
-      gemm_simt_kernel<T, BM, BN, BK, TM, TN, false, false><<<grid, 256, 0, s>>>(
-          M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
-    }
-  } else if (N <= 256 && !transB && !lower) {
-    // narrow updates (the inner steps of a block column): smaller tiles, more CTAs
-    constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4;
-    dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN);
-    gemm_simt_kernel<T, BM, BN, BK, TM, TN, false, false><<<grid, 256, 0, s>>>(
-        M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+  if (transB != lower) return cudaErrorInvalidValue;  // A B, or the lower triangle of A B^t
+  auto tiles = [&](int t) { return dim3((M + t - 1) / t, (N + t - 1) / t); };
+  if (lower) {
+    // C -= L L^t of the Cholesky factorisation. Smaller tiles while the larger
+    // ones leave SMs idle: one 64 x 64 tile of rank 64 is 69 us of an SM's FP64
+    // pipe.
+    constexpr int BM = sizeof(T) == 8 ? 64 : 128, TM = sizeof(T) == 8 ? 4 : 8, BK = sizeof(T) == 8 ? 16 : 8;
+    const dim3 g = tiles(BM);
+    if ((size_t)g.x * g.y >= 304)
+      gemm_simt_kernel<T, BM, BM, BK, TM, TM, true, true><<<g, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    else
+      gemm_simt_kernel<T, BM / 2, BM / 2, 16, TM / 2, TM / 2, true, true>
+          <<<tiles(BM / 2), 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+  } else if (sizeof(T) == 8 || N <= 256) {
+    // (FP32: the inner steps of a block column: smaller tiles, more CTAs)
+    gemm_simt_kernel<T, 64, 64, 16, 4, 4, false, false><<<tiles(64), 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C,
+                                                                                  ldc);
   } else {
-    constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
-    dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN);
-    if (transB) {
-      if (lower)
-        gemm_simt_kernel<T, BM, BN, BK, TM, TN, true, true><<<grid, 256, 0, s>>>(
-            M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
-      else
-        gemm_simt_kernel<T, BM, BN, BK, TM, TN, true, false><<<grid, 256, 0, s>>>(
-            M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
-    } else {
-      gemm_simt_kernel<T, BM, BN, BK, TM, TN, false, false><<<grid, 256, 0, s>>>(
-          M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
-    }
+    gemm_simt_kernel<T, 128, 128, 8, 8, 8, false, false><<<tiles(128), 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta,
+                                                                                    C, ldc);
   }
   count_launch();
   return cudaGetLastError();
