@@ -219,12 +219,15 @@ __global__ void __launch_bounds__(256)
 // The operations and their order depend on n alone: for a given factor this is a
 // fixed linear map of rhs (as GMRES requires), whatever CTAs do the tasks.
 //
-// Accuracy. x_s = D_s y_s instead of a substitution leaves an error of the order
-// of u |D||T_ss||x_s| in both cases as long as || |D||T_ss| || is moderate
-// (measured over dense LU and Cholesky factors: indistinguishable; it is a few
-// hundred there). The set-up computes that number; if a block exceeds
-// kTcMaxGrowth or is not finite (a zero pivot), the FP64 solves take the
-// substitution kernel above instead.
+// Accuracy. With g = || |D||T_ss| || the product x_s = D_s y_s leaves a residual of
+// up to g u |T_ss||x_s| where a substitution leaves u |T_ss||x_s|. g is a few hundred
+// for most blocks of dense LU and Cholesky factors, where the two cannot be told
+// apart in the solution (n = 512 .. 1500, L and U, against extended precision), and
+// now and then thousands (a small pivot inside a block). The set-up computes it:
+// blocks above kTcRefine get one step of refinement, x_s += D_s (y_s - T_ss x_s),
+// which brings the residual down by another factor g u; with a block above
+// kTcMaxGrowth, or one that is not finite (a zero pivot), the FP64 solves take the
+// substitution kernel above instead. The preconditioner needs neither.
 namespace gbla {
 
 constexpr int kTcWarps = 4;               // chain warps of a CTA per right-hand side
@@ -234,7 +237,8 @@ constexpr int kTcMaxG = 4;                // right-hand sides of a chain
 constexpr int kTcMaxC = 4;                // chains of a launch
 constexpr int kTcChunk = 16;              // blocks per helper task
 constexpr int kTcNear = 2;                // blocks the chain multiplies itself
-constexpr float kTcMaxGrowth = 4096.0f;
+constexpr float kTcRefine = 1024.0f;
+constexpr float kTcMaxGrowth = 1e8f;
 constexpr unsigned long long kXUnset = 0xffffffffffffffffull;
 
 // helper tasks of block s (two row halves by chunks) and of the blocks before it
@@ -260,11 +264,12 @@ static TcShape tc_shape(int nrhs) {
 }
 
 // control words: [0, kTcMaxC) tickets, [kTcMaxC] set when a diagonal block's
-// inverse is not safe, then the substitution kernel's flags
+// inverse is not safe, a word per block set when it is to be refined, then the
+// substitution kernel's flags
 constexpr int kTcCtrl = kTcMaxC + 1;
 static size_t tc_ctrl_words(int n, int nrhs) {
   const int per = nrhs < kTcMaxC * kTcMaxG ? nrhs : kTcMaxC * kTcMaxG;
-  return (kTcCtrl + trsv_flags_count(n, per) + 31) / 32 * 32;
+  return (kTcCtrl + (n + kTsBS - 1) / kTsBS + trsv_flags_count(n, per) + 31) / 32 * 32;
 }
 size_t diag_inv_doubles(int n) {
   return (size_t)((n + kTsBS - 1) / kTsBS) * kTsBS * kTsBS;
@@ -284,10 +289,9 @@ __global__ void __launch_bounds__(256)
   const double unset = __longlong_as_double((long long)kXUnset);
   for (size_t i = t0; i < (size_t)n * ncols; i += nt) X[i % n + (i / n) * ldx] = unset;
   for (size_t i = t0; i < np; i += nt) P[i] = unset;
-  // the words [ctrl0, ctrl1) are kept
+  // what the set-up found, the words [kTcMaxC, ctrl0), is kept
   for (size_t i = t0; i < (size_t)kTcMaxC; i += nt) ctrl[i] = 0u;
-  for (size_t i = kTcMaxC + t0; i < (size_t)ctrl1; i += nt)
-    if ((int)i >= ctrl0) ctrl[i] = 0u;
+  for (size_t i = ctrl0 + t0; i < (size_t)ctrl1; i += nt) ctrl[i] = 0u;
 }
 
 // D_b (row-major, block b of the matrix) of every diagonal block of op(T).
@@ -384,6 +388,7 @@ __global__ void __launch_bounds__(256)
     f += __shfl_xor_sync(0xffffffffu, f, 1);
     f += __shfl_xor_sync(0xffffffffu, f, 2);
     if (!(f <= kTcMaxGrowth)) *bad = 1u;
+    if (f > kTcRefine) bad[1 + b] = 1u;
   }
   double* Db = D + (size_t)b * kTsBS * kTsBS;
   for (int idx = tid; idx < kTsBS * 16; idx += 256) {
@@ -439,7 +444,7 @@ GBLA_DEVINL void tc_help_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTcHelp) 
 
 struct TcArgs {
   int n, nblk, ncols, G, C, ldt, ldr, ldx;
-  bool fwd;
+  bool fwd, unit;
   const double* D;
   const double* rhs;
   double* X;
@@ -587,6 +592,34 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
         load_t(0, 1, t1);
         load_t(0, 2, t2);
         load_d(0, d);
+        auto load_hard = [&](int s) {
+          return a.gated && s < nblk ? a.ctrl[kTcCtrl + (a.fwd ? s : nblk - 1 - s)] : 0u;
+        };
+        unsigned hard = load_hard(0);
+        int ny = 0;  // exchanges through s_y so far: one per step, three in a refined one
+        // v of every row to every CTA; false if a wait gave up
+        auto exchange_y = [&](double v) -> bool {
+          const int p = ny & 1;
+          if (pushes) tc_push(dst_y + p * kBuf, v, dbar_y + p * kBar);
+          const uint32_t ybar = cl_smem_u32(&s_bar[1][p][c]);
+          const bool got = cl_mbar_wait(ybar, (uint32_t)(ny >> 1) & 1u, a.wait_ns);
+          if (!__all_sync(0xffffffffu, got)) return false;
+          if (wr == 0 && lane == 0) cl_mbar_arm(ybar, kTsBS * 8);
+          ++ny;
+          return true;
+        };
+        auto row_sum = [&](double v) {
+#pragma unroll
+          for (int o = kRows; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          return v;
+        };
+        auto times_d = [&](double (&dd)[kCols]) {  // D_s times what the last exchange brought
+          const double* yv = s_y[(ny - 1) & 1][c];
+          double v = 0.0;
+#pragma unroll
+          for (int j = 0; j < kCols; ++j) v = fma(dd[j], yv[grp + kGrp * j], v);
+          return row_sum(v);
+        };
         for (int s = 0; s < nblk; ++s) {
           // every operand is loaded for the next step as soon as this one has used it
           const int par = s & 1;
@@ -627,26 +660,34 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
 #pragma unroll
             for (int j = 0; j < kCols; ++j) acc = fma(-(double)t1[j], s_x[par ^ 1][c][grp + kGrp * j], acc);
           }
-#pragma unroll
-          for (int o = kRows; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-          if (pushes) tc_push(dst_y + par * kBuf, acc, dbar_y + par * kBar);
+          acc = row_sum(acc);
           load_t(s + 1, 1, t1);
-          const uint32_t ybar = cl_smem_u32(&s_bar[1][par][c]);
-          ok = cl_mbar_wait(ybar, (uint32_t)(s >> 1) & 1u, a.wait_ns);
-          if (!__all_sync(0xffffffffu, ok)) {
-            ok = false;
-            break;
+          ok = exchange_y(acc);
+          if (!ok) break;
+          double x = times_d(d);
+          if (hard != 0u) {
+            // x += D (y - T_ss x)
+            ok = exchange_y(x);
+            if (!ok) break;
+            const int b0 = (a.fwd ? s : nblk - 1 - s) * kTsBS, r = b0 + rb;
+            const double* xv = s_y[(ny - 1) & 1][c];
+            double res = grp == 0 ? acc : 0.0;
+            for (int j = 0; j < kCols; ++j) {
+              const int cc = grp + kGrp * j, gc = b0 + cc;
+              if (r >= n || gc >= n || (a.fwd ? cc > rb : cc < rb)) continue;
+              const double tv = cc == rb && a.unit ? 1.0 : (double)(TRANS ? T[gc + (size_t)r * a.ldt] : T[r + (size_t)gc * a.ldt]);
+              res = fma(-tv, xv[cc], res);
+            }
+            res = row_sum(res);
+            ok = exchange_y(res);
+            if (!ok) break;
+            x += times_d(d);
           }
-          if (wr == 0 && lane == 0) cl_mbar_arm(ybar, kTsBS * 8);
-          double x = 0.0;
-#pragma unroll
-          for (int j = 0; j < kCols; ++j) x = fma(d[j], s_y[par][c][grp + kGrp * j], x);
-#pragma unroll
-          for (int o = kRows; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
           if (s + 1 < nblk && pushes) tc_push(dst_x + par * kBuf, x, dbar_x + par * kBar);
           const int r = (a.fwd ? s : nblk - 1 - s) * kTsBS + rb;
           if (grp == 0 && r < n) tc_announce(X + r, x);
           load_d(s + 1, d);
+          hard = load_hard(s + 1);
         }
       }
       __syncwarp();
@@ -921,7 +962,7 @@ static cudaError_t tc_launch_diag_inv(bool fwd, bool unit, int n, const Ts* T, i
 // One group of at most kTcMaxC * kTcMaxG right-hand sides. keep_bad: the word
 // that says whether the inverses are safe is left as it is.
 template <typename Ts, bool TRANS>
-static cudaError_t tc_apply(bool fwd, int n, int ncols, TcShape sh, const Ts* T, int ldt, const double* D, const double* rhs,
+static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, const Ts* T, int ldt, const double* D, const double* rhs,
                             int ldr, double* X, int ldx, char* scratch, size_t ctrl_words, bool gated, int* info,
                             cudaStream_t s) {
   TcArgs a;
@@ -934,6 +975,7 @@ static cudaError_t tc_apply(bool fwd, int n, int ncols, TcShape sh, const Ts* T,
   a.ldr = ldr;
   a.ldx = ldx;
   a.fwd = fwd;
+  a.unit = unit;
   a.D = D;
   a.rhs = rhs;
   a.X = X;
@@ -956,7 +998,8 @@ static cudaError_t tc_fill(int n, int ncols, TcShape sh, double* X, int ldx, cha
   if (grid > 608) grid = 608;
   tc_fill_kernel<<<(unsigned)grid, 256, 0, s>>>(n, ncols, X, ldx,
                                                 reinterpret_cast<double*>(scratch + ctrl_words * sizeof(unsigned)), np,
-                                                reinterpret_cast<unsigned*>(scratch), keep_bad ? kTcCtrl : kTcMaxC,
+                                                reinterpret_cast<unsigned*>(scratch),
+                                                keep_bad ? kTcCtrl + (n + kTsBS - 1) / kTsBS : kTcMaxC,
                                                 (int)ctrl_words);
   count_launch();
   return cudaGetLastError();
@@ -990,15 +1033,15 @@ cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, cons
                   : tc_launch_diag_inv<double, false>(fwd, unit, n, T, ldt, D, ctrl + kTcMaxC, s);
         if (e != cudaSuccess) return e;
       }
-      e = trans ? tc_apply<double, true>(fwd, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s)
-                : tc_apply<double, false>(fwd, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s);
+      e = trans ? tc_apply<double, true>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s)
+                : tc_apply<double, false>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s);
       if (e != cudaSuccess) return e;
     }
     const int C = trsv_chains(ncols);
     const int G = (ncols + C - 1) / C;
     const int Cl = (ncols + G - 1) / G;  // chains that hold columns
     const int grid = Cl * nblk;
-    unsigned* flags = ctrl + kTcCtrl;
+    unsigned* flags = ctrl + kTcCtrl + nblk;
     const unsigned* gate = blocks ? ctrl + kTcMaxC : nullptr;
 #define GBLA_TRSV(LW, TR, UN)                                                                         \
   trsv_chain_kernel<double, LW, TR, UN><<<grid, 256, 0, s>>>(n, ncols, G, Cl, T, ldt, R, ldr, Xc, ldx, \
@@ -1034,7 +1077,7 @@ cudaError_t launch_trsv_inv(bool lower, int n, const float* T, int ldt, const do
   char* sc = static_cast<char*>(scratch);
   cudaError_t e = tc_fill(n, 1, sh, X, n, sc, cw, false, s);
   if (e != cudaSuccess) return e;
-  return tc_apply<float, false>(lower, n, 1, sh, T, ldt, D, rhs, n, X, n, sc, cw, false, info, s);
+  return tc_apply<float, false>(lower, false, n, 1, sh, T, ldt, D, rhs, n, X, n, sc, cw, false, info, s);
 }
 
 }  // namespace gbla

@@ -77,6 +77,20 @@ def test_unsafe_diagonal_block_is_substituted():
     assert _residual(M, X, B, False) <= 8 * n * EPS
 
 
+@pytest.mark.parametrize("trans", [False, True])
+def test_badly_conditioned_diagonal_block_is_refined(trans):
+    # the inverse of this block has elements of size 1.25^62 (about 1e6)
+    n = 320
+    M, ipiv = _factors(n, 6)
+    M[64:128, 64:128] = torch.tril(M[64:128, 64:128], -1) - 0.25 * torch.triu(torch.ones(64, 64, dtype=M.dtype, device=M.device), 1) \
+        + torch.eye(64, dtype=M.dtype, device=M.device)
+    X = torch.randn((n, 3), dtype=torch.float64).cuda()
+    L = torch.tril(M, -1) + torch.eye(n, dtype=M.dtype, device=M.device)
+    B = torch.triu(M).t() @ (L.t() @ X) if trans else L @ (torch.triu(M) @ X)
+    X = api.lu_solve(M, ipiv, B, trans=trans)
+    assert _residual(M, X, B, trans) <= 8 * n * EPS
+
+
 def test_zero_pivot_and_nan_follow_ieee():
     n = 200
     M, ipiv = _factors(n, 7)
