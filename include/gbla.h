@@ -284,6 +284,9 @@ typedef struct {
 } gbla_gmresir_stats;
 
 size_t gbla_gmresir_workspace(int n, int restart_m);
+/* Room for min(nrhs, 4) columns that are refined together (see
+ * gbla_gmresir_solve_nrhs). */
+size_t gbla_gmresir_workspace_nrhs(int n, int nrhs, int restart_m);
 int gbla_gmresir_solve(int n, const double *A, int lda, const float *F, int ldf,
                        const int *ipiv, const double *b, double *x,
                        const gbla_gmresir_opts *opts, gbla_gmresir_stats *stats,
@@ -291,8 +294,11 @@ int gbla_gmresir_solve(int n, const double *A, int lda, const float *F, int ldf,
 
 /* The same refinement for nrhs right-hand sides (B, X: n x nrhs, ldb, ldx),
  * sharing one set-up of the factors (pivot permutation, inverted diagonal
- * blocks) and one workspace (gbla_gmresir_workspace(n, restart_m)); each
- * column is refined on its own, with its own entry of stats[0 .. nrhs).
+ * blocks) and one workspace; each column is refined on its own, with its own
+ * entry of stats[0 .. nrhs). Up to four columns share the launches of an
+ * iteration: as many as the workspace has room for, at least
+ * gbla_gmresir_workspace(n, restart_m), for four of them
+ * gbla_gmresir_workspace_nrhs(n, nrhs, restart_m).
  * Returns 0 when every column converged, GBLA_ERR_NOT_CONVERGED when one or
  * more did not (see stats[k].converged), GBLA_ERR_TIMEOUT on a wait that gave
  * up. Synchronous, like gbla_gmresir_solve. */

@@ -72,6 +72,7 @@ _SIGS = {
     "gbla_lu_factor_mixed_workspace": ([_i, _i, _i], _sz),
     "gbla_lu_factor_mixed": ([_i, _vp, _i, _vp, _i, _vp, _vp, _i, _i, _vp, _sz, _vp], _i),
     "gbla_gmresir_workspace": ([_i, _i], _sz),
+    "gbla_gmresir_workspace_nrhs": ([_i, _i, _i], _sz),
     "gbla_gmresir_solve": ([_i, _vp, _i, _vp, _i, _vp, _vp, _vp, ctypes.POINTER(GmresirOpts),
                             ctypes.POINTER(GmresirStats), _vp, _sz, _vp], _i),
     "gbla_gmresir_solve_nrhs": ([_i, _i, _vp, _i, _vp, _i, _vp, _vp, _i, _vp, _i,

@@ -172,7 +172,7 @@ def gmresir(A, F, ipiv, b, tol=1e-14, inner_tol=1e-8, max_outer=10, restart_m=50
     Ac = colmajor(A, torch.float64)
     Fc = colmajor(F, torch.float32)
     opts = _lib.GmresirOpts(tol, inner_tol, max_outer, restart_m, restarts)
-    ws = _ws(L.gbla_gmresir_workspace(n, restart_m), A.device)
+    ws = _ws(L.gbla_gmresir_workspace_nrhs(n, b.shape[1] if b.dim() == 2 else 1, restart_m), A.device)
     if b.dim() == 2:
         Bc = colmajor(b, torch.float64)
         k = Bc.shape[1]
@@ -270,7 +270,7 @@ def chol_gmresir(A, F, b, tol=1e-14, inner_tol=1e-8, max_outer=10, restart_m=50,
     X = torch.empty_strided((n, k), (1, max(1, n)), dtype=torch.float64, device=A.device)
     opts = _lib.GmresirOpts(tol, inner_tol, max_outer, restart_m, restarts)
     st = (_lib.GmresirStats * max(k, 1))()
-    ws = _ws(L.gbla_gmresir_workspace(n, restart_m), A.device)
+    ws = _ws(L.gbla_gmresir_workspace_nrhs(n, k, restart_m), A.device)
     rc = L.gbla_chol_gmresir_solve_nrhs(n, k, _p(Ac), _ld(Ac), _p(Fc), _ld(Fc), _p(Bc), _ld(Bc), _p(X),
                                         _ld(X), ctypes.byref(opts), st, _p(ws), ws.numel(), _stream())
     if rc not in (0, _lib.GBLA_ERR_NOT_CONVERGED):

@@ -960,13 +960,14 @@ struct IrWork {
   int* perm;
   double* V;
   int ldv;
+  size_t vstride;  // from one column's basis to the next one's
   double* w;
   double* r;
   double* H;
   double* cs;
   double* sn;
   double* g;
-  double* st;  // GmresState {res, pad}
+  double* st;  // GmresState {res, pad} of every column, then info
   double* slots;
   unsigned* counter;
   char* flags;  // scratch of the triangular solves
@@ -982,33 +983,40 @@ struct IrWork {
   double* d;   // the correction being built by the restart cycles
 };
 
-static size_t ir_layout(Carver& c, int n, int m, IrWork* w) {
+// Right-hand sides refined together: they share every launch of an iteration
+// (products with A and with the preconditioner, the Gram-Schmidt step), most of
+// whose time is the chain of the substitutions and barriers, not their work.
+constexpr int kIrCols = 4;
+
+static size_t ir_layout(Carver& c, int n, int m, IrWork* w, int cols = 1) {
   const int nn = std::max(n, 1);
   const int ldv = ((nn + 31) / 32) * 32;
+  const size_t k = (size_t)cols, vec = k * (size_t)nn;
   IrWork t;
   t.perm = c.take<int>(nn);
   t.ldv = ldv;
-  t.V = c.take<double>((size_t)ldv * (m + 1));
-  t.w = c.take<double>(nn);
-  t.r = c.take<double>(nn);
-  t.H = c.take<double>((size_t)(m + 1) * m);
-  t.cs = c.take<double>(m);
-  t.sn = c.take<double>(m);
-  t.g = c.take<double>(m + 1);
-  t.st = c.take<double>(2);
-  t.slots = c.take<double>(mgs_slots_doubles());
-  t.counter = c.take<unsigned>(1);
-  t.flags = c.take<char>(trsv_scratch_bytes(nn, 1));
-  t.t1 = c.take<double>(nn);
-  t.t2 = c.take<double>(nn);
+  t.vstride = (size_t)ldv * (m + 1);
+  t.V = c.take<double>(k * t.vstride);
+  t.w = c.take<double>(vec);
+  t.r = c.take<double>(vec);
+  t.H = c.take<double>(k * (m + 1) * m);
+  t.cs = c.take<double>(k * m);
+  t.sn = c.take<double>(k * m);
+  t.g = c.take<double>(k * (m + 1));
+  t.st = c.take<double>(2 * k + 1);
+  t.info = reinterpret_cast<int*>(t.st + 2 * k);
+  t.slots = c.take<double>(k * mgs_slots_doubles());
+  t.counter = c.take<unsigned>(k);
+  t.flags = c.take<char>(trsv_scratch_bytes(nn, cols));
+  t.t1 = c.take<double>(vec);
+  t.t2 = c.take<double>(vec);
   t.DinvL = c.take<double>(diag_inv_doubles(nn));
   t.DinvU = c.take<double>(diag_inv_doubles(nn));
-  t.info = c.take<int>(1);
   t.anorm = c.take<double>(1);
-  t.beta = c.take<double>(1);
-  t.part = c.take<double>(residual_work_doubles(nn, 1));
-  t.z = c.take<double>(nn);
-  t.d = c.take<double>(nn);
+  t.beta = c.take<double>(k);
+  t.part = c.take<double>(residual_work_doubles(nn, cols));
+  t.z = c.take<double>(vec);
+  t.d = c.take<double>(vec);
   if (w) *w = t;
   return c.off;
 }
@@ -1019,18 +1027,26 @@ size_t gbla_gmresir_workspace(int n, int restart_m) {
   return ir_layout(c, n, restart_m, nullptr);
 }
 
+size_t gbla_gmresir_workspace_nrhs(int n, int nrhs, int restart_m) {
+  if (n < 0 || nrhs < 0 || restart_m < 1 || restart_m > 128) return 0;
+  Carver c(nullptr, 0);
+  return ir_layout(c, n, restart_m, nullptr, std::min(std::max(nrhs, 1), kIrCols));
+}
+
 // dst <- M^{-1} src with M = P^t L U (FP32 factors, FP64 arithmetic, inverted
-// 64 x 64 diagonal blocks of L and U formed once per solve call); t1, t2:
-// n-double temporaries; src and dst distinct
+// 64 x 64 diagonal blocks of L and U formed once per solve call), k columns of a
+// call that refines up to `cols` together; t1, t2: n x k temporaries; src and dst
+// distinct
 static cudaError_t apply_minv(int n, const float* F, int ldf, const int* perm, const double* DinvL,
                               const double* DinvU, const double* src, double* dst, double* t1,
-                              double* t2, void* flags, int* info, cudaStream_t s) {
+                              double* t2, void* flags, int* info, cudaStream_t s, int k = 1, int cols = 1,
+                              int lds = 0, int ldd = 0) {
   cudaError_t e;
-  PROF(KK_PERM, s, launch_permute_rows(n, 1, perm, false, src, n, t1, n, s));
+  PROF(KK_PERM, s, launch_permute_rows(n, k, perm, false, src, lds ? lds : n, t1, n, s));
   if (e != cudaSuccess) return e;
-  PROF(KK_TRSV, s, launch_trsv_inv(true, n, F, ldf, DinvL, t1, t2, flags, info, s));
+  PROF(KK_TRSV, s, launch_trsv_inv(true, n, k, cols, F, ldf, DinvL, t1, n, t2, n, flags, info, s));
   if (e != cudaSuccess) return e;
-  PROF(KK_TRSV, s, launch_trsv_inv(false, n, F, ldf, DinvU, t2, dst, flags, info, s));
+  PROF(KK_TRSV, s, launch_trsv_inv(false, n, k, cols, F, ldf, DinvU, t2, n, dst, ldd ? ldd : n, flags, info, s));
   return e;
 }
 
@@ -1044,6 +1060,18 @@ static int read_scalar(double* host, const double* dev, const int* d_info, cudaS
   return info == GBLA_INFO_TIMEOUT ? GBLA_ERR_TIMEOUT : GBLA_OK;
 }
 
+// the residual norm of every column, and info, in one copy
+static int read_residuals(double* res, const IrWork& w, int cols, cudaStream_t s) {
+  double h[2 * kIrCols + 1];
+  if (cudaMemcpyAsync(h, w.st, sizeof(double) * (2 * cols + 1), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    return GBLA_ERR_CUDA;
+  if (cudaStreamSynchronize(s) != cudaSuccess) return GBLA_ERR_CUDA;
+  for (int c = 0; c < cols; ++c) res[c] = h[2 * c];
+  int info;
+  memcpy(&info, &h[2 * cols], sizeof(int));
+  return info == GBLA_INFO_TIMEOUT ? GBLA_ERR_TIMEOUT : GBLA_OK;
+}
+
 static int check_ir_opts(const gbla_gmresir_opts* o) {
   return (o && o->restart_m >= 1 && o->restart_m <= 128 && o->max_outer >= 0 && o->restarts >= 0 &&
           o->tol >= 0.0 && o->inner_tol >= 0.0)
@@ -1051,73 +1079,139 @@ static int check_ir_opts(const gbla_gmresir_opts* o) {
              : 1;
 }
 
-// One right-hand side, with the per-call set-up (perm, inverted diagonal
-// blocks, ||A||) already in w. Refinement step: r = b - A x and its backward
-// error; z = M^{-1} r; then up to `restarts` GMRES(m) cycles on
-// M^{-1} A d = z (cycle c > 0 restarts from the current d with the residual
+// Up to kIrCols right-hand sides, with the per-call set-up (perm, inverted
+// diagonal blocks, ||A||) already in w. For each of them, refinement step: r = b -
+// A x and its backward error; z = M^{-1} r; then up to `restarts` GMRES(m) cycles
+// on M^{-1} A d = z (cycle c > 0 restarts from the current d with the residual
 // z - M^{-1} A d), stopping once the least-squares residual is below
 // inner_tol * ||z||_2; x <- x + d.
-static int gmresir_one(int n, const double* A, int lda, const float* F, int ldf, const double* b,
-                       double* x, const gbla_gmresir_opts* opts, gbla_gmresir_stats* stats,
-                       const IrWork& w, cudaStream_t s) {
+// The columns advance together, each with its own basis, Hessenberg matrix and
+// stopping tests; a launch covers the columns from the first to the last one that
+// still needs it, and what it computes for one in between that does not (a next
+// basis vector, the column of H after its last) is not used.
+static int gmresir_group(int n, int cols, const double* A, int lda, const float* F, int ldf, const double* B, int ldb,
+                         double* X, int ldx, const gbla_gmresir_opts* opts, gbla_gmresir_stats* stats,
+                         const IrWork& w, cudaStream_t s) {
   const int m = opts->restart_m;
   const int cycles = std::max(1, opts->restarts);
-  memset(stats, 0, sizeof(*stats));
-  GBLA_TRY(apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, b, x, w.t1, w.t2, w.flags, w.info, s));
+  const size_t hs = (size_t)(m + 1) * m;
+  struct Range {
+    int lo, k;  // first column, number of columns
+  };
+  auto range = [&](const bool* on) {
+    int lo = 0, hi = cols;
+    while (lo < hi && !on[lo]) ++lo;
+    while (hi > lo && !on[hi - 1]) --hi;
+    return Range{lo, hi - lo};
+  };
+  auto col = [&](double* base, int c) { return base + (size_t)c * n; };
+  // dst <- M^{-1} src, columns of scratch
+  auto minv = [&](Range r, double* src, double* dst) {
+    return apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, col(src, r.lo), col(dst, r.lo), w.t1, w.t2, w.flags, w.info, s,
+                      r.k, cols);
+  };
+  auto mgs = [&](Range r, int j, double* v) {
+    const int c = r.lo;
+    return launch_mgs_step(n, j, w.V + c * w.vstride, w.ldv, col(v, c), w.H + c * hs, m + 1, w.cs + (size_t)c * m,
+                           w.sn + (size_t)c * m, w.g + (size_t)c * (m + 1), w.st + 2 * c,
+                           w.slots + c * mgs_slots_doubles(), w.counter + c, w.info, s, r.k, w.vstride, n, hs);
+  };
+  for (int c = 0; c < cols; ++c) memset(&stats[c], 0, sizeof(stats[c]));
+  GBLA_TRY(apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, B, X, w.t1, w.t2, w.flags, w.info, s, cols, cols, ldb, ldx));
+  bool live[kIrCols], cyc_on[kIrCols], it_on[kIrCols];
+  double beta[kIrCols], res[kIrCols], znorm[kIrCols] = {};
+  int k[kIrCols];
+  for (int c = 0; c < cols; ++c) live[c] = true;
   int rc = GBLA_OK;
   for (int outer = 0;; ++outer) {
-    GBLA_TRYK(KK_MATVEC, s, launch_residual(n, 1, A, lda, x, n, b, n, w.r, n, w.part, s));
-    GBLA_TRYK(KK_MATVEC, s, launch_backward_error_finish(n, 1, w.r, n, x, n, w.anorm, w.beta, s));
-    double beta = 0.0;
-    rc = read_scalar(&beta, w.beta, w.info, s);
+    Range r = range(live);
+    GBLA_TRYK(KK_MATVEC, s, launch_residual(n, r.k, A, lda, X + (size_t)r.lo * ldx, ldx, B + (size_t)r.lo * ldb, ldb,
+                                            col(w.r, r.lo), n, w.part, s));
+    GBLA_TRYK(KK_MATVEC, s, launch_backward_error_finish(n, r.k, col(w.r, r.lo), n, X + (size_t)r.lo * ldx, ldx, w.anorm,
+                                                         w.beta + r.lo, s));
+    GBLA_TRY(cudaMemcpyAsync(beta, w.beta, sizeof(double) * cols, cudaMemcpyDeviceToHost, s));
+    rc = read_residuals(res, w, cols, s);
     if (rc != GBLA_OK) return rc;
-    if (outer == 0) stats->beta0 = beta;
-    stats->beta = beta;
-    stats->outer = outer;
-    if (beta <= opts->tol) {
-      stats->converged = 1;
-      return GBLA_OK;
+    bool any = false;
+    for (int c = 0; c < cols; ++c) {
+      if (!live[c]) continue;
+      if (outer == 0) stats[c].beta0 = beta[c];
+      stats[c].beta = beta[c];
+      stats[c].outer = outer;
+      if (beta[c] <= opts->tol) {
+        stats[c].converged = 1;
+        live[c] = false;
+      } else {
+        any = true;
+      }
     }
+    if (!any) break;
     if (outer >= opts->max_outer) return GBLA_ERR_NOT_CONVERGED;
     // z = M^{-1} r; d = 0
-    GBLA_TRY(apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, w.r, w.z, w.t1, w.t2, w.flags, w.info, s));
-    GBLA_TRY(cudaMemsetAsync(w.d, 0, sizeof(double) * (size_t)n, s));
-    double znorm = 0.0;
+    r = range(live);
+    GBLA_TRY(minv(r, w.r, w.z));
+    GBLA_TRY(cudaMemsetAsync(col(w.d, r.lo), 0, sizeof(double) * (size_t)n * r.k, s));
+    for (int c = 0; c < cols; ++c) cyc_on[c] = live[c];
     for (int cyc = 0; cyc < cycles; ++cyc) {
       // v_0 = c / ||c|| with c = z (first cycle) or z - M^{-1} A d
-      const double* c0 = w.z;
+      r = range(cyc_on);
+      double* c0 = w.z;
       if (cyc > 0) {
-        GBLA_TRYK(KK_MATVEC, s, launch_residual(n, 1, A, lda, w.d, n, nullptr, n, w.w, n, w.part, s));
-        GBLA_TRY(apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, w.w, w.r, w.t1, w.t2, w.flags, w.info, s));
-        GBLA_TRYK(KK_UPDATE, s, launch_axpby(n, 1.0, w.z, -1.0, w.r, w.w, s));
+        GBLA_TRYK(KK_MATVEC, s, launch_residual(n, r.k, A, lda, col(w.d, r.lo), n, nullptr, n, col(w.w, r.lo), n, w.part, s));
+        GBLA_TRY(minv(r, w.w, w.r));
+        // the columns lie one after the other: one vector of r.k n elements
+        GBLA_TRYK(KK_UPDATE, s, launch_axpby((size_t)n * r.k, 1.0, col(w.z, r.lo), -1.0, col(w.r, r.lo), col(w.w, r.lo), s));
         c0 = w.w;
       }
-      GBLA_TRYK(KK_MGS, s, launch_mgs_step(n, -1, w.V, w.ldv, c0, w.H, m + 1, w.cs, w.sn, w.g, w.st, w.slots,
-                               w.counter, w.info, s));
-      double beta_in = 0.0;
-      rc = read_scalar(&beta_in, w.st, w.info, s);
+      GBLA_TRYK(KK_MGS, s, mgs(r, -1, c0));
+      rc = read_residuals(res, w, cols, s);
       if (rc != GBLA_OK) return rc;
-      if (cyc == 0) znorm = beta_in;
-      if (!(beta_in > opts->inner_tol * znorm) || !(beta_in > 0.0)) break;
-      int k = 0;
-      double res = beta_in;
-      for (int j = 0; j < m; ++j) {
-        // w = M^{-1} A v_j
-        GBLA_TRYK(KK_MATVEC, s, launch_residual(n, 1, A, lda, w.V + (size_t)j * w.ldv, n, nullptr, n, w.w, n, w.part, s));
-        GBLA_TRY(apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, w.w, w.r, w.t1, w.t2, w.flags, w.info, s));
-        GBLA_TRYK(KK_MGS, s, launch_mgs_step(n, j, w.V, w.ldv, w.r, w.H, m + 1, w.cs, w.sn, w.g, w.st, w.slots,
-                                 w.counter, w.info, s));
-        rc = read_scalar(&res, w.st, w.info, s);
-        if (rc != GBLA_OK) return rc;
-        k = j + 1;
-        if (res <= opts->inner_tol * znorm) break;
+      any = false;
+      for (int c = 0; c < cols; ++c) {
+        it_on[c] = false;
+        if (!cyc_on[c]) continue;
+        k[c] = 0;
+        if (cyc == 0) znorm[c] = res[c];
+        if (!(res[c] > opts->inner_tol * znorm[c]) || !(res[c] > 0.0)) cyc_on[c] = false;
+        it_on[c] = cyc_on[c];
+        any = any || cyc_on[c];
       }
-      stats->inner += k;
-      GBLA_TRYK(KK_UPDATE, s, launch_gmres_update(n, k, w.V, w.ldv, w.H, m + 1, w.g, w.d, s));
-      if (res <= opts->inner_tol * znorm) break;
+      if (!any) break;
+      double last[kIrCols];
+      for (int j = 0; j < m && any; ++j) {
+        // w = M^{-1} A v_j
+        r = range(it_on);
+        GBLA_TRYK(KK_MATVEC, s, launch_residual(n, r.k, A, lda, w.V + r.lo * w.vstride + (size_t)j * w.ldv, (int)w.vstride,
+                                                nullptr, n, col(w.w, r.lo), n, w.part, s));
+        GBLA_TRY(minv(r, w.w, w.r));
+        GBLA_TRYK(KK_MGS, s, mgs(r, j, w.r));
+        rc = read_residuals(res, w, cols, s);
+        if (rc != GBLA_OK) return rc;
+        any = false;
+        for (int c = 0; c < cols; ++c) {
+          if (!it_on[c]) continue;
+          last[c] = res[c];
+          k[c] = j + 1;
+          it_on[c] = !(res[c] <= opts->inner_tol * znorm[c]);
+          any = any || it_on[c];
+        }
+      }
+      any = false;
+      for (int c = 0; c < cols; ++c) {
+        if (!cyc_on[c]) continue;
+        stats[c].inner += k[c];
+        GBLA_TRYK(KK_UPDATE, s, launch_gmres_update(n, k[c], w.V + c * w.vstride, w.ldv, w.H + c * hs, m + 1,
+                                                    w.g + (size_t)c * (m + 1), col(w.d, c), s));
+        cyc_on[c] = !(last[c] <= opts->inner_tol * znorm[c]);
+        any = any || cyc_on[c];
+      }
+      if (!any) break;
     }
-    GBLA_TRYK(KK_UPDATE, s, launch_axpby(n, 1.0, w.d, 1.0, x, x, s));
+    for (int c = 0; c < cols; ++c)
+      if (live[c])
+        GBLA_TRYK(KK_UPDATE, s, launch_axpby((size_t)n, 1.0, col(w.d, c), 1.0, X + (size_t)c * ldx, X + (size_t)c * ldx, s));
   }
+  return GBLA_OK;
 }
 
 // Per-call set-up of the refinement: the permutation of the pivots, the
@@ -1152,10 +1246,15 @@ static int gmresir_nrhs(int n, int nrhs, const double* A, int lda, const float* 
   if (nrhs > 0 && !stats) return -13;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (!d_work || !aligned256(d_work)) return GBLA_ERR_WORKSPACE;
-  Carver c(d_work, work_bytes);
+  // as many columns together as the workspace has room for
   IrWork w;
-  ir_layout(c, n, opts->restart_m, &w);
-  if (!c.ok) return GBLA_ERR_WORKSPACE;
+  int cols = std::min(std::max(nrhs, 1), kIrCols);
+  for (;; --cols) {
+    Carver t(d_work, work_bytes);
+    ir_layout(t, n, opts->restart_m, &w, cols);
+    if (t.ok) break;
+    if (cols == 1) return GBLA_ERR_WORKSPACE;
+  }
   for (int k = 0; k < nrhs; ++k) memset(&stats[k], 0, sizeof(stats[k]));
   if (n == 0) {
     for (int k = 0; k < nrhs; ++k) stats[k].converged = 1;
@@ -1167,8 +1266,9 @@ static int gmresir_nrhs(int n, int nrhs, const double* A, int lda, const float* 
   int rc = gmresir_setup(n, A, lda, F, ldf, chol ? nullptr : ipiv, w, s);
   if (rc != GBLA_OK) return rc;
   int all = GBLA_OK;
-  for (int k = 0; k < nrhs; ++k) {
-    rc = gmresir_one(n, A, lda, F, ldf, B + (size_t)k * ldb, X + (size_t)k * ldx, opts, &stats[k], w, s);
+  for (int k = 0; k < nrhs; k += cols) {
+    const int kc = std::min(cols, nrhs - k);
+    rc = gmresir_group(n, kc, A, lda, F, ldf, B + (size_t)k * ldb, ldb, X + (size_t)k * ldx, ldx, opts, &stats[k], w, s);
     if (rc == GBLA_ERR_NOT_CONVERGED) all = rc;
     else if (rc != GBLA_OK) return rc;
   }

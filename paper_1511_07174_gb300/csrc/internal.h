@@ -192,10 +192,11 @@ size_t trsv_scratch_bytes(int n, int nrhs);
 // blocks of a triangular factor, formed once per set of factors ...
 size_t diag_inv_doubles(int n);
 cudaError_t launch_diag_inv(bool lower, bool unit, int n, const float* T, int ldt, double* D, cudaStream_t s);
-// ... and X <- T^{-1} rhs with them (X and rhs distinct; scratch:
-// trsv_scratch_bytes(n, 1)).
-cudaError_t launch_trsv_inv(bool lower, int n, const float* T, int ldt, const double* D, const double* rhs, double* X,
-                            void* scratch, int* info, cudaStream_t s);
+// ... and X <- T^{-1} rhs with them, nrhs columns (X and rhs distinct; scratch:
+// trsv_scratch_bytes(n, cols)). A call with cols > 1 takes the same operations
+// in the same order for any nrhs <= cols.
+cudaError_t launch_trsv_inv(bool lower, int n, int nrhs, int cols, const float* T, int ldt, const double* D,
+                            const double* rhs, int ldr, double* X, int ldx, void* scratch, int* info, cudaStream_t s);
 
 // ipiv == nullptr: the identity
 cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, cudaStream_t s);
@@ -221,9 +222,10 @@ cudaError_t launch_backward_error_finish(int n, int nrhs, const double* R, int l
 size_t mgs_slots_doubles();
 cudaError_t launch_mgs_step(int n, int j, double* V, int ldv, const double* w, double* H, int ldh,
                             double* cs, double* sn, double* g, void* st, double* slots,
-                            unsigned* counter, int* info, cudaStream_t s);
+                            unsigned* counter, int* info, cudaStream_t s,
+                            int cols = 1, size_t vstride = 0, size_t wstride = 0, size_t hstride = 0);
 // out = a x + b y (FP64 vectors; out may alias x or y)
-cudaError_t launch_axpby(int n, double a, const double* x, double b, const double* y, double* out,
+cudaError_t launch_axpby(size_t n, double a, const double* x, double b, const double* y, double* out,
                          cudaStream_t s);
 cudaError_t launch_gmres_update(int n, int k, const double* V, int ldv, const double* H, int ldh,
                                 const double* g, double* x, cudaStream_t s);

@@ -9,10 +9,20 @@
 namespace gbla {
 
 constexpr int kResRows = 256;   // rows per CTA (one thread per row)
-constexpr int kResCols = 512;   // columns per CTA
+constexpr int kResCols = 512;   // columns per CTA, at most
+
+// Columns per CTA: the product is bound by HBM (8 bytes per multiply-add) and by
+// the FP64 pipe alike, so every SM should have the same share of it; 512 while that
+// makes four CTAs per SM, else less (measured, n = 2500: 36 -> 14 us).
+static int res_cols(int n) {
+  const int sms = device_props().num_sms > 0 ? device_props().num_sms : 152;
+  int cols = kResCols;
+  while (cols > 64 && (size_t)((n + kResRows - 1) / kResRows) * ((n + cols - 1) / cols) < (size_t)4 * sms) cols /= 2;
+  return cols;
+}
 
 size_t residual_work_doubles(int n, int nrhs) {
-  const size_t chunks = (size_t)((n + kResCols - 1) / kResCols);
+  const size_t chunks = (size_t)((n + res_cols(n) - 1) / res_cols(n));
   return chunks * (size_t)(n > 0 ? n : 1) * (size_t)(nrhs > 0 ? nrhs : 1);
 }
 
@@ -22,16 +32,16 @@ size_t residual_work_doubles(int n, int nrhs) {
 // two independent FMA chains in flight.
 template <bool ABS, int NR>
 __global__ void __launch_bounds__(kResRows)
-    matvec_partial_kernel(int n, const double* __restrict__ A, int lda,
+    matvec_partial_kernel(int n, int cols, const double* __restrict__ A, int lda,
                           const double* __restrict__ X, int ldx, double* __restrict__ part) {
   __shared__ double xs[kResCols][NR];
   const int i = blockIdx.x * kResRows + threadIdx.x;
   const int chunk = blockIdx.y;
-  const int j0 = chunk * kResCols;
-  const int nc = min(kResCols, n - j0);
+  const int j0 = chunk * cols;
+  const int nc = min(cols, n - j0);
   if (!ABS) {
-    for (int idx = threadIdx.x; idx < kResCols * NR; idx += blockDim.x) {
-      const int jj = idx % kResCols, c = idx / kResCols;
+    for (int idx = threadIdx.x; idx < cols * NR; idx += blockDim.x) {
+      const int jj = idx % cols, c = idx / cols;
       xs[jj][c] = jj < nc ? X[(j0 + jj) + (size_t)c * ldx] : 0.0;
     }
     __syncthreads();
@@ -86,21 +96,21 @@ cudaError_t launch_residual(int n, int nrhs, const double* A, int lda, const dou
                             const double* B, int ldb, double* R, int ldr, double* work,
                             cudaStream_t s) {
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
-  const int chunks = (n + kResCols - 1) / kResCols;
+  const int cols = res_cols(n), chunks = (n + cols - 1) / cols;
   for (int c0 = 0; c0 < nrhs;) {
     const int left = nrhs - c0;
     const int nc = left >= 8 ? 8 : (left >= 4 ? 4 : (left >= 2 ? 2 : 1));
     dim3 grid((n + kResRows - 1) / kResRows, chunks);
     const double* Xc = X + (size_t)c0 * ldx;
     switch (nc) {
-      case 8: matvec_partial_kernel<false, 8><<<grid, kResRows, 0, s>>>(n, A, lda, Xc, ldx, work); break;
-      case 4: matvec_partial_kernel<false, 4><<<grid, kResRows, 0, s>>>(n, A, lda, Xc, ldx, work); break;
-      case 2: matvec_partial_kernel<false, 2><<<grid, kResRows, 0, s>>>(n, A, lda, Xc, ldx, work); break;
-      default: matvec_partial_kernel<false, 1><<<grid, kResRows, 0, s>>>(n, A, lda, Xc, ldx, work); break;
+      case 8: matvec_partial_kernel<false, 8><<<grid, kResRows, 0, s>>>(n, cols, A, lda, Xc, ldx, work); break;
+      case 4: matvec_partial_kernel<false, 4><<<grid, kResRows, 0, s>>>(n, cols, A, lda, Xc, ldx, work); break;
+      case 2: matvec_partial_kernel<false, 2><<<grid, kResRows, 0, s>>>(n, cols, A, lda, Xc, ldx, work); break;
+      default: matvec_partial_kernel<false, 1><<<grid, kResRows, 0, s>>>(n, cols, A, lda, Xc, ldx, work); break;
     }
-    int bx = (n + 255) / 256;
-    if (bx > 512) bx = 512;
-    residual_finish_kernel<<<dim3(bx, nc), 256, 0, s>>>(
+    int bx = (n + 63) / 64;
+    if (bx > 2048) bx = 2048;
+    residual_finish_kernel<<<dim3(bx, nc), 64, 0, s>>>(
         n, nc, chunks, work, B ? B + (size_t)c0 * ldb : nullptr, ldb, R + (size_t)c0 * ldr, ldr);
     count_launch(2);
     cudaError_t e = cudaGetLastError();
@@ -132,9 +142,9 @@ __global__ void __launch_bounds__(1024)
 cudaError_t launch_row_abs_sum_max(int n, const double* A, int lda, double* work, double* anorm,
                                    cudaStream_t s) {
   if (n <= 0) return cudaMemsetAsync(anorm, 0, sizeof(double), s);
-  const int chunks = (n + kResCols - 1) / kResCols;
+  const int cols = res_cols(n), chunks = (n + cols - 1) / cols;
   dim3 grid((n + kResRows - 1) / kResRows, chunks);
-  matvec_partial_kernel<true, 1><<<grid, kResRows, 0, s>>>(n, A, lda, nullptr, 0, work);
+  matvec_partial_kernel<true, 1><<<grid, kResRows, 0, s>>>(n, cols, A, lda, nullptr, 0, work);
   rowsum_max_kernel<<<1, 1024, 0, s>>>(n, chunks, work, anorm);
   count_launch(2);
   return cudaGetLastError();
@@ -211,7 +221,21 @@ __global__ void __launch_bounds__(kMgsThreads)
     mgs_step_kernel(int n, int j, int ldv, double* __restrict__ V, const double* __restrict__ w_in,
                     double* __restrict__ H, int ldh, double* __restrict__ cs, double* __restrict__ sn,
                     double* __restrict__ g, GmresState* st, double* __restrict__ slots,
-                    unsigned* __restrict__ counter, int* info, uint64_t wait_ns) {
+                    unsigned* __restrict__ counter, int* info, uint64_t wait_ns, size_t vstride, size_t wstride,
+                    size_t hstride, size_t sstride) {
+  {  // the column of this row of the grid: its own data, slots and barrier
+    const size_t q = blockIdx.y;
+    const int m = ldh - 1;
+    V += q * vstride;
+    w_in += q * wstride;
+    H += q * hstride;
+    cs += q * m;
+    sn += q * m;
+    g += q * ldh;
+    st += q;
+    slots += q * sstride;
+    counter += q;
+  }
   extern __shared__ double wsl[];  // this CTA's slice of w
   __shared__ double red[kMgsThreads / 32];
   __shared__ double s_h;
@@ -295,7 +319,8 @@ __global__ void __launch_bounds__(kMgsThreads)
 
 cudaError_t launch_mgs_step(int n, int j, double* V, int ldv, const double* w, double* H, int ldh,
                             double* cs, double* sn, double* g, void* st, double* slots,
-                            unsigned* counter, int* info, cudaStream_t s) {
+                            unsigned* counter, int* info, cudaStream_t s, int cols, size_t vstride, size_t wstride,
+                            size_t hstride) {
   const DeviceProps& dp = device_props();
   int C = (n + 255) / 256;
   if (C > dp.num_sms) C = dp.num_sms;
@@ -305,13 +330,16 @@ cudaError_t launch_mgs_step(int n, int j, double* V, int ldv, const double* w, d
   if (smem > dp.smem_optin) return cudaErrorInvalidValue;
   cudaError_t ea = ensure_dyn_smem(mgs_step_kernel, smem);
   if (ea != cudaSuccess) return ea;
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
+  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned) * cols, s);
   if (e != cudaSuccess) return e;
   GmresState* stp = static_cast<GmresState*>(st);
   uint64_t wait_ns = wait_timeout_ns();
-  void* args[] = {&n, &j, &ldv, &V, &w, &H, &ldh, &cs, &sn, &g, &stp, &slots, &counter, &info, &wait_ns};
+  size_t sstride = mgs_slots_doubles();
+  void* args[] = {&n, &j, &ldv, &V, &w, &H, &ldh, &cs, &sn, &g, &stp, &slots, &counter, &info, &wait_ns,
+                  &vstride, &wstride, &hstride, &sstride};
+  // every CTA of every column is resident (a cooperative launch)
   count_launch();
-  return cudaLaunchCooperativeKernel((const void*)mgs_step_kernel, dim3(C), dim3(kMgsThreads), args,
+  return cudaLaunchCooperativeKernel((const void*)mgs_step_kernel, dim3(C, cols), dim3(kMgsThreads), args,
                                      smem, s);
 }
 
@@ -344,17 +372,16 @@ __global__ void __launch_bounds__(256)
 }
 
 // out = a x + b y (FP64 vectors; out may alias x or y).
-__global__ void axpby_kernel(int n, double a, const double* x, double b, const double* y,
+__global__ void axpby_kernel(size_t n, double a, const double* x, double b, const double* y,
                              double* out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     out[i] = fma(a, x[i], b * y[i]);
 }
 
-cudaError_t launch_axpby(int n, double a, const double* x, double b, const double* y, double* out,
+cudaError_t launch_axpby(size_t n, double a, const double* x, double b, const double* y, double* out,
                          cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  int bx = (n + 255) / 256;
-  if (bx > 1024) bx = 1024;
+  if (n == 0) return cudaSuccess;
+  const int bx = (int)((n + 255) / 256 > 1024 ? 1024 : (n + 255) / 256);
   axpby_kernel<<<bx, 256, 0, s>>>(n, a, x, b, y, out);
   count_launch();
   return cudaGetLastError();

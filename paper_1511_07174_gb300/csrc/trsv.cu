@@ -963,8 +963,8 @@ static cudaError_t tc_launch_diag_inv(bool fwd, bool unit, int n, const Ts* T, i
 // that says whether the inverses are safe is left as it is.
 template <typename Ts, bool TRANS>
 static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, const Ts* T, int ldt, const double* D, const double* rhs,
-                            int ldr, double* X, int ldx, char* scratch, size_t ctrl_words, bool gated, int* info,
-                            cudaStream_t s) {
+                            int ldr, double* X, int ldx, char* scratch, size_t ctrl_words, bool gated, bool wide,
+                            int* info, cudaStream_t s) {
   TcArgs a;
   a.n = n;
   a.nblk = (n + kTsBS - 1) / kTsBS;
@@ -984,7 +984,7 @@ static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, c
   a.gated = gated;
   a.info = info;
   a.wait_ns = wait_timeout_ns();
-  if (ncols == 1) return tc_launch_solve<Ts, TRANS, 1, 8>(T, a, s);
+  if (ncols == 1 && !wide) return tc_launch_solve<Ts, TRANS, 1, 8>(T, a, s);
   if (sh.G == 1) return tc_launch_solve<Ts, TRANS, 1, 4>(T, a, s);
   if (sh.G == 2) return tc_launch_solve<Ts, TRANS, 2, 4>(T, a, s);
   return tc_launch_solve<Ts, TRANS, 4, 4>(T, a, s);
@@ -1033,8 +1033,8 @@ cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, cons
                   : tc_launch_diag_inv<double, false>(fwd, unit, n, T, ldt, D, ctrl + kTcMaxC, s);
         if (e != cudaSuccess) return e;
       }
-      e = trans ? tc_apply<double, true>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s)
-                : tc_apply<double, false>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s);
+      e = trans ? tc_apply<double, true>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, nrhs > 1, info, s)
+                : tc_apply<double, false>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, nrhs > 1, info, s);
       if (e != cudaSuccess) return e;
     }
     const int C = trsv_chains(ncols);
@@ -1068,16 +1068,18 @@ cudaError_t launch_diag_inv(bool lower, bool unit, int n, const float* T, int ld
   return tc_launch_diag_inv<float, false>(lower, unit, n, T, ldt, D, nullptr, s);
 }
 
-// ... and X = T^-1 rhs (one right-hand side, distinct buffers) as a fixed linear map
-cudaError_t launch_trsv_inv(bool lower, int n, const float* T, int ldt, const double* D, const double* rhs, double* X,
-                            void* scratch, int* info, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const size_t cw = tc_ctrl_words(n, 1);
-  const TcShape sh = tc_shape(1);
+// ... and X = T^-1 rhs (at most kTcMaxC columns, distinct buffers) as a fixed
+// linear map
+cudaError_t launch_trsv_inv(bool lower, int n, int nrhs, int cols, const float* T, int ldt, const double* D,
+                            const double* rhs, int ldr, double* X, int ldx, void* scratch, int* info, cudaStream_t s) {
+  if (n <= 0 || nrhs <= 0) return cudaSuccess;
+  if (nrhs > cols || cols > kTcMaxC) return cudaErrorInvalidValue;
+  const size_t cw = tc_ctrl_words(n, cols);
+  const TcShape sh = tc_shape(nrhs);
   char* sc = static_cast<char*>(scratch);
-  cudaError_t e = tc_fill(n, 1, sh, X, n, sc, cw, false, s);
+  cudaError_t e = tc_fill(n, nrhs, sh, X, ldx, sc, cw, false, s);
   if (e != cudaSuccess) return e;
-  return tc_apply<float, false>(lower, false, n, 1, sh, T, ldt, D, rhs, n, X, n, sc, cw, false, info, s);
+  return tc_apply<float, false>(lower, false, n, nrhs, sh, T, ldt, D, rhs, ldr, X, ldx, sc, cw, false, cols > 1, info, s);
 }
 
 }  // namespace gbla
