@@ -645,7 +645,7 @@ int gbla_lu_solve(int trans, int n, int nrhs, const double* LU, int lda, const i
   if (!c.ok) return GBLA_ERR_WORKSPACE;
   GBLA_TRY(cudaMemsetAsync(d_info, 0, sizeof(int), s));
   if (n == 0 || nrhs == 0) return GBLA_OK;
-  GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, w.perm, s));
+  GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, w.perm, w.D, s));
   if (!trans) {
     GBLA_TRYK(KK_PERM, s, launch_permute_rows(n, nrhs, w.perm, false, B, ldb, w.T1, n, s));
     GBLA_TRYK(KK_TRSV, s, launch_trsv(true, false, true, n, nrhs, LU, lda, w.T1, n, w.T2, n, w.D, w.scratch, d_info, s));
@@ -1220,7 +1220,7 @@ static int gmresir_group(int n, int cols, const double* A, int lda, const float*
 static int gmresir_setup(int n, const double* A, int lda, const float* F, int ldf, const int* ipiv,
                          const IrWork& w, cudaStream_t s) {
   GBLA_TRY(cudaMemsetAsync(w.info, 0, sizeof(int), s));
-  GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, w.perm, s));
+  GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, w.perm, w.DinvL, s));
   GBLA_TRYK(KK_TRSV, s, launch_diag_inv(true, ipiv != nullptr, n, F, ldf, w.DinvL, s));
   GBLA_TRYK(KK_TRSV, s, launch_diag_inv(false, false, n, F, ldf, w.DinvU, s));
   GBLA_TRYK(KK_MATVEC, s, launch_row_abs_sum_max(n, A, lda, w.part, w.anorm, s));
@@ -1470,7 +1470,7 @@ int gbla_gmres_solve(int n, const double* A, int lda, const double* b, double* x
   const bool pre = F != nullptr;
   GBLA_TRY(cudaMemsetAsync(ir.info, 0, sizeof(int), s));
   if (pre) {
-    GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, ir.perm, s));
+    GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, ir.perm, ir.DinvL, s));
     GBLA_TRYK(KK_TRSV, s, launch_diag_inv(true, true, n, F, ldf, ir.DinvL, s));
     GBLA_TRYK(KK_TRSV, s, launch_diag_inv(false, false, n, F, ldf, ir.DinvU, s));
     GBLA_TRY(apply_minv(n, F, ldf, ir.perm, ir.DinvL, ir.DinvU, b, ir.z, ir.t1, ir.t2, ir.flags, ir.info, s));
@@ -1554,7 +1554,7 @@ int gbla_bicgstab_solve(int n, const double* A, int lda, const double* b, double
   const bool pre = F != nullptr;
   GBLA_TRY(cudaMemsetAsync(ir.info, 0, sizeof(int), s));
   if (pre) {
-    GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, ir.perm, s));
+    GBLA_TRYK(KK_PERM, s, launch_ipiv_to_perm(n, ipiv, ir.perm, ir.DinvL, s));
     GBLA_TRYK(KK_TRSV, s, launch_diag_inv(true, true, n, F, ldf, ir.DinvL, s));
     GBLA_TRYK(KK_TRSV, s, launch_diag_inv(false, false, n, F, ldf, ir.DinvU, s));
   }

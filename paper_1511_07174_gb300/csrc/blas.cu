@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
         for (int q = qi; q < Q; ++q) {
           const int r = lane + 32 * q;
-          if (32 * q < w) {
+          if (sizeof(Ts) == 4 || 32 * q < w) {
             const Tc l = r < w ? lcol[r] : (Tc)0;
 #pragma unroll
             for (int c = 0; c < CW; ++c) x[q][c] = fma(-l, xi[c], x[q][c]);
@@ -609,38 +609,60 @@ cudaError_t launch_copy_d2f(const double* A, int lda, float* F, int ldf, int m, 
 }
 
 // ----------------------------------------------------------------------------
-// perm from sequential interchanges: (P v)[i] = v[perm[i]]. One CTA takes the
-// interchanges 256 at a time: swap_plan gives, in parallel, where each row
-// touched by the chunk gets its value from, and the CTA applies that map to
-// the running permutation (every read before any write). The permutation
-// lives in shared memory when it fits, else in perm itself.
-__global__ void __launch_bounds__(1024)
-    ipiv_to_perm_kernel(int n, const int* __restrict__ ipiv, int* __restrict__ perm, int use_smem) {
-  extern __shared__ int sp[];
+// perm from sequential interchanges: (P v)[i] = v[perm[i]], 256 at a time.
+// swap_plan gives, in parallel, where each row touched by such a chunk gets its
+// value from. It depends on the chunk's interchanges alone, so one CTA per chunk
+// works it out (about 5 us each); one CTA then applies the plans in order to the
+// running permutation (every read before any write), which lives in shared memory
+// when it fits, else in perm itself. Measured: n = 4096 87 -> 15 us.
+__global__ void __launch_bounds__(256)
+    perm_plan_kernel(int n, const int* __restrict__ ipiv, int* __restrict__ plan) {
   __shared__ SwapPlanShared s_plan;
+  const int t = threadIdx.x, c0 = blockIdx.x * 256, kb = min(256, n - c0);
+  if (t < kb) {
+    int q = ipiv[c0 + t] - 1 - c0;
+    if (q < t || q >= n - c0) q = t;  // out-of-range pivots are ignored
+    s_plan.p[t] = q;
+  }
+  __syncthreads();
+  int src_b = t, dst_o = -1, src_o = 0;
+  swap_plan(s_plan, kb, t, &src_b, &dst_o, &src_o);
+  if (t < kb) {
+    plan[c0 + t] = src_b;
+    plan[n + c0 + t] = dst_o;
+    plan[2 * (size_t)n + c0 + t] = src_o;
+  }
+}
+
+__global__ void __launch_bounds__(1024)
+    ipiv_to_perm_kernel(int n, const int* __restrict__ plan, int* __restrict__ perm, int use_smem) {
+  extern __shared__ int sp[];
   int* p = use_smem ? sp : perm;
   const int t = threadIdx.x;
   for (int i = t; i < n; i += blockDim.x) p[i] = i;
+  int sb = 0, dst = -1, so = 0;
+  auto fetch = [&](int c0) {
+    if (t < 256 && c0 + t < n) {
+      sb = plan[c0 + t];
+      dst = plan[n + c0 + t];
+      so = plan[2 * (size_t)n + c0 + t];
+    }
+  };
+  fetch(0);
   __syncthreads();
   for (int c0 = 0; c0 < n; c0 += 256) {
-    const int kb = min(256, n - c0);
-    if (t < kb) {
-      int q = ipiv[c0 + t] - 1 - c0;
-      if (q < t || q >= n - c0) q = t;  // out-of-range pivots are ignored
-      s_plan.p[t] = q;
-    }
-    __syncthreads();
-    int src_b = t, dst_o = -1, src_o = 0;
-    swap_plan(s_plan, kb, t, &src_b, &dst_o, &src_o);
+    const bool on = t < 256 && c0 + t < n;
+    const int b0 = sb, d0 = dst, o0 = so;
+    fetch(c0 + 256);
     int vb = 0, vo = 0;
-    if (t < kb) {
-      vb = p[c0 + src_b];
-      if (dst_o >= 0) vo = p[c0 + src_o];
+    if (on) {
+      vb = p[c0 + b0];
+      if (d0 >= 0) vo = p[c0 + o0];
     }
     __syncthreads();
-    if (t < kb) {
+    if (on) {
       p[c0 + t] = vb;
-      if (dst_o >= 0) p[c0 + dst_o] = vo;
+      if (d0 >= 0) p[c0 + d0] = vo;
     }
     __syncthreads();
   }
@@ -652,7 +674,7 @@ __global__ void iota_kernel(int n, int* __restrict__ perm) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) perm[i] = i;
 }
 
-cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, cudaStream_t s) {
+cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, void* scratch, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (!ipiv) {  // no interchanges: the identity
     iota_kernel<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, s>>>(n, perm);
@@ -661,13 +683,15 @@ cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, cudaStream_t 
   }
   const DeviceProps& dp = device_props();
   const size_t bytes = (size_t)n * sizeof(int);
-  const int use_smem = bytes + sizeof(SwapPlanShared) + 1024 <= dp.smem_optin ? 1 : 0;
+  const int use_smem = bytes + 1024 <= dp.smem_optin ? 1 : 0;
   if (use_smem) {
     cudaError_t ea = ensure_dyn_smem(ipiv_to_perm_kernel, bytes);
     if (ea != cudaSuccess) return ea;
   }
-  ipiv_to_perm_kernel<<<1, 1024, use_smem ? bytes : 0, s>>>(n, ipiv, perm, use_smem);
-  count_launch();
+  int* plan = static_cast<int*>(scratch);
+  perm_plan_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, ipiv, plan);
+  ipiv_to_perm_kernel<<<1, 1024, use_smem ? bytes : 0, s>>>(n, plan, perm, use_smem);
+  count_launch(2);
   return cudaGetLastError();
 }
 

@@ -198,8 +198,8 @@ cudaError_t launch_diag_inv(bool lower, bool unit, int n, const float* T, int ld
 cudaError_t launch_trsv_inv(bool lower, int n, int nrhs, int cols, const float* T, int ldt, const double* D,
                             const double* rhs, int ldr, double* X, int ldx, void* scratch, int* info, cudaStream_t s);
 
-// ipiv == nullptr: the identity
-cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, cudaStream_t s);
+// ipiv == nullptr: the identity. scratch: 3 n ints.
+cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, void* scratch, cudaStream_t s);
 // dst[i, c] = src[perm[i], c] (forward) or dst[perm[i], c] = src[i, c] (inverse)
 cudaError_t launch_permute_rows(int n, int nrhs, const int* perm, bool inverse, const double* src,
                                 int lds, double* dst, int ldd, cudaStream_t s);
