@@ -198,6 +198,8 @@ def solve_mixed(A, b, prec="bf16", nb=256, **kw):
     """Mixed-precision LU + GMRES-IR. Returns (x, stats). For a 2-D b (n x k) the
     matrix is factored once and every column is refined on its own: x is n x k and
     stats a list of k dicts."""
+    _require_cuda(A)
+    A = colmajor(A, torch.float64)  # one copy for the factorisation and the refinement
     F, ipiv, info = lu_factor_mixed(A, prec, nb)
     x, st = gmresir(A, F, ipiv, b, **kw)
     inf = int(info.item())
@@ -281,6 +283,8 @@ def chol_gmresir(A, F, b, tol=1e-14, inner_tol=1e-8, max_outer=10, restart_m=50,
 
 def solve_chol_mixed(A, b, prec="fp16x3", nb=256, **kw):
     """Mixed-precision Cholesky + GMRES-IR for SPD A. Returns (x, stats)."""
+    _require_cuda(A)
+    A = colmajor(A, torch.float64)
     F, info = chol_factor_mixed(A, prec, nb)
     x, st = chol_gmresir(A, F, b, **kw)
     inf = int(info.item())

@@ -48,6 +48,16 @@ GBLA_DEVINL bool gbla_wait_geq(const unsigned* p, unsigned target, uint64_t limi
   }
 }
 
+// FP32 -> FP64 with integer instructions: the conversion instruction occupies the
+// FP64 pipe like a multiply-add does (64 clocks a warp). Zeros, subnormals,
+// infinities and NaN take it.
+GBLA_DEVINL double to_f64(float f) {
+  const unsigned b = __float_as_uint(f);
+  if ((((b >> 23) + 1u) & 0xffu) <= 1u) return (double)f;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+GBLA_DEVINL double to_f64(double f) { return f; }
+
 template <typename T>
 GBLA_DEVINL T warp_sum(T v) {
 #pragma unroll

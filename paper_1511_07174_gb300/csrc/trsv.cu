@@ -237,6 +237,7 @@ constexpr int kTcMaxG = 4;                // right-hand sides of a chain
 constexpr int kTcMaxC = 4;                // chains of a launch
 constexpr int kTcChunk = 16;              // blocks per helper task
 constexpr int kTcNear = 2;                // blocks the chain multiplies itself
+constexpr int kTcLone = 4;                // blocks before those that a task takes one by one
 constexpr float kTcRefine = 1024.0f;
 constexpr float kTcMaxGrowth = 1e8f;
 constexpr unsigned long long kXUnset = 0xffffffffffffffffull;
@@ -471,7 +472,8 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
   __shared__ double s_x[2][NR][kTsBS];        // x_s, by parity of s
   __shared__ double s_y[2][NR][kTsBS];        // y_s
   __shared__ alignas(8) uint64_t s_bar[2][2][NR];
-  __shared__ double s_xq[2][NR][kTsBS];       // helpers: the x values of a block
+  __shared__ double s_xq[NR == 1 ? 1 : 2][NR][kTsBS];  // helpers: the x values of a block
+  __shared__ double s_xs[2][NR == 1 ? 4 : 1][kTsBS];   // or (one right-hand side) of four
   __shared__ double s_part[TRANS ? 32 * 33 : 8 * NR * 32];
   __shared__ volatile double s_y0[kTcRing][NR][kOwn];  // start values of y_s, by s mod kTcRing
   __shared__ volatile int s_have[NR][kOwn];   // steps whose start value is there
@@ -626,7 +628,7 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
           double acc = 0.0;
           if (s >= 2) {
 #pragma unroll
-            for (int j = 0; j < kCols; ++j) acc = fma(-(double)t2[j], s_x[par][c][grp + kGrp * j], acc);
+            for (int j = 0; j < kCols; ++j) acc = fma(-to_f64(t2[j]), s_x[par][c][grp + kGrp * j], acc);
           }
           load_t(s + 1, 2, t2);
           if (wr == 0 && lane == 0) s_step[c] = s;
@@ -658,7 +660,7 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
             }
             if (wr == 0 && lane == 0) cl_mbar_arm(bar, kTsBS * 8);
 #pragma unroll
-            for (int j = 0; j < kCols; ++j) acc = fma(-(double)t1[j], s_x[par ^ 1][c][grp + kGrp * j], acc);
+            for (int j = 0; j < kCols; ++j) acc = fma(-to_f64(t1[j]), s_x[par ^ 1][c][grp + kGrp * j], acc);
           }
           acc = row_sum(acc);
           load_t(s + 1, 1, t1);
@@ -778,46 +780,80 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
             if (rr < n && cc < n) tc_prefetch(TRANS ? T + cc + (size_t)rr * a.ldt : T + rr + (size_t)cc * a.ldt);
           }
         }
-        // one x value per thread and block: right-hand side xc, row xj of the block
+        // one x value per thread: right-hand side xc, row xj of the block (a single
+        // right-hand side: of four blocks at once)
         const int xj = tid & 63, xc = tid >> 6;
-        auto x_ptr = [&](int sp) -> const double* {
-          const int r = (a.fwd ? sp : nblk - 1 - sp) * kTsBS + xj;
-          return xc < nc && r < n ? X + r + (size_t)xc * a.ldx : nullptr;
-        };
-        // x is loaded one block ahead, tiles one or (a single right-hand side: little
-        // work per tile) two blocks ahead
-        constexpr int kAhead = NR == 1 ? 2 : 1;
-        Ts cur[8], n1[8], n2[8];
-        load(lo, cur);
-        if (kAhead == 2 && lo + 1 < hi) load(lo + 1, n1);
-        const double* xp = x_ptr(lo);
-        unsigned long long xb = xp ? tc_load(xp) : 0ull;
-        for (int sp = lo; sp < hi; ++sp) {
-          double(*xq)[kTsBS] = s_xq[sp & 1];
-          bool late = false;
-          double xv = __longlong_as_double((long long)xb);
-          if (xp && xb == kXUnset) late = !tc_poll(xp, a.wait_ns, &xv);
-          if (xc < NR) xq[xc][xj] = xv;
-          // after the use of x: a wait for it would also wait for loads issued before it
-          if (sp + 1 < hi) {
-            xp = x_ptr(sp + 1);
-            xb = xp ? tc_load(xp) : 0ull;
+        if constexpr (NR == 1) {
+          // Little work per tile: a round trip to L2 for x and a barrier per tile would
+          // be most of the time. Four blocks share them, but for the last ones of the
+          // row, which are waited for one by one.
+          const int lone = hi == s - kTcNear ? kTcLone : 0;  // blocks at the end taken singly
+          Ts cur[4][8];
+          int sp = lo, step = hi - lone - lo >= 4 ? 4 : 1;
+          auto fetch = [&](int b0, int nb) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (u < nb) load(b0 + u, cur[u]);
+          };
+          fetch(sp, step);
+          for (int par = 0; sp < hi; par ^= 1) {
+            bool late = false;
+            const int r = (a.fwd ? sp + xc : nblk - 1 - sp - xc) * kTsBS + xj;
+            double xv = 0.0;
+            if (xc < step && r < n) late = !tc_poll(X + r, a.wait_ns, &xv);
+            s_xs[par][xc][xj] = xv;
+            stop = tc_help_sync_or(late);
+            if (stop) break;
+            const int next = sp + step, nstep = hi - lone - next >= 4 ? 4 : 1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              if (u < step) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + 8 * j;
+                  acc[i][0] = fma(to_f64(cur[u][j]), s_xs[par][u][jj], acc[i][0]);
+                }
+              }
+              // straight into the registers just used: a move would wait for the load
+              if (u < nstep && next + u < hi) load(next + u, cur[u]);
+            }
+            sp = next;
+            step = nstep;
           }
-          if (sp + kAhead < hi) load(sp + kAhead, kAhead == 2 ? n2 : n1);
-          stop = tc_help_sync_or(late);
-          if (stop) break;
+        } else {
+          auto x_ptr = [&](int sp) -> const double* {
+            const int r = (a.fwd ? sp : nblk - 1 - sp) * kTsBS + xj;
+            return xc < nc && r < n ? X + r + (size_t)xc * a.ldx : nullptr;
+          };
+          // x and tiles are loaded one block ahead, which the work on a tile covers
+          Ts cur[8], n1[8];
+          load(lo, cur);
+          const double* xp = x_ptr(lo);
+          unsigned long long xb = xp ? tc_load(xp) : 0ull;
+          for (int sp = lo; sp < hi; ++sp) {
+            double(*xq)[kTsBS] = s_xq[sp & 1];
+            bool late = false;
+            double xv = __longlong_as_double((long long)xb);
+            if (xp && xb == kXUnset) late = !tc_poll(xp, a.wait_ns, &xv);
+            if (xc < NR) xq[xc][xj] = xv;
+            // after the use of x: a wait for it would also wait for loads issued before it
+            if (sp + 1 < hi) {
+              xp = x_ptr(sp + 1);
+              xb = xp ? tc_load(xp) : 0ull;
+              load(sp + 1, n1);
+            }
+            stop = tc_help_sync_or(late);
+            if (stop) break;
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const double v = (double)cur[j];
-            const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + 8 * j;
+            for (int j = 0; j < 8; ++j) {
+              const double v = to_f64(cur[j]);
+              const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + 8 * j;
 #pragma unroll
-            for (int c = 0; c < NR; ++c)
-              if (c < nc) acc[i][c] = fma(v, xq[c][jj], acc[i][c]);
-          }
+              for (int c = 0; c < NR; ++c)
+                if (c < nc) acc[i][c] = fma(v, xq[c][jj], acc[i][c]);
+            }
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            cur[j] = n1[j];
-            if (kAhead == 2) n1[j] = n2[j];
+            for (int j = 0; j < 8; ++j) cur[j] = n1[j];
           }
         }
         if (stop) {
