@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(256)
 // 5.2 ms for both factors with clusters of 8, 3.2 with 4).
 //
 // Measured (both factors of one solve): n = 4096, 16 right-hand sides 6.5 -> 1.04
-// ms; n = 8192 16.2 -> 3.2 ms; the preconditioner of n = 2500 0.25 -> 0.17 ms.
+// ms; n = 8192 16.2 -> 3.1 ms; the preconditioner of n = 2500 0.25 -> 0.14 ms.
 //
 // Progress. Tasks are drawn by ticket, per chain, in solve order, so a task only
 // waits for x values and partial sums of tasks already drawn by running CTAs.
@@ -232,7 +232,6 @@ namespace gbla {
 
 constexpr int kTcWarps = 4;               // chain warps of a CTA per right-hand side
 constexpr int kTcRing = 4;                // steps the start values of y may be ahead
-constexpr int kTcHelp = 256;              // threads of the helper part
 constexpr int kTcMaxG = 4;                // right-hand sides of a chain
 constexpr int kTcMaxC = 4;                // chains of a launch
 constexpr int kTcChunk = 16;              // blocks per helper task
@@ -432,16 +431,20 @@ GBLA_DEVINL void tc_push(uint32_t raddr, double v, uint32_t rbar) {
                "l"(__double_as_longlong(v)), "r"(rbar)
                : "memory");
 }
-// barrier of the helper part; true in every thread if f was in any
+// barrier of the helper part; the first, true in every thread if f was in any
+template <int H>
 GBLA_DEVINL bool tc_help_sync_or(bool f) {
   uint32_t r;
   asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
                : "=r"(r)
-               : "r"((uint32_t)f), "n"(kTcHelp)
+               : "r"((uint32_t)f), "n"(H)
                : "memory");
   return r != 0;
 }
-GBLA_DEVINL void tc_help_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTcHelp) : "memory"); }
+template <int H>
+GBLA_DEVINL void tc_help_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(H) : "memory");
+}
 
 struct TcArgs {
   int n, nblk, ncols, G, C, ldt, ldr, ldx;
@@ -457,14 +460,26 @@ struct TcArgs {
 };
 
 // threads: helpers, chain warps, the warp that fetches the start values of y
-template <int NR>
+// H helper threads: 256, or 128 in the variant that leaves room for others. The
+// latter, also held to 64 registers, is for the preconditioner of systems above 4096
+// rows: 288 threads leave an SM room for the 512 threads of 91 registers of such a
+// system's panel kernel, which needs 16 SMs of one GPC at the same time and would
+// otherwise wait for the whole substitution of another stream's system (three
+// systems of n = 16384 on three streams: 150 -> 141 ms; one alone 77.1 -> 78.7).
+// The panels of smaller systems fit beside the other variant, which is faster (n =
+// 2500, 4 right-hand sides: 22.5 -> 19.7 ms).
+template <int NR, int H>
 constexpr int tc_threads() {
-  return kTcHelp + 32 * kTcWarps * NR + 32;
+  return H + 32 * kTcWarps * NR + 32;
 }
+constexpr int kTcRoomy = 4096;  // rows up to which the panels fit beside 256 helper threads
 
-template <typename Ts, bool TRANS, int NR, int CL>
-__global__ void __launch_bounds__(tc_threads<NR>(), 1)
+template <typename Ts, bool TRANS, int NR, int CL, int H>
+__global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128 ? 3 : 1)
     tc_solve_kernel(const Ts* __restrict__ T, const TcArgs a) {
+  constexpr int kHelp = H;
+  constexpr int kHw = kHelp / 32;               // helper warps
+  constexpr int kEl = 32 * kTsBS / kHelp;       // elements of a 32 x 64 tile per helper thread
   constexpr int kRows = kTsBS / CL / kTcWarps;  // rows of every block per chain warp
   constexpr int kGrp = 32 / kRows;              // lanes that share a row
   constexpr int kCols = kTsBS / kGrp;           // columns of a block per lane
@@ -473,8 +488,8 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
   __shared__ double s_y[2][NR][kTsBS];        // y_s
   __shared__ alignas(8) uint64_t s_bar[2][2][NR];
   __shared__ double s_xq[NR == 1 ? 1 : 2][NR][kTsBS];  // helpers: the x values of a block
-  __shared__ double s_xs[2][NR == 1 ? 4 : 1][kTsBS];   // or (one right-hand side) of four
-  __shared__ double s_part[TRANS ? 32 * 33 : 8 * NR * 32];
+  __shared__ double s_xs[2][kHelp / 64][kTsBS];          // or (one right-hand side) of several
+  __shared__ double s_part[TRANS ? 32 * 33 : kHw * NR * 32];
   __shared__ volatile double s_y0[kTcRing][NR][kOwn];  // start values of y_s, by s mod kTcRing
   __shared__ volatile int s_have[NR][kOwn];   // steps whose start value is there
   __shared__ volatile int s_step[NR];         // the step the chain's first warp is at
@@ -510,7 +525,7 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
     cl_sync();  // every mbarrier of the cluster is ready for the first push
   }
 
-  if (warp == kTcHelp / 32 + kTcWarps * NR) {
+  if (warp == kHelp / 32 + kTcWarps * NR) {
     // ---- start values of y: rhs, or what the last helper task of the block left;
     // polled here so that the chain never waits for a load it issued too late ------
     if (in_chain) {
@@ -548,9 +563,9 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
         more = __any_sync(0xffffffffu, more);
       }
     }
-  } else if (warp >= kTcHelp / 32) {
+  } else if (warp >= kHelp / 32) {
     // ---- chain: four warps per right-hand side, each with its own rows ----------
-    const int c = (warp - kTcHelp / 32) / kTcWarps, wr = (warp - kTcHelp / 32) % kTcWarps;
+    const int c = (warp - kHelp / 32) / kTcWarps, wr = (warp - kHelp / 32) % kTcWarps;
     const int col = cluster * a.G + c;
     if (in_chain) {
       bool ok = true;
@@ -709,7 +724,7 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
       // the chain's operands (its rows of the blocks (s, s - 1) and (s, s - 2)), in
       // solve order: it loads them only one step ahead, less than HBM's latency
       constexpr int kU = TRANS ? kOwn * 2 * kTsBS / kLine : 2 * kTsBS;  // lines of a step
-      for (int i = tid; i < nblk * kU; i += kTcHelp) {
+      for (int i = tid; i < nblk * kU; i += kHelp) {
         const int s = i / kU, u = i % kU;
         const int r = (a.fwd ? s : nblk - 1 - s) * kTsBS + kOwn * (int)cl_ctarank() + (TRANS ? u % kOwn : 0);
         const int off = TRANS ? u / kOwn * kLine : u;  // column among those of the two blocks
@@ -726,7 +741,7 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
       int s = 0;
       bool stop = false;
       while (nc > 0 && !stop) {
-        tc_help_sync();  // the previous task's shared memory is no longer read
+        tc_help_sync<kHelp>();  // the previous task's shared memory is no longer read
         if (tid == 0) {
           bool draw = true;
           if (in_chain) {
@@ -745,27 +760,27 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
           const unsigned t = draw ? atomicAdd(&a.ctrl[ch], 1u) : 0xffffffffu;
           s_t = t < (unsigned)ntask ? (int)t : -1;
         }
-        tc_help_sync();
+        tc_help_sync<kHelp>();
         const int t = s_t;
         if (t < 0) break;
         while (tc_first(s + 1) <= t) ++s;
         const int idx = t - tc_first(s), chunk = idx >> 1, half = idx & 1;
         const int lo = chunk * kTcChunk, hi = min(lo + kTcChunk, s - kTcNear);
         const int r0 = (a.fwd ? s : nblk - 1 - s) * kTsBS + 32 * half;  // first of the 32 rows
-        constexpr int NA = TRANS ? 4 : 1;  // rows of a thread
+        constexpr int NA = TRANS ? kEl / 2 : 1;  // rows of a thread
         double acc[NA][NR];
 #pragma unroll
         for (int i = 0; i < NA; ++i)
 #pragma unroll
           for (int c = 0; c < NR; ++c) acc[i][c] = 0.0;
-        // a thread's 8 elements of a 32 x 64 tile: one row and columns warp + 8 j,
-        // or (stored transposed) rows 4 warp + i and columns lane + 32 h
-        auto load = [&](int sp, Ts (&v)[8]) {
+        // a thread's elements of a 32 x 64 tile: one row and columns warp + kHw j,
+        // or (stored transposed) rows NA warp + i and columns lane + 32 h
+        auto load = [&](int sp, Ts (&v)[kEl]) {
           const int c0 = (a.fwd ? sp : nblk - 1 - sp) * kTsBS;
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int rr = TRANS ? r0 + 4 * warp + (j >> 1) : r0 + lane;
-            const int cc = TRANS ? c0 + lane + 32 * (j & 1) : c0 + warp + 8 * j;
+          for (int j = 0; j < kEl; ++j) {
+            const int rr = TRANS ? r0 + NA * warp + (j >> 1) : r0 + lane;
+            const int cc = TRANS ? c0 + lane + 32 * (j & 1) : c0 + warp + kHw * j;
             v[j] = (rr < n && cc < n) ? (TRANS ? T[cc + (size_t)rr * a.ldt] : T[rr + (size_t)cc * a.ldt]) : (Ts)0;
           }
         };
@@ -775,24 +790,25 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
           const int c0 = (a.fwd ? lo : nblk - hi) * kTsBS, ncol = (hi - lo) * kTsBS;
           constexpr int kPer = 32 / kLine > 0 ? 32 / kLine : 1;  // lines of a 32-row column
           const int lines = TRANS ? 32 * (ncol / kLine) : ncol * kPer;
-          for (int i = tid; i < lines; i += kTcHelp) {
+          for (int i = tid; i < lines; i += kHelp) {
             const int rr = r0 + (TRANS ? i & 31 : i % kPer * kLine), cc = c0 + (TRANS ? (i >> 5) * kLine : i / kPer);
             if (rr < n && cc < n) tc_prefetch(TRANS ? T + cc + (size_t)rr * a.ldt : T + rr + (size_t)cc * a.ldt);
           }
         }
         // one x value per thread: right-hand side xc, row xj of the block (a single
-        // right-hand side: of four blocks at once)
+        // right-hand side: of kU blocks at once)
         const int xj = tid & 63, xc = tid >> 6;
         if constexpr (NR == 1) {
           // Little work per tile: a round trip to L2 for x and a barrier per tile would
-          // be most of the time. Four blocks share them, but for the last ones of the
+          // be most of the time. kU blocks share them, but for the last ones of the
           // row, which are waited for one by one.
           const int lone = hi == s - kTcNear ? kTcLone : 0;  // blocks at the end taken singly
-          Ts cur[4][8];
-          int sp = lo, step = hi - lone - lo >= 4 ? 4 : 1;
+          constexpr int kU = kHelp / 64;  // blocks of a group
+          Ts cur[kU][kEl];
+          int sp = lo, step = hi - lone - lo >= kU ? kU : 1;
           auto fetch = [&](int b0, int nb) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < kU; ++u)
               if (u < nb) load(b0 + u, cur[u]);
           };
           fetch(sp, step);
@@ -802,15 +818,15 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
             double xv = 0.0;
             if (xc < step && r < n) late = !tc_poll(X + r, a.wait_ns, &xv);
             s_xs[par][xc][xj] = xv;
-            stop = tc_help_sync_or(late);
+            stop = tc_help_sync_or<kHelp>(late);
             if (stop) break;
-            const int next = sp + step, nstep = hi - lone - next >= 4 ? 4 : 1;
+            const int next = sp + step, nstep = hi - lone - next >= kU ? kU : 1;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < kU; ++u) {
               if (u < step) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + 8 * j;
+                for (int j = 0; j < kEl; ++j) {
+                  const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + kHw * j;
                   acc[i][0] = fma(to_f64(cur[u][j]), s_xs[par][u][jj], acc[i][0]);
                 }
               }
@@ -826,7 +842,7 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
             return xc < nc && r < n ? X + r + (size_t)xc * a.ldx : nullptr;
           };
           // x and tiles are loaded one block ahead, which the work on a tile covers
-          Ts cur[8], n1[8];
+          Ts cur[kEl], n1[kEl];
           load(lo, cur);
           const double* xp = x_ptr(lo);
           unsigned long long xb = xp ? tc_load(xp) : 0ull;
@@ -842,18 +858,18 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
               xb = xp ? tc_load(xp) : 0ull;
               load(sp + 1, n1);
             }
-            stop = tc_help_sync_or(late);
+            stop = tc_help_sync_or<kHelp>(late);
             if (stop) break;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
+            for (int j = 0; j < kEl; ++j) {
               const double v = to_f64(cur[j]);
-              const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + 8 * j;
+              const int i = TRANS ? j >> 1 : 0, jj = TRANS ? lane + 32 * (j & 1) : warp + kHw * j;
 #pragma unroll
               for (int c = 0; c < NR; ++c)
                 if (c < nc) acc[i][c] = fma(v, xq[c][jj], acc[i][c]);
             }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) cur[j] = n1[j];
+            for (int j = 0; j < kEl; ++j) cur[j] = n1[j];
           }
         }
         if (stop) {
@@ -877,11 +893,13 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
 #pragma unroll
           for (int c = 0; c < NR; ++c)
             if (c < nc) part[warp][c][lane] = acc[0][c];
-          tc_help_sync();
-          for (int i = tid; i < 32 * nc; i += kTcHelp) {
+          tc_help_sync<kHelp>();
+          for (int i = tid; i < 32 * nc; i += kHelp) {
             const int rr = i & 31, c = i >> 5;
-            publish(rr, c, ((part[0][c][rr] + part[1][c][rr]) + (part[2][c][rr] + part[3][c][rr])) +
-                               ((part[4][c][rr] + part[5][c][rr]) + (part[6][c][rr] + part[7][c][rr])));
+            double sum = (part[0][c][rr] + part[1][c][rr]) + (part[2][c][rr] + part[3][c][rr]);
+            if constexpr (kHw == 8)
+              sum += (part[4][c][rr] + part[5][c][rr]) + (part[6][c][rr] + part[7][c][rr]);
+            publish(rr, c, sum);
           }
         } else {
           double(*part)[33] = reinterpret_cast<double(*)[33]>(s_part);
@@ -889,17 +907,20 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
           for (int c = 0; c < NR; ++c)
             if (c < nc) {
 #pragma unroll
-              for (int i = 0; i < 4; ++i) part[4 * warp + i][lane] = acc[i][c];
-              tc_help_sync();
-              const int rr = tid >> 3, e = tid & 7;
-              double sum = (part[rr][e] + part[rr][e + 8]) + (part[rr][e + 16] + part[rr][e + 24]);
+              for (int i = 0; i < NA; ++i) part[NA * warp + i][lane] = acc[i][c];
+              tc_help_sync<kHelp>();
+              constexpr int kPer = kHelp / 32;  // threads of a row
+              const int rr = tid / kPer, e = tid % kPer;
+              double sum = 0.0;
 #pragma unroll
-              for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+              for (int q = 0; q < 32 / kPer; ++q) sum += part[rr][e + kPer * q];
+#pragma unroll
+              for (int o = 1; o < kPer; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
               if (e == 0) publish(rr, c, sum);
-              tc_help_sync();
+              tc_help_sync<kHelp>();
             }
         }
-        if (tc_help_sync_or(late)) {
+        if (tc_help_sync_or<kHelp>(late)) {
           if (tid == 0) gbla_flag_timeout(a.info);
           break;
         }
@@ -925,7 +946,7 @@ __global__ void __launch_bounds__(tc_threads<NR>(), 1)
 }
 
 // clusters of CL CTAs that the device can hold at once (0: none)
-template <typename Ts, bool TRANS, int NR, int CL>
+template <typename Ts, bool TRANS, int NR, int CL, int H>
 static cudaError_t tc_max_clusters(int* out) {
   static std::mutex mu;
   static int known[64];
@@ -946,11 +967,11 @@ static cudaError_t tc_max_clusters(int* out) {
     at[0].val.clusterDim.x = CL;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     q.gridDim = dim3(CL);
-    q.blockDim = dim3(tc_threads<NR>());
+    q.blockDim = dim3(tc_threads<NR, H>());
     q.attrs = at;
     q.numAttrs = 1;
     int k = 0;
-    e = cudaOccupancyMaxActiveClusters(&k, tc_solve_kernel<Ts, TRANS, NR, CL>, &q);
+    e = cudaOccupancyMaxActiveClusters(&k, tc_solve_kernel<Ts, TRANS, NR, CL, H>, &q);
     if (e != cudaSuccess) return e;
     known[dev] = k;
   }
@@ -958,10 +979,10 @@ static cudaError_t tc_max_clusters(int* out) {
   return cudaSuccess;
 }
 
-template <typename Ts, bool TRANS, int NR, int CL>
+template <typename Ts, bool TRANS, int NR, int CL, int H>
 static cudaError_t tc_launch_solve(const Ts* T, TcArgs a, cudaStream_t s) {
   int maxc = 0;
-  cudaError_t e = tc_max_clusters<Ts, TRANS, NR, CL>(&maxc);
+  cudaError_t e = tc_max_clusters<Ts, TRANS, NR, CL, H>(&maxc);
   if (e != cudaSuccess) return e;
   if (maxc < 1) return cudaErrorNotSupported;
   // one CTA per SM: the FP64 units of an SM, which chain and tasks are bound by,
@@ -979,12 +1000,12 @@ static cudaError_t tc_launch_solve(const Ts* T, TcArgs a, cudaStream_t s) {
   at[0].val.clusterDim.x = CL;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)(clusters * CL));
-  cfg.blockDim = dim3(tc_threads<NR>());
+  cfg.blockDim = dim3(tc_threads<NR, H>());
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
   count_launch();
-  return cudaLaunchKernelEx(&cfg, tc_solve_kernel<Ts, TRANS, NR, CL>, T, a);
+  return cudaLaunchKernelEx(&cfg, tc_solve_kernel<Ts, TRANS, NR, CL, H>, T, a);
 }
 
 template <typename Ts, bool TRANS>
@@ -1020,10 +1041,18 @@ static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, c
   a.gated = gated;
   a.info = info;
   a.wait_ns = wait_timeout_ns();
-  if (ncols == 1 && !wide) return tc_launch_solve<Ts, TRANS, 1, 8>(T, a, s);
-  if (sh.G == 1) return tc_launch_solve<Ts, TRANS, 1, 4>(T, a, s);
-  if (sh.G == 2) return tc_launch_solve<Ts, TRANS, 2, 4>(T, a, s);
-  return tc_launch_solve<Ts, TRANS, 4, 4>(T, a, s);
+  const bool one = ncols == 1 && !wide;
+  if constexpr (sizeof(Ts) == 4) {
+    if (n > kTcRoomy && sh.G == 1)
+      return one ? tc_launch_solve<Ts, TRANS, 1, 8, 128>(T, a, s) : tc_launch_solve<Ts, TRANS, 1, 4, 128>(T, a, s);
+  }
+  if (one) return tc_launch_solve<Ts, TRANS, 1, 8, 256>(T, a, s);
+  if (sh.G == 1) return tc_launch_solve<Ts, TRANS, 1, 4, 256>(T, a, s);
+  if constexpr (sizeof(Ts) == 8) {
+    if (sh.G == 2) return tc_launch_solve<Ts, TRANS, 2, 4, 256>(T, a, s);
+    return tc_launch_solve<Ts, TRANS, 4, 4, 256>(T, a, s);
+  }
+  return cudaErrorInvalidValue;  // the preconditioner takes at most kTcMaxC columns
 }
 
 static cudaError_t tc_fill(int n, int ncols, TcShape sh, double* X, int ldx, char* scratch, size_t ctrl_words,

@@ -62,3 +62,12 @@ def test_smallest_workspace_and_step_limit():
     b1 = [s.beta0 for s in st]
     assert run(lib.gbla_gmresir_workspace_nrhs(n, k, 50), 0) == _lib.GBLA_ERR_NOT_CONVERGED
     assert not any(s.converged for s in st) and all(0.3 < s.beta0 / b < 3 for s, b in zip(st, b1))
+
+
+# above 4096 rows the preconditioner runs with half the helper threads
+@pytest.mark.parametrize("n,k", [(4160, 1), (4161, 3)])
+def test_large_preconditioner(n, k):
+    A, B = _case(n, k, 11)
+    F, ipiv, _ = api.lu_factor_mixed(A, "bf16")
+    X, st = api.gmresir(A, F, ipiv, B)
+    assert all(s["converged"] for s in st) and float(api.backward_error(A, X, B).max()) <= 1e-14
