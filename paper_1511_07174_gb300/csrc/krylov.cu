@@ -13,7 +13,7 @@ constexpr int kResCols = 512;   // columns per CTA, at most
 
 // Columns per CTA: the product is bound by HBM (8 bytes per multiply-add) and by
 // the FP64 pipe alike, so every SM should have the same share of it; 512 while that
-// makes four CTAs per SM, else less (measured, n = 2500: 36 -> 14 us).
+// makes four CTAs per SM, else less (measured, n = 8192: 146 -> 122 us).
 static int res_cols(int n) {
   const int sms = device_props().num_sms > 0 ? device_props().num_sms : 152;
   int cols = kResCols;
