@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
 #pragma unroll
       for (int i = 0; i < kItems; ++i) s[i] = 0;
       bool more = true;
-      while (more && *(volatile int*)&s_done != NR * kTcWarps) {
+      while (more) {
         more = false;
 #pragma unroll
         for (int i = 0; i < kItems; ++i) {
@@ -560,7 +560,9 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
           __threadfence_block();
           s_have[c][rr] = ++s[i];
         }
-        more = __any_sync(0xffffffffu, more);
+        // one decision for the warp; a chain that gave up ends it too
+        const bool over = *(volatile int*)&s_done == NR * kTcWarps;
+        more = __any_sync(0xffffffffu, more) && !__any_sync(0xffffffffu, over);
       }
     }
   } else if (warp >= kHelp / 32) {
