@@ -102,14 +102,15 @@ void gbla_set_wait_timeout_ns(uint64_t ns);
 uint64_t gbla_get_wait_timeout_ns(void);
 
 /*
- * Cap on the number of CTAs of the refinement's preconditioner substitution
- * (the inverted-diagonal-block forward and back solves inside
- * gbla_gmresir_solve*, gbla_chol_gmresir_solve_nrhs, gbla_gmres_solve and
- * gbla_bicgstab_solve). The substitution runs as a persistent grid of at most
- * one CTA per SM that draws its tasks in order; a cap leaves the other SMs
- * free for work on other streams (several systems solved concurrently). The
- * result does not depend on the cap. 0 (default): one CTA per SM.
- * Process-wide. Returns -1 for ctas < 0.
+ * Cap on the number of CTAs of the triangular solves (gbla_lu_solve,
+ * gbla_chol_solve, and the preconditioner inside gbla_gmresir_solve*,
+ * gbla_chol_gmresir_solve_nrhs, gbla_gmres_solve and gbla_bicgstab_solve). They
+ * run as a persistent grid of thread-block clusters of 4 or 8 CTAs, at most one
+ * CTA per SM, that draws its tasks in order; a cap leaves the other SMs free for
+ * work on other streams (several systems solved concurrently). It is rounded down
+ * to whole clusters, but for the one to four that hold the chains of right-hand
+ * sides, which always run. The result does not depend on the cap. 0 (default):
+ * as many as the device holds. Process-wide. Returns -1 for ctas < 0.
  */
 int gbla_set_substitution_ctas(int ctas);
 int gbla_get_substitution_ctas(void);
