@@ -967,7 +967,7 @@ struct IrWork {
   double* cs;
   double* sn;
   double* g;
-  double* st;  // GmresState {res, pad} of every column, then info
+  double* st;  // GmresState {res, pad} of every column; the word before them is info
   double* slots;
   unsigned* counter;
   char* flags;  // scratch of the triangular solves
@@ -1003,8 +1003,10 @@ static size_t ir_layout(Carver& c, int n, int m, IrWork* w, int cols = 1) {
   t.cs = c.take<double>(k * m);
   t.sn = c.take<double>(k * m);
   t.g = c.take<double>(k * (m + 1));
-  t.st = c.take<double>(2 * k + 1);
-  t.info = reinterpret_cast<int*>(t.st + 2 * k);
+  // info first: a group of fewer columns than the layout finds it at the same place
+  double* head = c.take<double>(2 * k + 1);
+  t.info = reinterpret_cast<int*>(head);
+  t.st = head + 1;
   t.slots = c.take<double>(k * mgs_slots_doubles());
   t.counter = c.take<unsigned>(k);
   t.flags = c.take<char>(trsv_scratch_bytes(nn, cols));
@@ -1060,15 +1062,15 @@ static int read_scalar(double* host, const double* dev, const int* d_info, cudaS
   return info == GBLA_INFO_TIMEOUT ? GBLA_ERR_TIMEOUT : GBLA_OK;
 }
 
-// the residual norm of every column, and info, in one copy
+// info, and the residual norm of every column of the group, in one copy
 static int read_residuals(double* res, const IrWork& w, int cols, cudaStream_t s) {
   double h[2 * kIrCols + 1];
-  if (cudaMemcpyAsync(h, w.st, sizeof(double) * (2 * cols + 1), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+  if (cudaMemcpyAsync(h, w.info, sizeof(double) * (2 * cols + 1), cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return GBLA_ERR_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return GBLA_ERR_CUDA;
-  for (int c = 0; c < cols; ++c) res[c] = h[2 * c];
+  for (int c = 0; c < cols; ++c) res[c] = h[2 * c + 1];
   int info;
-  memcpy(&info, &h[2 * cols], sizeof(int));
+  memcpy(&info, &h[0], sizeof(int));
   return info == GBLA_INFO_TIMEOUT ? GBLA_ERR_TIMEOUT : GBLA_OK;
 }
 
