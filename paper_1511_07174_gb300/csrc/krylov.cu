@@ -1,6 +1,7 @@
 // FP64 residual, norms and the GMRES building blocks (paper section 2: GMRES
 // with Gram-Schmidt orthogonalisation and restarts; here the inner solver of
 // iterative refinement).
+#include <algorithm>
 #include <climits>
 
 #include "common.cuh"
@@ -21,9 +22,16 @@ static int res_cols(int n) {
   return cols;
 }
 
+// n doubles per chunk and right-hand side. The number of chunks drops where their
+// width doubles, the size must not (a program's scratch for its largest order serves
+// every smaller one): chunks narrower than kResCols are at least 64 wide, and their
+// CTAs at most twice the 4 sms - 1 of chunks twice as wide, that is
+// n chunks <= 2 (4 sms - 1) kResRows.
 size_t residual_work_doubles(int n, int nrhs) {
-  const size_t chunks = (size_t)((n + res_cols(n) - 1) / res_cols(n));
-  return chunks * (size_t)(n > 0 ? n : 1) * (size_t)(nrhs > 0 ? nrhs : 1);
+  const size_t sms = (size_t)(device_props().num_sms > 0 ? device_props().num_sms : 152);
+  const size_t nn = (size_t)(n > 0 ? n : 1);
+  const size_t narrow = std::min(nn * ((nn + 63) / 64), 2 * (4 * sms - 1) * (size_t)kResRows);
+  return std::max(nn * ((nn + kResCols - 1) / kResCols), narrow) * (size_t)(nrhs > 0 ? nrhs : 1);
 }
 
 // part[chunk][c][i] = sum_{j in chunk} A[i, j] X[j, c]   (ABS: |A[i, j]|, X unused).
