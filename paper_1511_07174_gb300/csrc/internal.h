@@ -182,7 +182,7 @@ cudaError_t launch_gemm_tc(int kind, int M, int N, int K, const void* Ak, int ld
 // ---- triangular solves ------------------------------------------------------
 // lower: the stored triangle; trans: solve with its transpose; unit: unit diagonal.
 // X <- op(T)^-1 rhs (n x nrhs, FP64, distinct buffers). D: diag_inv_doubles(n)
-// doubles; scratch: trsv_scratch_bytes(n, nrhs), 8-byte aligned.
+// doubles; scratch: trsv_scratch_bytes(n, nrhs), 16-byte aligned.
 cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, const double* T, int ldt,
                         const double* rhs, int ldr, double* X, int ldx, double* D, void* scratch, int* info,
                         cudaStream_t s);

@@ -223,10 +223,12 @@ __global__ void __launch_bounds__(256)
 // up to g u |T_ss||x_s| where a substitution leaves u |T_ss||x_s|. g is a few hundred
 // for most blocks of dense LU and Cholesky factors, where the two cannot be told
 // apart in the solution (n = 512 .. 1500, L and U, against extended precision), and
-// now and then thousands (a small pivot inside a block). The set-up computes it:
-// blocks above kTcRefine get one step of refinement, x_s += D_s (y_s - T_ss x_s),
-// which brings the residual down by another factor g u; with a block above
-// kTcMaxGrowth, or one that is not finite (a zero pivot), the FP64 solves take the
+// now and then thousands (a small pivot inside a block). The set-up computes a bound
+// of it: the four CTAs that share a block each leave the largest row sum over their
+// 16 columns of |D||T_ss|, and g is at most the sum of the four. Blocks whose bound is
+// above kTcRefine get one step of refinement, x_s += D_s (y_s - T_ss x_s), which
+// brings the residual down by another factor g u; with a block of which one part is
+// above kTcMaxPart, or not finite (a zero pivot), the FP64 solves take the
 // substitution kernel above instead. The preconditioner needs neither.
 namespace gbla {
 
@@ -238,7 +240,7 @@ constexpr int kTcChunk = 16;              // blocks per helper task
 constexpr int kTcNear = 2;                // blocks the chain multiplies itself
 constexpr int kTcLone = 4;                // blocks before those that a task takes one by one
 constexpr float kTcRefine = 1024.0f;
-constexpr float kTcMaxGrowth = 1e8f;
+constexpr float kTcMaxPart = 0.25e8f;     // a quarter of the growth that one refinement step is good for
 constexpr unsigned long long kXUnset = 0xffffffffffffffffull;
 
 // helper tasks of block s (two row halves by chunks) and of the blocks before it
@@ -264,12 +266,12 @@ static TcShape tc_shape(int nrhs) {
 }
 
 // control words: [0, kTcMaxC) tickets, [kTcMaxC] set when a diagonal block's
-// inverse is not safe, a word per block set when it is to be refined, then the
-// substitution kernel's flags
-constexpr int kTcCtrl = kTcMaxC + 1;
+// inverse is not safe, from kTcCtrl on four per block with the parts of its growth
+// (floats; 16-byte aligned), then the substitution kernel's flags
+constexpr int kTcCtrl = 2 * kTcMaxC;
 static size_t tc_ctrl_words(int n, int nrhs) {
   const int per = nrhs < kTcMaxC * kTcMaxG ? nrhs : kTcMaxC * kTcMaxG;
-  return (kTcCtrl + (n + kTsBS - 1) / kTsBS + trsv_flags_count(n, per) + 31) / 32 * 32;
+  return (kTcCtrl + (size_t)4 * ((n + kTsBS - 1) / kTsBS) + trsv_flags_count(n, per) + 31) / 32 * 32;
 }
 size_t diag_inv_doubles(int n) {
   return (size_t)((n + kTsBS - 1) / kTsBS) * kTsBS * kTsBS;
@@ -387,8 +389,10 @@ __global__ void __launch_bounds__(256)
       }
     f += __shfl_xor_sync(0xffffffffu, f, 1);
     f += __shfl_xor_sync(0xffffffffu, f, 2);
-    if (!(f <= kTcMaxGrowth)) *bad = 1u;
-    if (f > kTcRefine) bad[1 + b] = 1u;
+    if (!(f <= kTcMaxPart)) *bad = 1u;
+    // floats >= 0 order like their bits
+    const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(f));
+    if ((tid & 31) == 0) atomicMax(&bad[kTcCtrl - kTcMaxC + blockIdx.x], top);
   }
   double* Db = D + (size_t)b * kTsBS * kTsBS;
   for (int idx = tid; idx < kTsBS * 16; idx += 256) {
@@ -611,10 +615,11 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
         load_t(0, 1, t1);
         load_t(0, 2, t2);
         load_d(0, d);
-        auto load_hard = [&](int s) {
-          return a.gated && s < nblk ? a.ctrl[kTcCtrl + (a.fwd ? s : nblk - 1 - s)] : 0u;
+        auto load_growth = [&](int s) {
+          return a.gated && s < nblk ? reinterpret_cast<const float4*>(a.ctrl + kTcCtrl)[a.fwd ? s : nblk - 1 - s]
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
         };
-        unsigned hard = load_hard(0);
+        float4 growth = load_growth(0);
         int ny = 0;  // exchanges through s_y so far: one per step, three in a refined one
         // v of every row to every CTA; false if a wait gave up
         auto exchange_y = [&](double v) -> bool {
@@ -684,7 +689,7 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
           ok = exchange_y(acc);
           if (!ok) break;
           double x = times_d(d);
-          if (hard != 0u) {
+          if ((growth.x + growth.y) + (growth.z + growth.w) > kTcRefine) {
             // x += D (y - T_ss x)
             ok = exchange_y(x);
             if (!ok) break;
@@ -706,7 +711,7 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
           const int r = (a.fwd ? s : nblk - 1 - s) * kTsBS + rb;
           if (grp == 0 && r < n) tc_announce(X + r, x);
           load_d(s + 1, d);
-          hard = load_hard(s + 1);
+          growth = load_growth(s + 1);
         }
       }
       __syncwarp();
@@ -1066,7 +1071,7 @@ static cudaError_t tc_fill(int n, int ncols, TcShape sh, double* X, int ldx, cha
   tc_fill_kernel<<<(unsigned)grid, 256, 0, s>>>(n, ncols, X, ldx,
                                                 reinterpret_cast<double*>(scratch + ctrl_words * sizeof(unsigned)), np,
                                                 reinterpret_cast<unsigned*>(scratch),
-                                                keep_bad ? kTcCtrl + (n + kTsBS - 1) / kTsBS : kTcMaxC,
+                                                keep_bad ? kTcCtrl + 4 * ((n + kTsBS - 1) / kTsBS) : kTcMaxC,
                                                 (int)ctrl_words);
   count_launch();
   return cudaGetLastError();
@@ -1108,7 +1113,7 @@ cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, cons
     const int G = (ncols + C - 1) / C;
     const int Cl = (ncols + G - 1) / G;  // chains that hold columns
     const int grid = Cl * nblk;
-    unsigned* flags = ctrl + kTcCtrl + nblk;
+    unsigned* flags = ctrl + kTcCtrl + 4 * nblk;
     const unsigned* gate = blocks ? ctrl + kTcMaxC : nullptr;
 #define GBLA_TRSV(LW, TR, UN)                                                                         \
   trsv_chain_kernel<double, LW, TR, UN><<<grid, 256, 0, s>>>(n, ncols, G, Cl, T, ldt, R, ldr, Xc, ldx, \
