@@ -221,15 +221,24 @@ __global__ void __launch_bounds__(256)
 //
 // Accuracy. With g = || |D||T_ss| || the product x_s = D_s y_s leaves a residual of
 // up to g u |T_ss||x_s| where a substitution leaves u |T_ss||x_s|. g is a few hundred
-// for most blocks of dense LU and Cholesky factors, where the two cannot be told
-// apart in the solution (n = 512 .. 1500, L and U, against extended precision), and
-// now and then thousands (a small pivot inside a block). The set-up computes a bound
-// of it: the four CTAs that share a block each leave the largest row sum over their
-// 16 columns of |D||T_ss|, and g is at most the sum of the four. Blocks whose bound is
-// above kTcRefine get one step of refinement, x_s += D_s (y_s - T_ss x_s), which
-// brings the residual down by another factor g u; with a block of which one part is
-// above kTcMaxPart, or not finite (a zero pivot), the FP64 solves take the
-// substitution kernel above instead. The preconditioner needs neither.
+// for most blocks of U of a dense matrix, less for L and Cholesky factors, and now and
+// then thousands (a small pivot inside a block). The set-up computes a bound of it:
+// the four CTAs that share a block each leave the largest row sum over their 16
+// columns of |D||T_ss|, and g is at most the sum of the four. Blocks whose bound is
+// above a limit get one step of refinement, x_s += D_s (y_s - T_ss x_s), which brings
+// the residual down by another factor g u; with a block of which one part is above
+// kTcMaxPart, or not finite (a zero pivot), the FP64 solves take the substitution
+// kernel above instead. The preconditioner needs neither.
+// The limit is where the solution is no further from the exact one than that of the
+// substitution kernel for the same factors (LU of uniform random matrices, extended
+// precision, ratio of the errors' 2-norms, geometric mean over seeds, A and A^t):
+//   n                  100        200        300        512        1000       2500
+//   limit 1024      1.62 1.57  1.84 1.57  1.36 1.33  1.29 1.02  0.88 0.73  0.68 0.41
+//   limit 128       0.91 0.83  0.96 0.95  0.88 0.82  0.80 0.79  0.77 0.60  0.72 0.39
+// With few blocks their own residuals are what counts, with many the sums over the
+// blocks before them, which are shorter here than in that kernel's chains. The
+// refinement of most blocks costs the solve of n = 512 180 -> 214 us, 1000 211 -> 267
+// and would cost 4096 451 -> 752.
 namespace gbla {
 
 constexpr int kTcWarps = 4;               // chain warps of a CTA per right-hand side
@@ -239,7 +248,7 @@ constexpr int kTcMaxC = 4;                // chains of a launch
 constexpr int kTcChunk = 16;              // blocks per helper task
 constexpr int kTcNear = 2;                // blocks the chain multiplies itself
 constexpr int kTcLone = 4;                // blocks before those that a task takes one by one
-constexpr float kTcRefine = 1024.0f;
+constexpr float tc_refine_limit(int n) { return n <= 1024 ? 128.0f : 1024.0f; }
 constexpr float kTcMaxPart = 0.25e8f;     // a quarter of the growth that one refinement step is good for
 constexpr unsigned long long kXUnset = 0xffffffffffffffffull;
 
@@ -459,6 +468,7 @@ struct TcArgs {
   double* P;
   unsigned* ctrl;
   bool gated;
+  float refine;  // blocks of larger growth are refined
   int* info;
   uint64_t wait_ns;
 };
@@ -689,7 +699,7 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
           ok = exchange_y(acc);
           if (!ok) break;
           double x = times_d(d);
-          if ((growth.x + growth.y) + (growth.z + growth.w) > kTcRefine) {
+          if ((growth.x + growth.y) + (growth.z + growth.w) > a.refine) {
             // x += D (y - T_ss x)
             ok = exchange_y(x);
             if (!ok) break;
@@ -1046,6 +1056,7 @@ static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, c
   a.ctrl = reinterpret_cast<unsigned*>(scratch);
   a.P = reinterpret_cast<double*>(scratch + ctrl_words * sizeof(unsigned));
   a.gated = gated;
+  a.refine = tc_refine_limit(n);
   a.info = info;
   a.wait_ns = wait_timeout_ns();
   const bool one = ncols == 1 && !wide;
