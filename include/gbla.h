@@ -392,8 +392,10 @@ int gbla_bicgstab_solve(int n, const double *A, int lda, const double *b, double
  * d_nrhs (0..4 right-hand sides each; NULL = factor only), d_B (n_i x nrhs_i,
  * overwritten by X), d_ldb, d_info (first zero pivot per system or 0; may be
  * NULL). max_n: an upper bound on the orders (sizes shared memory).
- * ctas_per_sm (0 = as many as fit) is a tuning knob; threads (a multiple of 32,
- * or 0) is checked and otherwise ignored: every CTA has 256.
+ * Tuning knobs: ctas_per_sm (0 = as many as fit), and for max_n > 512 threads (a
+ * multiple of 32 up to 1024, or 0): CTAs of 1024 or 512 threads when it is at least
+ * that, 256 otherwise. Up to max_n = 512 threads is checked only, and the CTA has
+ * 128 threads (max_n <= 128, FP32 up to 256) or 256.
  * ------------------------------------------------------------------------ */
 size_t gbla_lu_batched_workspace(int batch);
 int gbla_lu_solve_batched(int batch, const int *d_n, double *const *d_A, const int *d_lda,

@@ -5,9 +5,10 @@ its launch shape.
 BatchedLU packs the systems into two flat device buffers (column-major
 matrices and right-hand sides), builds the device pointer / size arrays the C
 ABI takes (gbla_lu_solve_batched[_f32], or gbla_chol_solve_batched[_f32] with
-method="chol"), orders the systems largest first and calls the library. The autotuner times the candidate launch shapes (threads
-per CTA x CTAs per SM) on the actual batch and remembers the fastest per GPU,
-dtype and batch profile in a JSON cache.
+method="chol"), orders the systems largest first and calls the library. The autotuner
+times the candidate launch shapes (CTAs per SM, and with orders above 512 threads per
+CTA) on the actual batch and remembers the fastest per GPU, dtype and batch profile in
+a JSON cache.
 """
 import ctypes
 import json
@@ -18,7 +19,9 @@ import torch
 from . import _lib
 from .api import _check, _stream, _ws
 
-CANDIDATES = [(256, c) for c in (0, 1, 2)]  # CTAs per SM; 0: as many as fit
+# (threads, CTAs per SM; 0: as many as fit). The threads count for orders above 512 only.
+CANDIDATES = [(256, c) for c in (0, 1, 2)]
+CANDIDATES_LARGE = [(t, c) for t in (256, 512, 1024) for c in (0, 1, 2)]
 
 
 def _cache_path():
@@ -203,7 +206,7 @@ class BatchedLU:
             self.threads, self.ctas_per_sm = cache[k]["threads"], cache[k]["ctas_per_sm"]
             return cache[k]
         res = {}
-        for t, c in CANDIDATES:
+        for t, c in (CANDIDATES if self.max_n <= 512 else CANDIDATES_LARGE):
             self.restore()
             self.run(t, c)
             times = []

@@ -764,7 +764,7 @@ static int lu_batched_entry(int batch, const int* d_n, T* const* d_A, const int*
   if (!c.ok) return GBLA_ERR_WORKSPACE;
   if (batch == 0) return GBLA_OK;
   GBLA_TRYK(KK_BATCHED, s, launch_lu_batched<T>(batch, d_n, d_A, d_lda, d_ipiv, d_nrhs, d_B, d_ldb, d_info,
-                                              d_order, max_n, ctas_per_sm, counter, solve_only, s));
+                                              d_order, max_n, threads, ctas_per_sm, counter, solve_only, s));
   return GBLA_OK;
 }
 
@@ -843,7 +843,7 @@ static int chol_batched_entry(int batch, const int* d_n, T* const* d_A, const in
   if (!c.ok) return GBLA_ERR_WORKSPACE;
   if (batch == 0) return GBLA_OK;
   GBLA_TRYK(KK_BATCHED, s, launch_chol_batched<T>(batch, d_n, d_A, d_lda, d_nrhs, d_B, d_ldb, d_info,
-                                                d_order, max_n, ctas_per_sm, counter,
+                                                d_order, max_n, threads, ctas_per_sm, counter,
                                                 solve_only, s));
   return GBLA_OK;
 }

@@ -46,11 +46,12 @@ constexpr int kBatchMaxRhs = 4;
 // CTAs per SM the register budget is cut for (256 threads: 3 rather than 2 measured
 // 15.2 against 16.5 ms in FP64 LU and 5.7 against 6.6 ms in FP64 Cholesky, spills included).
 template <typename T>
-constexpr int bt_min_ctas(int nt, int rpt) {
-  return nt == 256 ? 3 : (sizeof(T) == 4 ? 6 : 5);
+constexpr int bt_min_ctas(int nt) {
+  return nt > 256 ? 1024 / nt : nt == 256 ? 3 : (sizeof(T) == 4 ? 6 : 5);
 }
 
 constexpr int kBtW = 16;  // panel width
+constexpr int kBtCap = 512;  // largest order that is factored in panels
 
 // Stride of one column of U in shared memory: 16-byte aligned rows of kBtW
 // values, padded by one vector so that consecutive columns start in other banks.
@@ -593,6 +594,24 @@ __device__ void bt_substitute(const T* a, int ld, int n, int nrhs, T* __restrict
 }
 
 // ---- systems too large for the launch's shared memory: column by column in place
+// c_i -= l_i u for rows i0, i0 + 32, .. < n of one column, by one warp. Bound by the
+// latency of L2: four rows of a lane are loaded before the first is stored.
+template <typename T>
+GBLA_DEVINL void bt_column_update(T* c, const T* l, T u, int i0, int n) {
+  for (int i = i0; i < n; i += 128) {
+    T lv[4], cv[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + 32 * q < n) {
+        lv[q] = l[i + 32 * q];
+        cv[q] = c[i + 32 * q];
+      }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + 32 * q < n) c[i + 32 * q] = fma(-lv[q], u, cv[q]);
+  }
+}
+
 template <typename T, int NT>
 __device__ int bt_lu_in_place(T* a, int ld, int n, int* piv, BtShared<T, NT>& sh) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -641,11 +660,8 @@ __device__ int bt_lu_in_place(T* a, int ld, int n, int* piv, BtShared<T, NT>& sh
     if (rp != (T)0)
       for (int i = j + 1 + tid; i < n; i += NT) a[i + (size_t)j * ld] *= rp;
     __syncthreads();
-    const long long m = n - j - 1;
-    for (long long e = tid; e < m * m; e += NT) {
-      const int i = j + 1 + (int)(e % m), k = j + 1 + (int)(e / m);
-      a[i + (size_t)k * ld] = fma(-a[i + (size_t)j * ld], a[j + (size_t)k * ld], a[i + (size_t)k * ld]);
-    }
+    for (int k = j + 1 + warp; k < n; k += NT / 32)
+      bt_column_update<T>(a + (size_t)k * ld, a + (size_t)j * ld, a[j + (size_t)k * ld], j + 1 + lane, n);
     __syncthreads();
   }
   return info;
@@ -653,7 +669,7 @@ __device__ int bt_lu_in_place(T* a, int ld, int n, int* piv, BtShared<T, NT>& sh
 
 template <typename T, int NT>
 __device__ int bt_chol_in_place(T* a, int ld, int n, BtShared<T, NT>& sh) {
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int j = 0; j < n; ++j) {
     const T d = a[j + (size_t)j * ld];
     if (!(d > (T)0)) return j + 1;  // the same decision in every thread
@@ -662,11 +678,8 @@ __device__ int bt_chol_in_place(T* a, int ld, int n, BtShared<T, NT>& sh) {
     if (tid == 0) a[j + (size_t)j * ld] = l;
     for (int i = j + 1 + tid; i < n; i += NT) a[i + (size_t)j * ld] *= rl;
     __syncthreads();
-    const long long m = n - j - 1;
-    for (long long e = tid; e < m * m; e += NT) {
-      const int i = j + 1 + (int)(e % m), k = j + 1 + (int)(e / m);
-      if (i >= k) a[i + (size_t)k * ld] = fma(-a[i + (size_t)j * ld], a[k + (size_t)j * ld], a[i + (size_t)k * ld]);
-    }
+    for (int k = j + 1 + warp; k < n; k += NT / 32)
+      bt_column_update<T>(a + (size_t)k * ld, a + (size_t)j * ld, a[k + (size_t)j * ld], k + lane, n);
     __syncthreads();
   }
   return 0;
@@ -686,7 +699,7 @@ GBLA_DEVINL int bt_next(int batch, const int* __restrict__ order, unsigned* coun
 // solve_only: the matrices already hold L\U and ipiv the pivots (a previous
 // factor-only launch); only the right-hand sides are solved and written.
 template <typename T, int NT, int RPT>
-__global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT, RPT))
+__global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT))
     batched_lu_kernel(int batch, const int* __restrict__ nv, T* const* __restrict__ Av,
                       const int* __restrict__ ldav, int* const* __restrict__ ipivv,
                       const int* __restrict__ nrhsv, T* const* __restrict__ Bv,
@@ -773,7 +786,7 @@ __global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT, RPT))
 }
 
 template <typename T, int NT, int RPT>
-__global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT, RPT))
+__global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT))
     batched_chol_kernel(int batch, const int* __restrict__ nv, T* const* __restrict__ Av,
                         const int* __restrict__ ldav, const int* __restrict__ nrhsv,
                         T* const* __restrict__ Bv, const int* __restrict__ ldbv,
@@ -834,7 +847,14 @@ __global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT, RPT))
 template <typename T, int NT, int RPT, typename K>
 static cudaError_t bt_shape(K kern, int batch, int max_n, int ctas_per_sm, int* cap, size_t* smem, int* grid) {
   const DeviceProps& dp = device_props();
-  int c = max_n < NT * RPT ? max_n : NT * RPT;
+  constexpr int top = NT * RPT < kBtCap ? NT * RPT : kBtCap;
+  int c = max_n < top ? max_n : top;
+  // with systems that are eliminated in place, the CTAs the caller asks for per SM
+  // are to fit, with panels for what then remains of the shared memory
+  if (max_n > kBtCap && ctas_per_sm > 1) {
+    const int rows = (int)((dp.smem_optin / ctas_per_sm - 4096) / bt_smem_bytes<T>(1));  // at most 32 CTAs
+    if (c > rows) c = rows & ~15;
+  }
   if (c < 32) c = 32;
   c = (c + 3) & ~3;
   *cap = c;
@@ -856,19 +876,22 @@ static cudaError_t bt_shape(K kern, int batch, int max_n, int ctas_per_sm, int* 
 // panel in registers at two rows per thread and runs more of them per SM (LU,
 // orders up to 256: 128 threads 2.28 ms, 256 threads 2.59 ms). FP64 is bound by
 // the FP64 pipe and does not care (15.2 / 15.4 ms); 256 threads keep one row
-// each, with half the registers.
+// each, with half the registers. A batch with larger orders, whose elimination in
+// place is bound by the loads one CTA has in flight, gets the CTA the caller asks for.
 #define GBLA_BT_DISPATCH(RUN)                                        \
   if (max_n <= 128) RUN(128, 1)                                      \
   if (max_n <= 256) {                                                \
     if (sizeof(T) == 4) RUN(128, 2)                                  \
     RUN(256, 1)                                                      \
   }                                                                  \
+  if (max_n > kBtCap && threads >= 1024) RUN(1024, 1)                \
+  if (max_n > kBtCap && threads >= 512) RUN(512, 1)                  \
   RUN(256, 2)
 
 template <typename T>
 cudaError_t launch_lu_batched(int batch, const int* n, T* const* A, const int* lda, int* const* ipiv,
                               const int* nrhs, T* const* B, const int* ldb, int* info,
-                              const int* order, int max_n, int ctas_per_sm, unsigned* counter,
+                              const int* order, int max_n, int threads, int ctas_per_sm, unsigned* counter,
                               bool solve_only, cudaStream_t s) {
   if (batch <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
@@ -892,7 +915,7 @@ cudaError_t launch_lu_batched(int batch, const int* n, T* const* A, const int* l
 template <typename T>
 cudaError_t launch_chol_batched(int batch, const int* n, T* const* A, const int* lda, const int* nrhs,
                                 T* const* B, const int* ldb, int* info, const int* order, int max_n,
-                                int ctas_per_sm, unsigned* counter, bool solve_only, cudaStream_t s) {
+                                int threads, int ctas_per_sm, unsigned* counter, bool solve_only, cudaStream_t s) {
   if (batch <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
@@ -916,10 +939,10 @@ cudaError_t launch_chol_batched(int batch, const int* n, T* const* A, const int*
 #define GBLA_BT_INST(T)                                                                             \
   template cudaError_t launch_lu_batched<T>(int, const int*, T* const*, const int*, int* const*,    \
                                             const int*, T* const*, const int*, int*, const int*,    \
-                                            int, int, unsigned*, bool, cudaStream_t);               \
+                                            int, int, int, unsigned*, bool, cudaStream_t);          \
   template cudaError_t launch_chol_batched<T>(int, const int*, T* const*, const int*, const int*,   \
                                               T* const*, const int*, int*, const int*, int, int,    \
-                                              unsigned*, bool, cudaStream_t);
+                                              int, unsigned*, bool, cudaStream_t);
 GBLA_BT_INST(double)
 GBLA_BT_INST(float)
 #undef GBLA_BT_INST

@@ -261,13 +261,13 @@ cudaError_t launch_rank_k(int m, int n, int k, double alpha, const double* U, in
 template <typename T>
 cudaError_t launch_lu_batched(int batch, const int* n, T* const* A, const int* lda, int* const* ipiv,
                               const int* nrhs, T* const* B, const int* ldb, int* info,
-                              const int* order, int max_n, int ctas_per_sm, unsigned* counter,
-                              bool solve_only, cudaStream_t s);
+                              const int* order, int max_n, int threads, int ctas_per_sm,
+                              unsigned* counter, bool solve_only, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_chol_batched(int batch, const int* n, T* const* A, const int* lda, const int* nrhs,
                                 T* const* B, const int* ldb, int* info, const int* order, int max_n,
-                                int ctas_per_sm, unsigned* counter, bool solve_only, cudaStream_t s);
+                                int threads, int ctas_per_sm, unsigned* counter, bool solve_only, cudaStream_t s);
 
 // ---- Cholesky (chol.cu) ------------------------------------------------------
 // nb: outer block width, a multiple of 64 up to 256 (0: 64)
