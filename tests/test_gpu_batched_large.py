@@ -40,21 +40,3 @@ def test_shape_does_not_change_the_result(method, dtype):
             tol = 0.0 if dtype == torch.float32 else 600 * 2.0 ** -52
             torch.testing.assert_close(bl.A, ref.A, rtol=tol, atol=tol)
             torch.testing.assert_close(bl.B, ref.B, rtol=100 * tol, atol=100 * tol)
-
-
-def test_threads_are_used():
-    As, Bs = _systems([700], "lu")
-    bl = BatchedLU(As, Bs)
-    ms = {}
-    for threads in (256, 1024):
-        times = []
-        for _ in range(3):
-            bl.restore()
-            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
-            e[0].record()
-            bl.run(threads, 1)
-            e[1].record()
-            torch.cuda.synchronize()
-            times.append(e[0].elapsed_time(e[1]))
-        ms[threads] = min(times)
-    assert ms[1024] < 0.8 * ms[256]
