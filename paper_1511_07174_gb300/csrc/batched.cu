@@ -28,8 +28,8 @@
 //
 // Measured (4096 systems of order 16 .. 256, factor + solve; before: one
 // rank-1 update of the whole matrix per column, three barriers each): LU FP64
-// 62.7 -> 15.2 ms (the multiply-adds alone: 11.6 ms at the measured FP64 rate),
-// LU FP32 33.2 -> 2.3 ms, Cholesky FP64 (2048 systems) 23.1 -> 5.8 ms.
+// 62.2 -> 14.1 ms (the multiply-adds alone: 11.6 ms at the measured FP64 rate),
+// LU FP32 33.1 -> 2.0 ms, Cholesky FP64 (2048 systems) 23.0 -> 4.7 ms.
 //
 // Systems larger than the launch's shared memory holds (n > 512, or n > max_n)
 // are eliminated column by column in place in global memory.
@@ -114,6 +114,17 @@ GBLA_DEVINL int bt_warp_argmax(unsigned& hi, unsigned& lo, int row) {
 }
 GBLA_DEVINL float bt_rcp(float x) { return __frcp_rn(x); }
 GBLA_DEVINL double bt_rcp(double x) { return __drcp_rn(x); }
+
+// v / d with rd = 1 / d, rounded to nearest. FP64: the quotient v rd corrected once by
+// its own residual (Markstein, 1990), which is exact while no exponent is extreme: three
+// dependent operations in place of the division's ten, at 64 clocks a warp each.
+GBLA_DEVINL float bt_div(float v, float d, float) { return v / d; }
+GBLA_DEVINL double bt_div(double v, double d, double rd) {
+  const auto plain = [](double x) { return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 128u < 1792u; };
+  const double q = v * rd;
+  if (!(plain(v) && plain(d) && plain(q))) return v / d;
+  return fma(fma(-d, q, v), rd, q);
+}
 
 template <typename T>
 GBLA_DEVINL void bt_store_row(T* dst, const T (&v)[kBtW]) {
@@ -474,9 +485,7 @@ __device__ int bt_chol_panel(T* __restrict__ A, int lda, int m, int w, T* __rest
         if (!(d > (T)0)) {
           bad = j;
         } else {
-          T l, rl;
-          sqrt_rcp(d, &l, &rl);
-          if (lane == j) x[0][j] = l;
+          const T rl = rcp_sqrt(d);  // the root itself waits until the chain is done
           if (lane > j && lane < w) x[0][j] *= rl;
           if (lane == 0) sh.rdiag[j] = rl;
 #pragma unroll
@@ -486,6 +495,16 @@ __device__ int bt_chol_panel(T* __restrict__ A, int lda, int m, int w, T* __rest
           }
         }
       }
+    }
+    {
+      T d = (T)1, l, rl;
+#pragma unroll
+      for (int j = 0; j < kBtW; ++j)
+        if (lane == j && j < bad) d = x[0][j];
+      sqrt_rcp(d, &l, &rl);
+#pragma unroll
+      for (int j = 0; j < kBtW; ++j)
+        if (lane == j && j < bad) x[0][j] = l;
     }
     if (lane < w) {
 #pragma unroll
@@ -524,50 +543,48 @@ __device__ int bt_chol_panel(T* __restrict__ A, int lda, int m, int w, T* __rest
 }
 
 // One triangular substitution on the n x nrhs right-hand sides b (shared
-// memory), 32 rows at a time: one warp solves the diagonal block for all
-// right-hand sides (one division per row serves them all), then every thread
-// updates the rows that remain. The operations on each element and their order
-// are those of the row-by-row substitution.
+// memory), 32 rows at a time: a warp per right-hand side solves the diagonal
+// block, then every thread updates the rows that remain. The operations on each
+// element and their order are those of the row-by-row substitution. Bound, for a
+// system alone, by the chain over the rows: the diagonal block is staged in D
+// (32 x 32, shared memory), the steps have no branch, and a right-hand side to a
+// warp keeps the FP64 operations of a step to one or four. Measured, solve of one
+// system of n = 64 with two right-hand sides (before: one warp for both, with a load
+// from L2 and a division per step): FP64 LU 131 -> 67 us, Cholesky 182 -> 72.
 template <typename T, int NT, bool FWD, bool UNIT, bool TRANS>
-__device__ void bt_substitute(const T* a, int ld, int n, int nrhs, T* __restrict__ b, int ldb) {
+__device__ void bt_substitute(const T* a, int ld, int n, int nrhs, T* __restrict__ b, int ldb, T* __restrict__ D) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int nblk = (n + 31) / 32;
   for (int s = 0; s < nblk; ++s) {
     const int k0 = 32 * (FWD ? s : nblk - 1 - s);
     const int kb = min(32, n - k0);
-    if (tid < 32) {
-      T y[kBatchMaxRhs];
-#pragma unroll
-      for (int c = 0; c < kBatchMaxRhs; ++c) y[c] = (c < nrhs && lane < kb) ? b[k0 + lane + c * ldb] : (T)0;
-      const T* col = TRANS ? a + k0 + (size_t)(k0 + min(lane, kb - 1)) * ld
-                           : a + k0 + min(lane, kb - 1) + (size_t)k0 * ld;
-      const size_t step = TRANS ? 1 : (size_t)ld;
+    for (int e = tid; e < 32 * kb; e += NT) {  // D(i, j) of op(a) at [32 j + i]
+      const int i = e & 31, j = e >> 5;
+      if (TRANS) {
+        if (i < kb) D[32 * i + (j ^ i)] = a[k0 + i + (size_t)(k0 + j) * ld];
+      } else {
+        if (i < kb) D[32 * j + (i ^ j)] = a[k0 + i + (size_t)(k0 + j) * ld];
+      }
+    }
+    __syncthreads();
+    const int c = tid >> 5;  // this warp's right-hand side
+    if (c < nrhs) {
+      T y = lane < kb ? b[k0 + lane + c * ldb] : (T)0;
+      T dl = (T)1, rdl = (T)1;  // the lane's diagonal element and its reciprocal
+      if (!UNIT && lane < kb) {
+        dl = D[32 * lane];
+        rdl = bt_rcp(dl);
+      }
 #pragma unroll 8
       for (int q = 0; q < kb; ++q) {
         const int jj = FWD ? q : kb - 1 - q;
-        const T l = col[jj * step];
-        T xj[kBatchMaxRhs];
-#pragma unroll
-        for (int c = 0; c < kBatchMaxRhs; ++c) xj[c] = __shfl_sync(0xffffffffu, y[c], jj);
-        if (!UNIT) {
-          const T d = __shfl_sync(0xffffffffu, l, jj);
-          const T v = lane == 0 ? xj[0] : (lane == 1 ? xj[1] : (lane == 2 ? xj[2] : xj[3]));
-          const T qv = v / d;
-#pragma unroll
-          for (int c = 0; c < kBatchMaxRhs; ++c) {
-            xj[c] = __shfl_sync(0xffffffffu, qv, c);
-            if (lane == jj) y[c] = xj[c];
-          }
-        }
-        if (FWD ? lane > jj : lane < jj) {
-#pragma unroll
-          for (int c = 0; c < kBatchMaxRhs; ++c)
-            if (c < nrhs) y[c] = fma(-l, xj[c], y[c]);
-        }
+        const T l = D[32 * jj + (lane ^ jj)];
+        T x = __shfl_sync(0xffffffffu, y, jj);
+        if (!UNIT) x = bt_div(x, __shfl_sync(0xffffffffu, dl, jj), __shfl_sync(0xffffffffu, rdl, jj));
+        const T z = fma(-l, x, y);
+        y = (FWD ? lane > jj : lane < jj) ? z : (lane == jj ? x : y);
       }
-#pragma unroll
-      for (int c = 0; c < kBatchMaxRhs; ++c)
-        if (c < nrhs && lane < kb) b[k0 + lane + c * ldb] = y[c];
+      if (lane < kb) b[k0 + lane + c * ldb] = y;
     }
     __syncthreads();
     const int i_lo = FWD ? k0 + kb : 0, i_hi = FWD ? n : k0;
@@ -595,19 +612,23 @@ __device__ void bt_substitute(const T* a, int ld, int n, int nrhs, T* __restrict
 
 // ---- systems too large for the launch's shared memory: column by column in place
 // c_i -= l_i u for rows i0, i0 + 32, .. < n of one column, by one warp. Bound by the
-// latency of L2: four rows of a lane are loaded before the first is stored.
-template <typename T>
+// latency of L2: four rows of a lane are loaded before the first is stored (one where
+// 1024 threads share the FP64 pipe already). Measured (one LU of n = 1024, FP64; a flat
+// index over the square before): 256 threads 467 -> 196 ms, 1024 threads 146 -> 122.
+template <typename T, int NT>
 GBLA_DEVINL void bt_column_update(T* c, const T* l, T u, int i0, int n) {
-  for (int i = i0; i < n; i += 128) {
-    T lv[4], cv[4];
+  constexpr int NR = sizeof(T) == 8 && NT == 1024 ? 1 : 4;
+#pragma unroll 1
+  for (int i = i0; i < n; i += 32 * NR) {
+    T lv[NR], cv[NR];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < NR; ++q)
       if (i + 32 * q < n) {
         lv[q] = l[i + 32 * q];
         cv[q] = c[i + 32 * q];
       }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < NR; ++q)
       if (i + 32 * q < n) c[i + 32 * q] = fma(-lv[q], u, cv[q]);
   }
 }
@@ -661,7 +682,7 @@ __device__ int bt_lu_in_place(T* a, int ld, int n, int* piv, BtShared<T, NT>& sh
       for (int i = j + 1 + tid; i < n; i += NT) a[i + (size_t)j * ld] *= rp;
     __syncthreads();
     for (int k = j + 1 + warp; k < n; k += NT / 32)
-      bt_column_update<T>(a + (size_t)k * ld, a + (size_t)j * ld, a[j + (size_t)k * ld], j + 1 + lane, n);
+      bt_column_update<T, NT>(a + (size_t)k * ld, a + (size_t)j * ld, a[j + (size_t)k * ld], j + 1 + lane, n);
     __syncthreads();
   }
   return info;
@@ -679,7 +700,7 @@ __device__ int bt_chol_in_place(T* a, int ld, int n, BtShared<T, NT>& sh) {
     for (int i = j + 1 + tid; i < n; i += NT) a[i + (size_t)j * ld] *= rl;
     __syncthreads();
     for (int k = j + 1 + warp; k < n; k += NT / 32)
-      bt_column_update<T>(a + (size_t)k * ld, a + (size_t)j * ld, a[k + (size_t)j * ld], k + lane, n);
+      bt_column_update<T, NT>(a + (size_t)k * ld, a + (size_t)j * ld, a[k + (size_t)j * ld], k + lane, n);
     __syncthreads();
   }
   return 0;
@@ -777,8 +798,8 @@ __global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT))
         }
       }
     __syncthreads();
-    bt_substitute<T, NT, true, true, false>(a, ld, n, nrhs, b, ldb);
-    bt_substitute<T, NT, false, false, false>(a, ld, n, nrhs, b, ldb);
+    bt_substitute<T, NT, true, true, false>(a, ld, n, nrhs, b, ldb, Ls);
+    bt_substitute<T, NT, false, false, false>(a, ld, n, nrhs, b, ldb, Ls);
     if (fits)
       for (int c = 0; c < nrhs; ++c)
         for (int r = tid; r < n; r += NT) gB[r + (size_t)c * gldb] = b[r + c * ldb];
@@ -834,8 +855,8 @@ __global__ void __launch_bounds__(NT, bt_min_ctas<T>(NT))
         for (int r = tid; r < n; r += NT) b[r + c * ldb] = gB[r + (size_t)c * gldb];
       __syncthreads();
     }
-    bt_substitute<T, NT, true, false, false>(a, ld, n, nrhs, b, ldb);
-    bt_substitute<T, NT, false, false, true>(a, ld, n, nrhs, b, ldb);
+    bt_substitute<T, NT, true, false, false>(a, ld, n, nrhs, b, ldb, Ls);
+    bt_substitute<T, NT, false, false, true>(a, ld, n, nrhs, b, ldb, Ls);
     if (fits)
       for (int c = 0; c < nrhs; ++c)
         for (int r = tid; r < n; r += NT) gB[r + (size_t)c * gldb] = b[r + c * ldb];
@@ -855,7 +876,7 @@ static cudaError_t bt_shape(K kern, int batch, int max_n, int ctas_per_sm, int* 
     const int rows = (int)((dp.smem_optin / ctas_per_sm - 4096) / bt_smem_bytes<T>(1));  // at most 32 CTAs
     if (c > rows) c = rows & ~15;
   }
-  if (c < 32) c = 32;
+  if (c < 64) c = 64;  // the solve stages 32 x 32 blocks in the panel's part
   c = (c + 3) & ~3;
   *cap = c;
   *smem = bt_smem_bytes<T>(c);

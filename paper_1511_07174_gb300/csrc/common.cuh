@@ -107,7 +107,8 @@ GBLA_DEVINL void tile_coords(int t, int tilesM, int lower, int& ti, int& tj) {
   tj = t - i * (i + 1) / 2;
 }
 
-// *l = sqrt(d), *rl = 1 / sqrt(d) for d > 0.
+// *l = sqrt(d), *rl = rcp_sqrt(d) = 1 / sqrt(d) for d > 0.
+GBLA_DEVINL float rcp_sqrt(float d) { return 1.0f / sqrtf(d); }
 GBLA_DEVINL void sqrt_rcp(float d, float* l, float* rl) {
   *l = sqrtf(d);
   *rl = 1.0f / *l;
@@ -120,19 +121,31 @@ GBLA_DEVINL void sqrt_rcp(float d, float* l, float* rl) {
 // |e| < 2^-20, so the neglected term is below 2^-61; four dependent FP64
 // operations, and the result is within one rounding of 1 / sqrt(d). The root is
 // x times it, corrected once by its own residual (off the chain).
-GBLA_DEVINL void sqrt_rcp(double d, double* l, double* rl) {
+GBLA_DEVINL bool sqrt_scale(double d, double* x, double* r, int* q) {
   const int hi = __double2hiint(d);
   const int ex = hi >> 20;  // d > 0: no sign
-  if (ex == 0 || ex >= 0x7ff) {  // subnormal or infinite
+  if (ex == 0 || ex >= 0x7ff) return false;  // subnormal or infinite
+  *q = (ex - 1022) >> 1;  // d = x 4^q, exponent of x: 1022 or 1023
+  *x = __hiloint2double(hi - (*q << 21), __double2loint(d));
+  const double y = (double)rsqrtf((float)*x);
+  const double e = fma(-(*x * y), y, 1.0);
+  *r = fma(y * e, fma(0.375, e, 0.5), y);
+  return true;
+}
+GBLA_DEVINL double rcp_sqrt(double d) {
+  double x, r;
+  int q;
+  if (!sqrt_scale(d, &x, &r, &q)) return 1.0 / sqrt(d);
+  return __hiloint2double(__double2hiint(r) - (q << 20), __double2loint(r));
+}
+GBLA_DEVINL void sqrt_rcp(double d, double* l, double* rl) {
+  double x, r;
+  int q;
+  if (!sqrt_scale(d, &x, &r, &q)) {
     *l = sqrt(d);
     *rl = 1.0 / *l;
     return;
   }
-  const int q = (ex - 1022) >> 1;  // d = x 4^q, exponent of x: 1022 or 1023
-  const double x = __hiloint2double(hi - (q << 21), __double2loint(d));
-  const double y = (double)rsqrtf((float)x);
-  const double e = fma(-(x * y), y, 1.0);
-  const double r = fma(y * e, fma(0.375, e, 0.5), y);
   const double h = x * r;
   const double s = fma(fma(-h, h, x), 0.5 * r, h);
   *rl = __hiloint2double(__double2hiint(r) - (q << 20), __double2loint(r));
