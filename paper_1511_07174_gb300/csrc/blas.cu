@@ -614,7 +614,8 @@ cudaError_t launch_copy_d2f(const double* A, int lda, float* F, int ldf, int m, 
 // value from. It depends on the chunk's interchanges alone, so one CTA per chunk
 // works it out (about 5 us each); one CTA then applies the plans in order to the
 // running permutation (every read before any write), which lives in shared memory
-// when it fits, else in perm itself. Measured: n = 4096 87 -> 15 us.
+// when it fits, else in perm itself. Measured: n = 4096 87 -> 15 us. The plan of a
+// single chunk is the permutation.
 __global__ void __launch_bounds__(256)
     perm_plan_kernel(int n, const int* __restrict__ ipiv, int* __restrict__ plan) {
   __shared__ SwapPlanShared s_plan;
@@ -629,6 +630,7 @@ __global__ void __launch_bounds__(256)
   swap_plan(s_plan, kb, t, &src_b, &dst_o, &src_o);
   if (t < kb) {
     plan[c0 + t] = src_b;
+    if (gridDim.x == 1) return;
     plan[n + c0 + t] = dst_o;
     plan[2 * (size_t)n + c0 + t] = src_o;
   }
@@ -678,6 +680,11 @@ cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, void* scratch
   if (n <= 0) return cudaSuccess;
   if (!ipiv) {  // no interchanges: the identity
     iota_kernel<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, s>>>(n, perm);
+    count_launch();
+    return cudaGetLastError();
+  }
+  if (n <= 256) {
+    perm_plan_kernel<<<1, 256, 0, s>>>(n, ipiv, perm);
     count_launch();
     return cudaGetLastError();
   }
