@@ -296,7 +296,8 @@ int gbla_gmresir_solve(int n, const double *A, int lda, const float *F, int ldf,
 /* The same refinement for nrhs right-hand sides (B, X: n x nrhs, ldb, ldx),
  * sharing one set-up of the factors (pivot permutation, inverted diagonal
  * blocks) and one workspace; each column is refined on its own, with its own
- * entry of stats[0 .. nrhs). Up to four columns share the launches of an
+ * entry of stats[0 .. nrhs) and, bit for bit, the result of a call for it alone,
+ * whatever nrhs and work_bytes are. Up to four columns share the launches of an
  * iteration: as many as the workspace has room for, at least
  * gbla_gmresir_workspace(n, restart_m), for four of them
  * gbla_gmresir_workspace_nrhs(n, nrhs, restart_m).

@@ -1036,19 +1036,18 @@ size_t gbla_gmresir_workspace_nrhs(int n, int nrhs, int restart_m) {
 }
 
 // dst <- M^{-1} src with M = P^t L U (FP32 factors, FP64 arithmetic, inverted
-// 64 x 64 diagonal blocks of L and U formed once per solve call), k columns of a
-// call that refines up to `cols` together; t1, t2: n x k temporaries; src and dst
-// distinct
+// 64 x 64 diagonal blocks of L and U formed once per solve call), k columns; t1,
+// t2: n x k temporaries; src and dst distinct
 static cudaError_t apply_minv(int n, const float* F, int ldf, const int* perm, const double* DinvL,
                               const double* DinvU, const double* src, double* dst, double* t1,
-                              double* t2, void* flags, int* info, cudaStream_t s, int k = 1, int cols = 1,
+                              double* t2, void* flags, int* info, cudaStream_t s, int k = 1,
                               int lds = 0, int ldd = 0) {
   cudaError_t e;
   PROF(KK_PERM, s, launch_permute_rows(n, k, perm, false, src, lds ? lds : n, t1, n, s));
   if (e != cudaSuccess) return e;
-  PROF(KK_TRSV, s, launch_trsv_inv(true, n, k, cols, F, ldf, DinvL, t1, n, t2, n, flags, info, s));
+  PROF(KK_TRSV, s, launch_trsv_inv(true, n, k, F, ldf, DinvL, t1, n, t2, n, flags, info, s));
   if (e != cudaSuccess) return e;
-  PROF(KK_TRSV, s, launch_trsv_inv(false, n, k, cols, F, ldf, DinvU, t2, n, dst, ldd ? ldd : n, flags, info, s));
+  PROF(KK_TRSV, s, launch_trsv_inv(false, n, k, F, ldf, DinvU, t2, n, dst, ldd ? ldd : n, flags, info, s));
   return e;
 }
 
@@ -1090,7 +1089,9 @@ static int check_ir_opts(const gbla_gmresir_opts* o) {
 // The columns advance together, each with its own basis, Hessenberg matrix and
 // stopping tests; a launch covers the columns from the first to the last one that
 // still needs it, and what it computes for one in between that does not (a next
-// basis vector, the column of H after its last) is not used.
+// basis vector, the column of H after its last) is not used. Every launch does the
+// same operations in the same order on a column whatever columns it covers, so a
+// column's result is that of its own call, bit for bit.
 static int gmresir_group(int n, int cols, const double* A, int lda, const float* F, int ldf, const double* B, int ldb,
                          double* X, int ldx, const gbla_gmresir_opts* opts, gbla_gmresir_stats* stats,
                          const IrWork& w, cudaStream_t s) {
@@ -1110,7 +1111,7 @@ static int gmresir_group(int n, int cols, const double* A, int lda, const float*
   // dst <- M^{-1} src, columns of scratch
   auto minv = [&](Range r, double* src, double* dst) {
     return apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, col(src, r.lo), col(dst, r.lo), w.t1, w.t2, w.flags, w.info, s,
-                      r.k, cols);
+                      r.k);
   };
   auto mgs = [&](Range r, int j, double* v) {
     const int c = r.lo;
@@ -1119,7 +1120,7 @@ static int gmresir_group(int n, int cols, const double* A, int lda, const float*
                            w.slots + c * mgs_slots_doubles(), w.counter + c, w.info, s, r.k, w.vstride, n, hs);
   };
   for (int c = 0; c < cols; ++c) memset(&stats[c], 0, sizeof(stats[c]));
-  GBLA_TRY(apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, B, X, w.t1, w.t2, w.flags, w.info, s, cols, cols, ldb, ldx));
+  GBLA_TRY(apply_minv(n, F, ldf, w.perm, w.DinvL, w.DinvU, B, X, w.t1, w.t2, w.flags, w.info, s, cols, ldb, ldx));
   bool live[kIrCols], cyc_on[kIrCols], it_on[kIrCols];
   double beta[kIrCols], res[kIrCols], znorm[kIrCols] = {};
   int k[kIrCols];

@@ -192,11 +192,11 @@ size_t trsv_scratch_bytes(int n, int nrhs);
 // blocks of a triangular factor, formed once per set of factors ...
 size_t diag_inv_doubles(int n);
 cudaError_t launch_diag_inv(bool lower, bool unit, int n, const float* T, int ldt, double* D, cudaStream_t s);
-// ... and X <- T^{-1} rhs with them, nrhs columns (X and rhs distinct; scratch:
-// trsv_scratch_bytes(n, cols)). A call with cols > 1 takes the same operations
-// in the same order for any nrhs <= cols.
-cudaError_t launch_trsv_inv(bool lower, int n, int nrhs, int cols, const float* T, int ldt, const double* D,
-                            const double* rhs, int ldr, double* X, int ldx, void* scratch, int* info, cudaStream_t s);
+// ... and X <- T^{-1} rhs with them, at most four columns (X and rhs distinct;
+// scratch: trsv_scratch_bytes(n, nrhs)). The result for a column does not depend on
+// the others.
+cudaError_t launch_trsv_inv(bool lower, int n, int nrhs, const float* T, int ldt, const double* D, const double* rhs,
+                            int ldr, double* X, int ldx, void* scratch, int* info, cudaStream_t s);
 
 // ipiv == nullptr: the identity. scratch: 3 n ints.
 cudaError_t launch_ipiv_to_perm(int n, const int* ipiv, int* perm, void* scratch, cudaStream_t s);

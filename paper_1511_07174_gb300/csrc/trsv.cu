@@ -216,8 +216,9 @@ __global__ void __launch_bounds__(256)
 // while, so a chain finishes even if no other CTA of the grid is ever scheduled
 // beside it. All waits are bounded.
 //
-// The operations and their order depend on n alone: for a given factor this is a
-// fixed linear map of rhs (as GMRES requires), whatever CTAs do the tasks.
+// The operations on a right-hand side and their order depend on n alone: for a given
+// factor this is a fixed linear map of rhs (as GMRES requires), whatever CTAs do the
+// tasks and whatever other right-hand sides share the launch.
 //
 // Accuracy. With g = || |D||T_ss| || the product x_s = D_s y_s leaves a residual of
 // up to g u |T_ss||x_s| where a substitution leaves u |T_ss||x_s|. g is a few hundred
@@ -497,6 +498,8 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
   constexpr int kRows = kTsBS / CL / kTcWarps;  // rows of every block per chain warp
   constexpr int kGrp = 32 / kRows;              // lanes that share a row
   constexpr int kCols = kTsBS / kGrp;           // columns of a block per lane
+  constexpr int kAcc = 16 / kGrp;               // of the 16 sums of a row (column mod 16) a lane's
+  static_assert(kAcc == 1 || kAcc == 2, "clusters of 8 or 4");
   constexpr int kOwn = kTsBS / CL;              // rows of every block per CTA
   __shared__ double s_x[2][NR][kTsBS];        // x_s, by parity of s
   __shared__ double s_y[2][NR][kTsBS];        // y_s
@@ -642,25 +645,28 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
           ++ny;
           return true;
         };
-        auto row_sum = [&](double v) {
+        // The 16 sums of a row, added in one order whatever the cluster's size: h and h + 8
+        // first (one lane's two, or two lanes'), then the bits of h from the lowest.
+        auto row_sum = [&](const double (&p)[kAcc]) {
+          double v = p[0] + (kAcc == 2 ? p[kAcc - 1] : __shfl_xor_sync(0xffffffffu, p[0], 16));
 #pragma unroll
-          for (int o = kRows; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          for (int o = kRows; o < 8 * kRows; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
           return v;
         };
         auto times_d = [&](double (&dd)[kCols]) {  // D_s times what the last exchange brought
           const double* yv = s_y[(ny - 1) & 1][c];
-          double v = 0.0;
+          double v[kAcc] = {};
 #pragma unroll
-          for (int j = 0; j < kCols; ++j) v = fma(dd[j], yv[grp + kGrp * j], v);
+          for (int j = 0; j < kCols; ++j) v[j % kAcc] = fma(dd[j], yv[grp + kGrp * j], v[j % kAcc]);
           return row_sum(v);
         };
         for (int s = 0; s < nblk; ++s) {
           // every operand is loaded for the next step as soon as this one has used it
           const int par = s & 1;
-          double acc = 0.0;
+          double part[kAcc] = {};
           if (s >= 2) {
 #pragma unroll
-            for (int j = 0; j < kCols; ++j) acc = fma(-to_f64(t2[j]), s_x[par][c][grp + kGrp * j], acc);
+            for (int j = 0; j < kCols; ++j) part[j % kAcc] = fma(-to_f64(t2[j]), s_x[par][c][grp + kGrp * j], part[j % kAcc]);
           }
           load_t(s + 1, 2, t2);
           if (wr == 0 && lane == 0) s_step[c] = s;
@@ -682,7 +688,7 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
             if (told && lane == 0) s_stuck[c] = 0;
             if (!ok) break;
           }
-          if (grp == 0) acc += s_y0[s % kTcRing][c][ro];
+          if (grp == 0) part[0] += s_y0[s % kTcRing][c][ro];
           if (s >= 1) {
             const uint32_t bar = cl_smem_u32(&s_bar[0][par ^ 1][c]);
             ok = cl_mbar_wait(bar, (uint32_t)((s - 1) >> 1) & 1u, a.wait_ns);
@@ -692,9 +698,10 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
             }
             if (wr == 0 && lane == 0) cl_mbar_arm(bar, kTsBS * 8);
 #pragma unroll
-            for (int j = 0; j < kCols; ++j) acc = fma(-to_f64(t1[j]), s_x[par ^ 1][c][grp + kGrp * j], acc);
+            for (int j = 0; j < kCols; ++j)
+              part[j % kAcc] = fma(-to_f64(t1[j]), s_x[par ^ 1][c][grp + kGrp * j], part[j % kAcc]);
           }
-          acc = row_sum(acc);
+          const double acc = row_sum(part);
           load_t(s + 1, 1, t1);
           ok = exchange_y(acc);
           if (!ok) break;
@@ -705,15 +712,16 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
             if (!ok) break;
             const int b0 = (a.fwd ? s : nblk - 1 - s) * kTsBS, r = b0 + rb;
             const double* xv = s_y[(ny - 1) & 1][c];
-            double res = grp == 0 ? acc : 0.0;
+            double rp[kAcc] = {};
+            if (grp == 0) rp[0] = acc;
+#pragma unroll
             for (int j = 0; j < kCols; ++j) {
               const int cc = grp + kGrp * j, gc = b0 + cc;
               if (r >= n || gc >= n || (a.fwd ? cc > rb : cc < rb)) continue;
               const double tv = cc == rb && a.unit ? 1.0 : (double)(TRANS ? T[gc + (size_t)r * a.ldt] : T[r + (size_t)gc * a.ldt]);
-              res = fma(-tv, xv[cc], res);
+              rp[j % kAcc] = fma(-tv, xv[cc], rp[j % kAcc]);
             }
-            res = row_sum(res);
-            ok = exchange_y(res);
+            ok = exchange_y(row_sum(rp));
             if (!ok) break;
             x += times_d(d);
           }
@@ -1037,8 +1045,8 @@ static cudaError_t tc_launch_diag_inv(bool fwd, bool unit, int n, const Ts* T, i
 // that says whether the inverses are safe is left as it is.
 template <typename Ts, bool TRANS>
 static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, const Ts* T, int ldt, const double* D, const double* rhs,
-                            int ldr, double* X, int ldx, char* scratch, size_t ctrl_words, bool gated, bool wide,
-                            int* info, cudaStream_t s) {
+                            int ldr, double* X, int ldx, char* scratch, size_t ctrl_words, bool gated, int* info,
+                            cudaStream_t s) {
   TcArgs a;
   a.n = n;
   a.nblk = (n + kTsBS - 1) / kTsBS;
@@ -1059,7 +1067,7 @@ static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, c
   a.refine = tc_refine_limit(n);
   a.info = info;
   a.wait_ns = wait_timeout_ns();
-  const bool one = ncols == 1 && !wide;
+  const bool one = ncols == 1;
   if constexpr (sizeof(Ts) == 4) {
     if (n > kTcRoomy && sh.G == 1)
       return one ? tc_launch_solve<Ts, TRANS, 1, 8, 128>(T, a, s) : tc_launch_solve<Ts, TRANS, 1, 4, 128>(T, a, s);
@@ -1120,8 +1128,8 @@ cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, cons
                   : tc_launch_diag_inv<double, false>(fwd, unit, n, T, ldt, D, ctrl + kTcMaxC, s);
         if (e != cudaSuccess) return e;
       }
-      e = trans ? tc_apply<double, true>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, nrhs > 1, info, s)
-                : tc_apply<double, false>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, nrhs > 1, info, s);
+      e = trans ? tc_apply<double, true>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s)
+                : tc_apply<double, false>(fwd, unit, n, ncols, sh, T, ldt, D, R, ldr, Xc, ldx, sc, cw, true, info, s);
       if (e != cudaSuccess) return e;
     }
     const int C = trsv_chains(ncols);
@@ -1156,16 +1164,16 @@ cudaError_t launch_diag_inv(bool lower, bool unit, int n, const float* T, int ld
 
 // ... and X = T^-1 rhs (at most kTcMaxC columns, distinct buffers) as a fixed
 // linear map
-cudaError_t launch_trsv_inv(bool lower, int n, int nrhs, int cols, const float* T, int ldt, const double* D,
-                            const double* rhs, int ldr, double* X, int ldx, void* scratch, int* info, cudaStream_t s) {
+cudaError_t launch_trsv_inv(bool lower, int n, int nrhs, const float* T, int ldt, const double* D, const double* rhs,
+                            int ldr, double* X, int ldx, void* scratch, int* info, cudaStream_t s) {
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
-  if (nrhs > cols || cols > kTcMaxC) return cudaErrorInvalidValue;
-  const size_t cw = tc_ctrl_words(n, cols);
+  if (nrhs > kTcMaxC) return cudaErrorInvalidValue;
+  const size_t cw = tc_ctrl_words(n, nrhs);
   const TcShape sh = tc_shape(nrhs);
   char* sc = static_cast<char*>(scratch);
   cudaError_t e = tc_fill(n, nrhs, sh, X, ldx, sc, cw, false, s);
   if (e != cudaSuccess) return e;
-  return tc_apply<float, false>(lower, false, n, nrhs, sh, T, ldt, D, rhs, ldr, X, ldx, sc, cw, false, cols > 1, info, s);
+  return tc_apply<float, false>(lower, false, n, nrhs, sh, T, ldt, D, rhs, ldr, X, ldx, sc, cw, false, info, s);
 }
 
 }  // namespace gbla
