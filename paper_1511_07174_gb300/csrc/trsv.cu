@@ -688,6 +688,7 @@ __global__ void __launch_bounds__(H == 128 ? 320 : tc_threads<NR, H>(), H == 128
             if (told && lane == 0) s_stuck[c] = 0;
             if (!ok) break;
           }
+          __threadfence_block();  // s_have before s_y0, as they were written
           if (grp == 0) part[0] += s_y0[s % kTcRing][c][ro];
           if (s >= 1) {
             const uint32_t bar = cl_smem_u32(&s_bar[0][par ^ 1][c]);
