@@ -438,7 +438,7 @@ def fma_peak(precision="fp64", iters=1 << 16):
 # ------------------------------------------------------------------ autotuning
 def _tune_nb(kind, n, candidates, run, device, use_cache):
     from . import batched as _b
-    key = "%s_nb|%s|%d" % (kind, torch.cuda.get_device_name(device), n)
+    key = "%s_nb|%s|%d|k%d" % (kind, torch.cuda.get_device_name(device), n, _b.TUNED_KERNELS)
     cache = _b._load_cache() if use_cache else {}
     if key in cache:
         return cache[key]["nb"]

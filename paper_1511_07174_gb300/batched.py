@@ -23,6 +23,10 @@ from .api import _check, _stream, _ws
 CANDIDATES = [(256, c) for c in (0, 1, 2)]
 CANDIDATES_LARGE = [(t, c) for t in (256, 512, 1024) for c in (0, 1, 2)]
 
+# Part of every key of the cache: raised when the kernels that are timed or their candidates
+# change, so that a choice made for others is not taken over.
+TUNED_KERNELS = 2
+
 
 def _cache_path():
     base = os.environ.get("GBLA_CACHE") or os.path.join(
@@ -196,7 +200,7 @@ class BatchedLU:
     def key(self):
         name = torch.cuda.get_device_name(self.device)
         prof = (self.batch, min(self.sizes, default=0), self.max_n, sum(n ** 3 for n in self.sizes) // (1 << 20))
-        return "%s|%s|%s|%d|%d|%d|%d" % ((name, self.method, str(self.dtype)) + prof)
+        return "%s|%s|%s|%d|%d|%d|%d|k%d" % ((name, self.method, str(self.dtype)) + prof + (TUNED_KERNELS,))
 
     def autotune(self, reps=2, use_cache=True):
         """Time every candidate (threads, CTAs per SM) on this batch; keep the fastest."""
