@@ -158,7 +158,8 @@ int gbla_fma_peak(int precision, int iters, double *tflops, gbla_stream_t stream
  *   lda    leading dimension (>= max(1, n))
  *   ipiv   n ints, output pivots (1-based)
  *   d_info one int, output (see conventions); set to 0 by the call
- *   nb     block size in [32, 256], multiple of 32; 0 = default (128)
+ *   nb     block size in [32, 256], multiple of 32; 0 = default: 128, or 256 when
+ *          d_work has room for that one's scratch only
  * ------------------------------------------------------------------------ */
 size_t gbla_lu_factor_workspace(int n, int nb);
 /* The scratch with which gbla_lu_factor does its trailing updates on the
@@ -193,7 +194,8 @@ int gbla_lu_factor(int n, double *A, int lda, int *ipiv, int *d_info, int nb,
  *   (each call clears it before use): calls whose work overlaps on the GPU --
  *   on different streams, or from different host threads -- race with each
  *   other and must be serialised by the caller.
- * Arguments and d_info as for gbla_lu_factor.
+ * Arguments and d_info as for gbla_lu_factor; nb = 0 is 256 here, and every
+ * trailing update runs on the FP64 pipe.
  */
 int gbla_lu_factor_static(int n, double *A, int lda, int *ipiv, int *d_info, int nb,
                           gbla_stream_t stream);

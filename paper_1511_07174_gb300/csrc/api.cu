@@ -543,6 +543,7 @@ int gbla_lu_factor(int n, double* A, int lda, int* ipiv, int* d_info, int nb, vo
   if (lda < std::max(1, n)) return -3;
   if (n > 0 && !ipiv) return -4;
   if (!d_info) return -5;
+  const bool any_nb = nb == 0;
   nb = check_nb_f64(nb);
   if (nb < 0) return -6;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -550,6 +551,11 @@ int gbla_lu_factor(int n, double* A, int lda, int* ipiv, int* d_info, int nb, vo
   Carver c(d_work, work_bytes);
   LuWork w;
   lu_work_layout(c, n, nb, 0, &w);
+  if (!c.ok && any_nb) {  // wider blocks need less
+    nb = 256;
+    c = Carver(d_work, work_bytes);
+    lu_work_layout(c, n, nb, 0, &w);
+  }
   if (!c.ok) return GBLA_ERR_WORKSPACE;
   // room for the digits: the trailing update runs on the tensor cores
   if (lu_uses_digits(nb) && n > nb) digits_layout(c, n, nb, true, &w.dig);
