@@ -485,7 +485,9 @@ __device__ int bt_chol_panel(T* __restrict__ A, int lda, int m, int w, T* __rest
         if (!(d > (T)0)) {
           bad = j;
         } else {
-          const T rl = rcp_sqrt(d);  // the root itself waits until the chain is done
+          T l, rl;
+          sqrt_rcp(d, &l, &rl);
+          if (lane == j) x[0][j] = l;
           if (lane > j && lane < w) x[0][j] *= rl;
           if (lane == 0) sh.rdiag[j] = rl;
 #pragma unroll
@@ -495,16 +497,6 @@ __device__ int bt_chol_panel(T* __restrict__ A, int lda, int m, int w, T* __rest
           }
         }
       }
-    }
-    {
-      T d = (T)1, l, rl;
-#pragma unroll
-      for (int j = 0; j < kBtW; ++j)
-        if (lane == j && j < bad) d = x[0][j];
-      sqrt_rcp(d, &l, &rl);
-#pragma unroll
-      for (int j = 0; j < kBtW; ++j)
-        if (lane == j && j < bad) x[0][j] = l;
     }
     if (lane < w) {
 #pragma unroll

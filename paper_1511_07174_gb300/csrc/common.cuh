@@ -107,48 +107,40 @@ GBLA_DEVINL void tile_coords(int t, int tilesM, int lower, int& ti, int& tj) {
   tj = t - i * (i + 1) / 2;
 }
 
-// *l = sqrt(d), *rl = rcp_sqrt(d) = 1 / sqrt(d) for d > 0.
-GBLA_DEVINL float rcp_sqrt(float d) { return 1.0f / sqrtf(d); }
+// *l = sqrt(d), *rl = 1 / *l for d > 0.
 GBLA_DEVINL void sqrt_rcp(float d, float* l, float* rl) {
   *l = sqrtf(d);
   *rl = 1.0f / *l;
 }
 // FP64: sqrt followed by a division is a chain of some twenty dependent FP64
 // operations per column, at the latency this GPU's FP64 pipe has. Instead, d is
-// scaled by a power of four to x in [1/2, 2), 1 / sqrt(x) comes from the FP32
-// approximation y and one third-order step of the series
-//   x^-1/2 = y (1 - e)^-1/2 = y (1 + e/2 + 3/8 e^2 + O(e^3)),  e = 1 - x y^2,
-// |e| < 2^-20, so the neglected term is below 2^-61; four dependent FP64
-// operations, and the result is within one rounding of 1 / sqrt(d). The root is
-// x times it, corrected once by its own residual (off the chain).
-GBLA_DEVINL bool sqrt_scale(double d, double* x, double* r, int* q) {
+// scaled by a power of four to x in [1/2, 2); with the FP32 approximation y of
+// 1 / sqrt(x) and e = 1 - x y^2, |e| < 2^-20, one third-order step of the series
+//   (1 - e)^-1/2 = 1 + e/2 + 3/8 e^2 + O(e^3)
+// takes y to 1 / sqrt(x) and x y to sqrt(x), side by side, the neglected term below
+// 2^-61. The root is then corrected by its residual, and the reciprocal by its
+// product with the root as rounded: it is the reciprocal of that root, not of
+// sqrt(d), so that a column scaled with it leaves the residual that one divided by
+// the root leaves (with 1 / sqrt(d) rounded on its own, 1.2 times that, rms).
+GBLA_DEVINL void sqrt_rcp(double d, double* l, double* rl) {
   const int hi = __double2hiint(d);
   const int ex = hi >> 20;  // d > 0: no sign
-  if (ex == 0 || ex >= 0x7ff) return false;  // subnormal or infinite
-  *q = (ex - 1022) >> 1;  // d = x 4^q, exponent of x: 1022 or 1023
-  *x = __hiloint2double(hi - (*q << 21), __double2loint(d));
-  const double y = (double)rsqrtf((float)*x);
-  const double e = fma(-(*x * y), y, 1.0);
-  *r = fma(y * e, fma(0.375, e, 0.5), y);
-  return true;
-}
-GBLA_DEVINL double rcp_sqrt(double d) {
-  double x, r;
-  int q;
-  if (!sqrt_scale(d, &x, &r, &q)) return 1.0 / sqrt(d);
-  return __hiloint2double(__double2hiint(r) - (q << 20), __double2loint(r));
-}
-GBLA_DEVINL void sqrt_rcp(double d, double* l, double* rl) {
-  double x, r;
-  int q;
-  if (!sqrt_scale(d, &x, &r, &q)) {
+  if (ex == 0 || ex >= 0x7ff) {  // subnormal or infinite
     *l = sqrt(d);
     *rl = 1.0 / *l;
     return;
   }
-  const double h = x * r;
+  const int q = (ex - 1022) >> 1;  // d = x 4^q, exponent of x: 1022 or 1023
+  const double x = __hiloint2double(hi - (q << 21), __double2loint(d));
+  const double y = (double)rsqrtf((float)x);
+  const double g = x * y;
+  const double e = fma(-g, y, 1.0);
+  const double p = fma(0.375, e, 0.5);
+  const double r = fma(y * e, p, y);
+  const double h = fma(g * e, p, g);
   const double s = fma(fma(-h, h, x), 0.5 * r, h);
-  *rl = __hiloint2double(__double2hiint(r) - (q << 20), __double2loint(r));
+  const double t = fma(r, fma(-s, r, 1.0), r);
+  *rl = __hiloint2double(__double2hiint(t) - (q << 20), __double2loint(t));
   *l = __hiloint2double(__double2hiint(s) + (q << 20), __double2loint(s));
 }
 
