@@ -232,14 +232,23 @@ __global__ void __launch_bounds__(128)
   __syncthreads();
   if (tid < kCholNb) rdiag[tid] = (T)1 / Ls[tid][tid];
   __syncthreads();
+  // What the first 32 columns give the others is summed on its own and subtracted
+  // once: half as many roundings at the size of the elements.
+  constexpr int kHalf = kCholNb / 8;
+  T acc[kHalf] = {};
 #pragma unroll
   for (int j = 0; j < kCholNb; ++j) {
+    if (j == kCholNb / 2) {
+#pragma unroll
+      for (int t = 0; t < kHalf; ++t) x[kHalf + t] -= acc[t];
+    }
     const T xj = __shfl_sync(0xffffffffu, x[j / 4], (lane & 7) + 8 * (j & 3)) * rdiag[j];
     if (g == (j & 3)) x[j / 4] = xj;
 #pragma unroll
     for (int t = j / 4; t < kCholNb / 4; ++t) {
       const int k = g + 4 * t;
-      if (t > j / 4) x[t] = fma(-xj, Ls[k][j], x[t]);
+      if (j < kCholNb / 2 && t >= kHalf) acc[t - kHalf] = fma(xj, Ls[k][j], acc[t - kHalf]);
+      else if (t > j / 4) x[t] = fma(-xj, Ls[k][j], x[t]);
       else if (k > j) x[t] = fma(-xj, Ls[k][j], x[t]);
     }
   }
