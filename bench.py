@@ -664,6 +664,15 @@ def chol_mixed_vs_fp64(n, args):
             "workload": "A = B B^t/n + I (B iid N(0,1), product in FP32), x_true N(0,1), fp16x3 update"}
 
 
+def digit_products(tflops, on_tensor_cores, pk):
+    """The BF16 products an FP64 factorisation at this rate executes, and their share of the measured
+    BF16 peak: its trailing updates take 35 products of digits per multiply-add."""
+    if not on_tensor_cores:
+        return {}
+    return {"bf16_products_tflops": 35 * tflops,
+            "frac_of_bf16_peak": 35 * tflops / pk["bf16_tflops"] if pk.get("bf16_tflops") else None}
+
+
 def secondary(args, pk):
     """The other measured workloads of the solver (one GPU): FP64 LU n = 512 and
     n = 8192 (16 RHS, block size autotuned), FP64 Cholesky n = 8192, the batched
@@ -712,8 +721,8 @@ def secondary(args, pk):
     X = api.lu_solve(LU, piv, B)
     beta = float(api.backward_error(A, X, B).max().item())
     tf = lu_flops(n) / (ms_f * 1e-3) / 1e12
-    out["lu_n8192_fp64"] = {"nb": nb, "factor_ms": ms_f, "tflops": tf, "frac_of_fp64_dgemm": tf / fp64_peak,
-                            "frac_of_fp64_fma_peak": tf / fma64,
+    out["lu_n8192_fp64"] = {"nb": nb, "factor_ms": ms_f, "tflops": tf, "times_fp64_dgemm": tf / fp64_peak,
+                            **digit_products(tf, nb % 128 == 0, pk),
                             "solve16_ms": ms_s,
                             "solve_gbs": (n * n * 8) / (ms_s * 1e-3) / 1e9, "beta_max": beta}
     del LU, X
@@ -726,8 +735,8 @@ def secondary(args, pk):
     ms_c = _event_ms(lambda: api.chol_factor(S, nb=nbc))
     Xc = api.chol_solve(F, Bs)
     tfc = n ** 3 / 3.0 / (ms_c * 1e-3) / 1e12
-    out["chol_n8192_fp64"] = {"nb": nbc, "factor_ms": ms_c, "tflops": tfc, "frac_of_fp64_dgemm": tfc / fp64_peak,
-                              "frac_of_fp64_fma_peak": tfc / fma64,
+    out["chol_n8192_fp64"] = {"nb": nbc, "factor_ms": ms_c, "tflops": tfc, "times_fp64_dgemm": tfc / fp64_peak,
+                              **digit_products(tfc, True, pk),
                               "beta_max": float(api.backward_error(S, Xc, Bs).max().item())}
     del S, F, Xc, A, B
     # mixed-precision Cholesky + GMRES-IR against the FP64 Cholesky, SPD n = 16384

@@ -164,12 +164,14 @@ int gbla_fma_peak(int precision, int iters, double *tflops, gbla_stream_t stream
 size_t gbla_lu_factor_workspace(int n, int nb);
 /* The scratch with which gbla_lu_factor does its trailing updates on the
  * tensor cores: gbla_lu_factor_workspace(n, nb) plus, when nb is a multiple of
- * 128, 8 bytes per element of two n x nb operands in 8-bit digits and their
- * scales. The operands are split exactly to 2^-55 of a row's largest magnitude
- * and multiplied exactly, and tiles for which that would be less accurate than
- * FP64 multiply-adds are done by those. Any work_bytes from
- * gbla_lu_factor_workspace up is accepted; below this size every update runs
- * on the FP64 pipe. */
+ * 128, 16 bytes per element of two n x nb operands (eight slices of 8-bit
+ * digits) and their scales. The operands are rounded to 2^-55 of the largest
+ * magnitude of their row (A) or column (B) and written in seven digits; of the
+ * 49 products of digits the 34 of the largest weights are formed and summed, and
+ * the sum is rounded once, at 2^-52 of the product of those two magnitudes.
+ * Tiles for which that would be less accurate than FP64 multiply-adds are
+ * done by those. Any work_bytes from gbla_lu_factor_workspace up is accepted;
+ * below this size, and for any other nb, every update runs on the FP64 pipe. */
 size_t gbla_lu_factor_workspace_tensor(int n, int nb);
 int gbla_lu_factor(int n, double *A, int lda, int *ipiv, int *d_info, int nb,
                    void *d_work, size_t work_bytes, gbla_stream_t stream);

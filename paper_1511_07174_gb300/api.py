@@ -75,7 +75,9 @@ def get_wait_timeout_ns():
 
 # ---------------------------------------------------------------------- LU FP64
 def lu_factor(A, nb=0):
-    """P A = L U (FP64, partial pivoting). Returns (LU, ipiv int32 1-based, info device int32[1])."""
+    """P A = L U (FP64, partial pivoting). Returns (LU, ipiv int32 1-based, info device int32[1]).
+    nb: block width, a multiple of 32 up to 256 (0: the library's choice); the trailing updates run
+    on the tensor cores for 128 and 256 only."""
     _require_cuda(A)
     L = _lib.load()
     n = A.shape[0]

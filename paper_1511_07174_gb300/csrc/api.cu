@@ -200,21 +200,6 @@ static void lookahead_release(const LookAhead& r) {
   g_la_pool.push_back(r);
 }
 
-// ----------------------------------------------------------------------------
-// Blocked right-looking LU over a generic storage type. Outer blocks of width
-// nb; inside each, inner panels of width kPanelWidth factored by the panel
-// kernel (which also applies the panel's row interchanges to the other
-// columns of the outer block), followed by the inner substitution and update
-// restricted to the outer block (one fused launch). After the outer block:
-// its interchanges on every other column (one launch), the U row block and
-// the trailing update.
-//
-// Look-ahead (when enabled): the trailing update is split into the next
-// outer block's columns and the rest. Once the first part is done, the next
-// block's panels are factored on a high-priority stream while the rest of the
-// update runs on the caller's stream on all SMs but 16 (the panel's cluster);
-// the caller's stream then waits for the panels. Every element receives the
-// same operations in the same order as without look-ahead.
 // Scratch of the FP64 trailing update on the tensor cores (both operands when
 // `cols`, else the rows of A only).
 static void digits_layout(Carver& c, int n, int nb, bool cols, F64Digits* d) {
@@ -230,7 +215,8 @@ static void digits_layout(Carver& c, int n, int nb, bool cols, F64Digits* d) {
 
 // The digits of L21 and U12 in 128 x 128 tiles: with nb a multiple of 128 the
 // look-ahead's split of an update falls on a tile boundary, so the same tiles
-// go to the FP64 pipe with and without it.
+// go to the FP64 pipe with and without it. With any other nb the whole update
+// stays on that pipe (n = 4000: nb = 96 52 ms, 128 19 ms).
 static bool lu_uses_digits(int nb) { return nb % 128 == 0; }
 
 static size_t lu_work_layout(Carver& c, int n, int nb, int prec, LuWork* w) {
@@ -262,6 +248,21 @@ static size_t lu_work_layout(Carver& c, int n, int nb, int prec, LuWork* w) {
   return c.off;
 }
 
+// ----------------------------------------------------------------------------
+// Blocked right-looking LU over a generic storage type. Outer blocks of width
+// nb; inside each, inner panels of width kPanelWidth factored by the panel
+// kernel (which also applies the panel's row interchanges to the other
+// columns of the outer block), followed by the inner substitution and update
+// restricted to the outer block (one fused launch). After the outer block:
+// its interchanges on every other column (one launch), the U row block and
+// the trailing update.
+//
+// Look-ahead (when enabled): the trailing update is split into the next
+// outer block's columns and the rest. Once the first part is done, the next
+// block's panels are factored on a high-priority stream while the rest of the
+// update runs on the caller's stream on all SMs but 16 (the panel's cluster);
+// the caller's stream then waits for the panels. Every element receives the
+// same operations in the same order as without look-ahead.
 template <typename Ts>
 cudaError_t blocked_lu(int n, Ts* A, int lda, int* ipiv, int* info, int nb, int prec,
                               const LuWork& w, cudaStream_t s) {

@@ -1,5 +1,5 @@
 // FP64 trailing update C -= A B (paper section 2: the rank-k "delayed update")
-// on the 5th-generation tensor cores, as exact products of 8-bit digits
+// on the 5th-generation tensor cores, as products of 8-bit digits
 // (the error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012, with
 // integer-aligned slices).
 //
@@ -11,12 +11,14 @@
 //     x = d_0 + d_1 2^-8 + ... + d_6 2^-48,   -128 <= d_t <= 128 integers,
 // each d_t 2^-8t a BF16 number. A digit product is at most 2^14 and the sum of
 // K <= 256 of them at most 2^22, so the FP32 accumulator of the tensor cores
-// holds the sum of up to four digit pairs exactly, and of the seven that the
-// lower groups have unless every digit is near 128 (where its rounding lies
-// below 2^-54 of the result). The pairs with s + t <= 7 (34 of 49) are
-// multiplied, those with the same s + t = g into one accumulator (6 and 7
-// share one); the epilogue adds the accumulators in 64-bit fixed point, rounds
-// once to FP64 and subtracts from C with one FP64 operation per element.
+// holds the sum of up to four digit pairs exactly, and of five or six unless every
+// digit is near 128. The pairs with s + t <= 7 (34 of 49) are multiplied, those with
+// the same s + t = g into one accumulator. 6 and 7 share one, whose sums (13 pairs in
+// units of 2^-56) need some 26 bits: it rounds, at 2^-55 for typical digits and at
+// 2^-48 with every digit near 128. The epilogue rounds the accumulators to 2^-40,
+// adds them in 64-bit fixed point, rounds once to FP64 and subtracts from C with one
+// FP64 operation per element; what the 15 pairs left out would add is below that
+// 2^-40 (typically 2^-46).
 //
 // Accuracy. With A_i, B_j scaled as above and P = sum_k |a_ik| |b_kj|, the
 // representation (2^-49 per element, zero for elements within a factor 4 of

@@ -33,9 +33,9 @@ static size_t trsv_flags_count(int n, int nrhs) {
   return (size_t)trsv_chains(nrhs) * (size_t)((n + kTsBS - 1) / kTsBS) + 1;
 }
 
-template <typename Ts, bool LOWER, bool TRANS, bool UNIT>
+template <bool LOWER, bool TRANS, bool UNIT>
 __global__ void __launch_bounds__(256)
-    trsv_chain_kernel(int n, int ncols, int G, int C, const Ts* __restrict__ T, int ldt,
+    trsv_chain_kernel(int n, int ncols, int G, int C, const double* __restrict__ T, int ldt,
                       const double* rhs, int ldr, double* X, int ldx, unsigned* flags,
                       const unsigned* gate, int* info, uint64_t wait_ns) {
   if (gate && *gate == 0u) return;  // the inverted diagonal blocks were good: nothing left to do
@@ -77,8 +77,7 @@ __global__ void __launch_bounds__(256)
       }
       double v = 0.0;
       if (rr < nr && jj < nc)
-        v = TRANS ? (double)T[(c0 + jj) + (size_t)(r0 + rr) * ldt]
-                  : (double)T[(r0 + rr) + (size_t)(c0 + jj) * ldt];
+        v = TRANS ? T[(c0 + jj) + (size_t)(r0 + rr) * ldt] : T[(r0 + rr) + (size_t)(c0 + jj) * ldt];
       tile[rr][jj] = v;
     }
   };
@@ -479,10 +478,13 @@ struct TcArgs {
 // latter, also held to 64 registers, is for the preconditioner of systems above 4096
 // rows: 288 threads leave an SM room for the 512 threads of 91 registers of such a
 // system's panel kernel, which needs 16 SMs of one GPC at the same time and would
-// otherwise wait for the whole substitution of another stream's system (three
-// systems of n = 16384 on three streams: 150 -> 141 ms; one alone 77.1 -> 78.7).
-// The panels of smaller systems fit beside the other variant, which is faster (n =
-// 2500, 4 right-hand sides: 22.5 -> 19.7 ms).
+// otherwise wait for the whole substitution of another stream's system, and for the
+// updates, of LU and Cholesky alike. Three systems of n = 16384 on three streams
+// (python bench.py): 185.0 -> 180.6 ms a step; three mixed Cholesky solves of n = 16384
+// 64.3 -> 58.2 ms, of 8192 17.6 -> 16.1. One alone pays: mixed LU of n = 8192 23.0 ->
+// 23.4 ms, mixed Cholesky 10.6 -> 11.0, of n = 16384 30.4 -> 31.7. The panels of
+// smaller systems fit beside the other variant, which is faster (n = 2500, 4
+// right-hand sides: 22.5 -> 19.7 ms).
 template <int NR, int H>
 constexpr int tc_threads() {
   return H + 32 * kTcWarps * NR + 32;
@@ -1042,8 +1044,7 @@ static cudaError_t tc_launch_diag_inv(bool fwd, bool unit, int n, const Ts* T, i
   return cudaGetLastError();
 }
 
-// One group of at most kTcMaxC * kTcMaxG right-hand sides. keep_bad: the word
-// that says whether the inverses are safe is left as it is.
+// One group of at most kTcMaxC * kTcMaxG right-hand sides.
 template <typename Ts, bool TRANS>
 static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, const Ts* T, int ldt, const double* D, const double* rhs,
                             int ldr, double* X, int ldx, char* scratch, size_t ctrl_words, bool gated, int* info,
@@ -1082,6 +1083,7 @@ static cudaError_t tc_apply(bool fwd, bool unit, int n, int ncols, TcShape sh, c
   return cudaErrorInvalidValue;  // the preconditioner takes at most kTcMaxC columns
 }
 
+// keep_bad: what the set-up found about the inverses is left as it is.
 static cudaError_t tc_fill(int n, int ncols, TcShape sh, double* X, int ldx, char* scratch, size_t ctrl_words,
                            bool keep_bad, cudaStream_t s) {
   const size_t np = (size_t)tc_first((n + kTsBS - 1) / kTsBS) * sh.C * sh.G * 32;
@@ -1102,6 +1104,7 @@ cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, cons
                         const double* rhs, int ldr, double* X, int ldx, double* D, void* scratch, int* info,
                         cudaStream_t s) {
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
+  if (!lower && unit) return cudaErrorInvalidValue;  // no factorisation leaves one
   const int nblk = (n + kTsBS - 1) / kTsBS;
   const uint64_t wait_ns = wait_timeout_ns();
   const bool fwd = lower != trans;
@@ -1139,15 +1142,13 @@ cudaError_t launch_trsv(bool lower, bool trans, bool unit, int n, int nrhs, cons
     const int grid = Cl * nblk;
     const unsigned* gate = blocks ? ctrl + kTcMaxC : nullptr;
 #define GBLA_TRSV(LW, TR, UN)                                                                         \
-  trsv_chain_kernel<double, LW, TR, UN><<<grid, 256, 0, s>>>(n, ncols, G, Cl, T, ldt, R, ldr, Xc, ldx, \
-                                                             flags, gate, info, wait_ns)
+  trsv_chain_kernel<LW, TR, UN><<<grid, 256, 0, s>>>(n, ncols, G, Cl, T, ldt, R, ldr, Xc, ldx, flags, \
+                                                     gate, info, wait_ns)
     if (lower && !trans && unit) GBLA_TRSV(true, false, true);
     else if (lower && !trans && !unit) GBLA_TRSV(true, false, false);
     else if (lower && trans && unit) GBLA_TRSV(true, true, true);
     else if (lower && trans && !unit) GBLA_TRSV(true, true, false);
-    else if (!lower && !trans && unit) GBLA_TRSV(false, false, true);
-    else if (!lower && !trans && !unit) GBLA_TRSV(false, false, false);
-    else if (!lower && trans && unit) GBLA_TRSV(false, true, true);
+    else if (!trans) GBLA_TRSV(false, false, false);
     else GBLA_TRSV(false, true, false);
 #undef GBLA_TRSV
     count_launch();
