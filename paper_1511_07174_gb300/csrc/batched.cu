@@ -492,8 +492,10 @@ __device__ int bt_chol_panel(T* __restrict__ A, int lda, int m, int w, T* __rest
           if (lane == 0) sh.rdiag[j] = rl;
 #pragma unroll
           for (int k = j + 1; k < kBtW; ++k) {
-            const T lk = __shfl_sync(0xffffffffu, x[0][j], k);
-            if (lane >= k && lane < w && k < w) x[0][k] = fma(-x[0][j], lk, x[0][k]);
+            if (k < w) {
+              const T z = fma(-x[0][j], __shfl_sync(0xffffffffu, x[0][j], k), x[0][k]);
+              if (lane >= k && lane < w) x[0][k] = z;
+            }
           }
         }
       }
