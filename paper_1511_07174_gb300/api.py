@@ -116,6 +116,9 @@ def chol_factor(A, nb=0):
     n = A.shape[0]
     F = colmajor(A, torch.float64, copy=True)
     info = torch.zeros(1, dtype=torch.int32, device=A.device)
+    if n <= 64:  # one diagonal block: no update, no scratch
+        _check("gbla_chol_factor", L.gbla_chol_factor(n, _p(F), _ld(F), _p(info), int(nb), _stream()))
+        return F, info
     ws = _ws(L.gbla_chol_factor_workspace(n, int(nb)), A.device)
     _check("gbla_chol_factor_ws", L.gbla_chol_factor_ws(n, _p(F), _ld(F), _p(info), int(nb), _p(ws), ws.numel(),
                                                         _stream()))
